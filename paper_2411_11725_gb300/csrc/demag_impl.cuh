@@ -158,6 +158,7 @@ template <typename T, bool CELL_IN, int LG>
 __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
     k_x_fwd(Geom g, DemagBufs<T> b, const T *__restrict__ in, int lpb)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     constexpr int Q = 1 << LG, H = Q / 2, LSZ = f3::padded(Q);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -215,6 +216,7 @@ __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
 template <typename T, bool CELL_IN>
 __global__ void k_x_fwd1(Geom g, DemagBufs<T> b, const T *__restrict__ in)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     const int nlines = 3 * g.N2 * g.N3;
     const int L = blockIdx.x * blockDim.x + threadIdx.x;
@@ -232,6 +234,7 @@ template <typename T, bool CELL_OUT, int LG>
 __global__ void __launch_bounds__(kXiThreads<T>, sizeof(T) == 4 ? 16 : 4)
     k_x_inv(Geom g, DemagBufs<T> b, T *__restrict__ out, int lpb)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     constexpr int Q = 1 << LG, H = Q / 2, LSZ = f3::padded(Q);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -302,6 +305,7 @@ __global__ void __launch_bounds__(kXiThreads<T>, sizeof(T) == 4 ? 16 : 4)
 template <typename T, bool CELL_OUT>
 __global__ void k_x_inv1(Geom g, DemagBufs<T> b, T *__restrict__ out)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     const int nlines = 3 * g.N2 * g.N3;
     const int L = blockIdx.x * blockDim.x + threadIdx.x;
@@ -408,6 +412,7 @@ template <typename T, int LG>
 __global__ void __launch_bounds__(kMaxThreads<T, LG>, kMinBlocks<T, LG>)
     k_y_fwd(Geom g, DemagBufs<T> b, const __grid_constant__ CUtensorMap tm)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     constexpr int P2 = 1 << LG, G = YTile<T, LG>::G, LFP = YTile<T, LG>::LFP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -446,6 +451,7 @@ template <typename T, int LG>
 __global__ void __launch_bounds__(kMaxThreads<T, LG>, kMinBlocks<T, LG>)
     k_y_inv(Geom g, DemagBufs<T> b, const __grid_constant__ CUtensorMap tm)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     constexpr int G = YTile<T, LG>::G, LFP = YTile<T, LG>::LFP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -557,6 +563,7 @@ __device__ __forceinline__ void z_tile_load(const Geom &g, const DemagBufs<T> &b
 template <typename T, int LG>
 __global__ void __launch_bounds__(kMaxThreads<T>, kMinBlocks<T>) k_z_conv(Geom g, DemagBufs<T> b)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     using Z = ZTile<T, LG>;
     constexpr int P3 = 1 << LG, H3 = P3 / 2 + 1, G = Z::G, KY = Z::KY;
@@ -638,6 +645,7 @@ template <int LG>
 __global__ void __launch_bounds__(ZRTile<LG, kZRSplit<LG>>::THREADS, kZRSplit<LG> == 4 ? 3 : (LG >= 6 ? 4 : 2))
     k_z_conv_r(Geom g, DemagBufs<float> b)
 {
+    pdl_enter();
     using T = float;
     constexpr int S = kZRSplit<LG>;
     using Z = ZRTile<LG, S>;
@@ -806,6 +814,7 @@ __global__ void __launch_bounds__(ZRTile<LG, kZRSplit<LG>>::THREADS, kZRSplit<LG
 template <typename T, int LG>
 __global__ void __launch_bounds__(kMaxThreadsYC<T>, 1) k_y_conv(Geom g, DemagBufs<T> b, int G)
 {
+    pdl_enter();
     if (b.ctl && b.ctl->done) return;
     constexpr int P2 = 1 << LG;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1052,11 +1061,11 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
     if (g.N3 > 1 && g.P2 > 1 && !b.ymap) return;
     const int nlines = 3 * g.N2 * g.N3;
     if (g.P1 == 1) {
-        k_x_fwd1<T, CELL><<<div_up(nlines, 256), 256, 0, st>>>(g, b, in);
+        launch_pdl(k_x_fwd1<T, CELL>, div_up(nlines, 256), 256, 0, st, g, b, in);
     } else {
         f3::lg_dispatch<1, 10>(g.lgQ, [&](auto c) {
             constexpr int LG = decltype(c)::value;
-            k_x_fwd<T, CELL, LG><<<div_up(nlines, p.x_lpb), p.x_threads, p.x_smem, st>>>(g, b, in, p.x_lpb);
+            launch_pdl(k_x_fwd<T, CELL, LG>, div_up(nlines, p.x_lpb), p.x_threads, p.x_smem, st, g, b, in, p.x_lpb);
         });
     }
     b.mark("demag_x_fwd");
@@ -1064,7 +1073,7 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
         if (g.P2 > 1) {
             f3::lg_dispatch<1, 11>(g.lgP2, [&](auto c) {
                 constexpr int LG = decltype(c)::value;
-                k_y_fwd<T, LG><<<dim3(g.Xp / p.y_G, 3 * g.N3), p.y_threads, p.yi_smem, st>>>(g, b, *b.ymap);
+                launch_pdl(k_y_fwd<T, LG>, dim3(g.Xp / p.y_G, 3 * g.N3), p.y_threads, p.yi_smem, st, g, b, *b.ymap);
             });
             b.mark("demag_y_fwd");
         }
@@ -1072,37 +1081,37 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
             if (p.z_reg) {
                 f3::lg_dispatch<2, 6>(g.lgP3, [&](auto c) {
                     constexpr int LG = decltype(c)::value;
-                    k_z_conv_r<LG><<<dim3(g.Xp / p.z_G, div_up(g.H2, p.z_KY)), p.z_threads, p.z_smem, st>>>(g, b);
+                    launch_pdl(k_z_conv_r<LG>, dim3(g.Xp / p.z_G, div_up(g.H2, p.z_KY)), p.z_threads, p.z_smem, st, g, b);
                 });
             }
         }
         if (!p.z_reg) {
             f3::lg_dispatch<1, 7>(g.lgP3, [&](auto c) {
                 constexpr int LG = decltype(c)::value;
-                k_z_conv<T, LG><<<dim3(g.Xp / p.z_G, div_up(g.H2, p.z_KY)), p.z_threads, p.z_smem, st>>>(g, b);
+                launch_pdl(k_z_conv<T, LG>, dim3(g.Xp / p.z_G, div_up(g.H2, p.z_KY)), p.z_threads, p.z_smem, st, g, b);
             });
         }
         b.mark("demag_z_conv");
         if (g.P2 > 1) {
             f3::lg_dispatch<1, 11>(g.lgP2, [&](auto c) {
                 constexpr int LG = decltype(c)::value;
-                k_y_inv<T, LG><<<dim3(g.Xp / p.y_G, 3 * g.N3), p.y_threads, p.yi_smem, st>>>(g, b, *b.ymap);
+                launch_pdl(k_y_inv<T, LG>, dim3(g.Xp / p.y_G, 3 * g.N3), p.y_threads, p.yi_smem, st, g, b, *b.ymap);
             });
             b.mark("demag_y_inv");
         }
     } else {
         f3::lg_dispatch<0, 11>(g.lgP2, [&](auto c) {
             constexpr int LG = decltype(c)::value;
-            k_y_conv<T, LG><<<g.Xp / p.yc_G, p.yc_threads, p.yc_smem, st>>>(g, b, p.yc_G);
+            launch_pdl(k_y_conv<T, LG>, g.Xp / p.yc_G, p.yc_threads, p.yc_smem, st, g, b, p.yc_G);
         });
         b.mark("demag_y_conv");
     }
     if (g.P1 == 1) {
-        k_x_inv1<T, CELL><<<div_up(nlines, 256), 256, 0, st>>>(g, b, out);
+        launch_pdl(k_x_inv1<T, CELL>, div_up(nlines, 256), 256, 0, st, g, b, out);
     } else {
         f3::lg_dispatch<1, 10>(g.lgQ, [&](auto c) {
             constexpr int LG = decltype(c)::value;
-            k_x_inv<T, CELL, LG><<<div_up(nlines, p.xi_lpb), p.xi_threads, p.xi_smem, st>>>(g, b, out, p.xi_lpb);
+            launch_pdl(k_x_inv<T, CELL, LG>, div_up(nlines, p.xi_lpb), p.xi_threads, p.xi_smem, st, g, b, out, p.xi_lpb);
         });
     }
     b.mark("demag_x_inv");

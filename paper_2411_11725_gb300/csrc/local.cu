@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(kTX *kTY<T>, sizeof(T) == 4 ? 6 : 3) k_node(Lo
                                                         T *__restrict__ out, T *__restrict__ y_next, StageArgs sa,
                                                         double t_heff, NodeGrid ng)
 {
+    pdl_enter();
     static_assert(!OWN || (sizeof(T) == 4 && STAGE && !DMI), "own-value staging is for FP32 stage kernels");
     if (STAGE && sa.ctl && sa.ctl->done) return;
     constexpr int TY = kTY<T>;
@@ -557,6 +558,7 @@ template <typename T, bool STAGE>
 __global__ void __launch_bounds__(256) k_node2d(LocalParams<T> p, const T *__restrict__ y, T *__restrict__ out,
                                                 T *__restrict__ y_next, StageArgs sa, double t_heff)
 {
+    pdl_enter();
     if (STAGE && sa.ctl && sa.ctl->done) return;
     const Geom &g = p.g;
     const int n1 = blockIdx.x * 32 + (threadIdx.x & 31), n2 = blockIdx.y * 8 + (threadIdx.x >> 5);
@@ -706,6 +708,7 @@ __global__ void __launch_bounds__(kNode1dThreads) k_node1d(LocalParams<T> p, con
                                                            T *__restrict__ out, T *__restrict__ y_next, StageArgs sa,
                                                            double t_heff)
 {
+    pdl_enter();
     if (STAGE && sa.ctl && sa.ctl->done) return;
     const Geom &g = p.g;
     const int n1 = blockIdx.x;
@@ -852,6 +855,7 @@ __global__ void __launch_bounds__(kNode1dThreads) k_node1d(LocalParams<T> p, con
 template <typename T>
 __global__ void __launch_bounds__(256) k_dmi(LocalParams<T> p, const T *__restrict__ y, T *__restrict__ out)
 {
+    pdl_enter();
     const Geom &g = p.g;
     const long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= g.n_nodes) return;
@@ -933,42 +937,42 @@ template <typename T>
 void launch_heff(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaStream_t st)
 {
     if (p.g.basis == 2) {
-        k_node2d<T, false><<<dim3(div_up(p.g.nn1, 32), div_up(p.g.nn2, 8)), 256, 0, st>>>(p, y, h_out, nullptr,
+        launch_pdl(k_node2d<T, false>, dim3(div_up(p.g.nn1, 32), div_up(p.g.nn2, 8)), 256, 0, st, p, y, h_out, nullptr,
                                                                                           StageArgs{}, t);
         return;
     }
     if (p.g.basis == 1) {
-        k_node1d<T, false><<<p.g.nn1, kNode1dThreads, 0, st>>>(p, y, h_out, nullptr, StageArgs{}, t);
+        launch_pdl(k_node1d<T, false>, p.g.nn1, kNode1dThreads, 0, st, p, y, h_out, nullptr, StageArgs{}, t);
         return;
     }
     int nb;
     if (p.hdmi) {
         const NodeGrid ng = node_grid<T, false, true>(p.g, &nb);
-        k_dmi<T><<<div_up(p.g.n_nodes, 256), 256, 0, st>>>(p, y, p.hdmi);
-        k_node<T, false, true><<<nb, kTX * kTY<T>, 0, st>>>(p, y, h_out, nullptr, StageArgs{}, t, ng);
+        launch_pdl(k_dmi<T>, div_up(p.g.n_nodes, 256), 256, 0, st, p, y, p.hdmi);
+        launch_pdl(k_node<T, false, true>, nb, kTX * kTY<T>, 0, st, p, y, h_out, nullptr, StageArgs{}, t, ng);
         return;
     }
     const NodeGrid ng = node_grid<T, false, false>(p.g, &nb);
-    k_node<T, false><<<nb, kTX * kTY<T>, 0, st>>>(p, y, h_out, nullptr, StageArgs{}, t, ng);
+    launch_pdl(k_node<T, false>, nb, kTX * kTY<T>, 0, st, p, y, h_out, nullptr, StageArgs{}, t, ng);
 }
 
 template <typename T>
 void launch_llg_stage(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa, cudaStream_t st)
 {
     if (p.g.basis == 2) {
-        k_node2d<T, true><<<dim3(div_up(p.g.nn1, 32), div_up(p.g.nn2, 8)), 256, 0, st>>>(p, y, k_out, y_next, sa,
+        launch_pdl(k_node2d<T, true>, dim3(div_up(p.g.nn1, 32), div_up(p.g.nn2, 8)), 256, 0, st, p, y, k_out, y_next, sa,
                                                                                          0.0);
         return;
     }
     if (p.g.basis == 1) {
-        k_node1d<T, true><<<p.g.nn1, kNode1dThreads, 0, st>>>(p, y, k_out, y_next, sa, 0.0);
+        launch_pdl(k_node1d<T, true>, p.g.nn1, kNode1dThreads, 0, st, p, y, k_out, y_next, sa, 0.0);
         return;
     }
     int nb;
     if (p.hdmi) {
         const NodeGrid ng = node_grid<T, true, true>(p.g, &nb);
-        k_dmi<T><<<div_up(p.g.n_nodes, 256), 256, 0, st>>>(p, y, p.hdmi);
-        k_node<T, true, true><<<nb, kTX * kTY<T>, 0, st>>>(p, y, k_out, y_next, sa, 0.0, ng);
+        launch_pdl(k_dmi<T>, div_up(p.g.n_nodes, 256), 256, 0, st, p, y, p.hdmi);
+        launch_pdl(k_node<T, true, true>, nb, kTX * kTY<T>, 0, st, p, y, k_out, y_next, sa, 0.0, ng);
         return;
     }
     if constexpr (sizeof(T) == 4) {
@@ -982,12 +986,12 @@ void launch_llg_stage(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, 
                 carveout = true;
             }
             const NodeGrid ng = node_grid<T, true, false, true>(p.g, &nb);
-            k_node<T, true, false, true><<<nb, kTX * kTY<T>, 0, st>>>(p, y, k_out, y_next, sa, 0.0, ng);
+            launch_pdl(k_node<T, true, false, true>, nb, kTX * kTY<T>, 0, st, p, y, k_out, y_next, sa, 0.0, ng);
             return;
         }
     }
     const NodeGrid ng = node_grid<T, true, false>(p.g, &nb);
-    k_node<T, true><<<nb, kTX * kTY<T>, 0, st>>>(p, y, k_out, y_next, sa, 0.0, ng);
+    launch_pdl(k_node<T, true>, nb, kTX * kTY<T>, 0, st, p, y, k_out, y_next, sa, 0.0, ng);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -995,6 +999,7 @@ template <typename T>
 __global__ void k_mass(Geom g, const double *__restrict__ Ms, double Ms0, double mu0V8, T *inv_mass,
                        unsigned long long *n_active)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= g.n_nodes) return;
     const int n1 = (int)(n % g.nn1);
@@ -1033,7 +1038,7 @@ template <typename T>
 void launch_mass(const Geom &g, const double *Ms_d, double Ms0, double V, T *inv_mass, unsigned long long *n_active,
                  cudaStream_t st)
 {
-    k_mass<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g, Ms_d, Ms0, kMu0 * V / 8.0, inv_mass, n_active);
+    launch_pdl(k_mass<T>, div_up(g.n_nodes, 256), 256, 0, st, g, Ms_d, Ms0, kMu0 * V / 8.0, inv_mass, n_active);
 }
 
 template void launch_heff<float>(const LocalParams<float> &, const float *, float *, double, cudaStream_t);

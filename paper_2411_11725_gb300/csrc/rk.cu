@@ -13,6 +13,7 @@ template <typename T>
 __global__ void k_stage_input(long n_nodes, long ns, const double *__restrict__ m, KList k, const StepCtl *ctl,
                               T *__restrict__ y, const float *__restrict__ mf)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     if (ctl->done) return;
@@ -35,6 +36,7 @@ __global__ void k_stage_input(long n_nodes, long ns, const double *__restrict__ 
 __global__ void k_stage_input_f4(long n_nodes, long ns, KList k, const StepCtl *ctl, float *__restrict__ y,
                                  const float *__restrict__ mf)
 {
+    pdl_enter();
     const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (ctl->done) return;
     const float dtf = (float)ctl->dt;
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dp5_err(long n_nodes, long ns, 
                                                           const StepCtl *ctl, double *partials,
                                                           const float *__restrict__ mf)
 {
+    pdl_enter();
     __shared__ double sh[kRedThreads];
     if (ctl->done) return;
     const double dt = ctl->dt, rtol = ctl->rtol, atol = ctl->atol;
@@ -183,6 +186,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dp5_err_f4(long n_nodes, long n
                                                              const float *__restrict__ inv_mass, const StepCtl *ctl,
                                                              double *partials, const float *__restrict__ mf)
 {
+    pdl_enter();
     __shared__ double sh[kRedThreads];
     if (ctl->done) return;
     const float dtf = (float)ctl->dt, rtol = (float)ctl->rtol, atol = (float)ctl->atol;
@@ -243,6 +247,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dp5_err_f4(long n_nodes, long n
 __global__ void __launch_bounds__(1024) k_dp5_ctl(const double *partials, int nparts, double n_active, StepCtl *ctl,
                                                   int max_rej)
 {
+    pdl_enter();
     __shared__ double sh[1024];
     if (ctl->done) {
         if (threadIdx.x == 0) ctl->accepted = 0;
@@ -367,6 +372,7 @@ __device__ __forceinline__ void advance_f32(double v[3], const float d[3], int r
 __global__ void k_dp5_update_f4(long n_nodes, long ns, double *__restrict__ m, KList kb, const float *__restrict__ k7,
                                 float *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf)
 {
+    pdl_enter();
     const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (!ctl->accepted) return;
     const float dtf = (float)ctl->dt_used;
@@ -442,6 +448,7 @@ template <typename T>
 __global__ void k_dp5_update(long n_nodes, long ns, double *__restrict__ m, KList kb, const T *__restrict__ k7,
                              T *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     if (!ctl->accepted) return;
@@ -460,6 +467,7 @@ template <typename T>
 __global__ void k_rk4_update(long n_nodes, long ns, double *__restrict__ m, KList kb, const StepCtl *ctl, int renorm,
                              float *__restrict__ mf)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     if (ctl->done) return;
@@ -473,6 +481,7 @@ __global__ void k_rk4_update(long n_nodes, long ns, double *__restrict__ m, KLis
 
 __global__ void k_rk4_advance(StepCtl *ctl)
 {
+    pdl_enter();
     if (ctl->done) return;
     ctl->t += ctl->dt;
     ctl->n_acc += 1;
@@ -490,6 +499,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_mean_partials(long n_nodes, long ns, const double *__restrict__ m,
                                                                 const T *__restrict__ vol, double *partials)
 {
+    pdl_enter();
     __shared__ double sh[kRedThreads];
     double a[4] = {0, 0, 0, 0};
     for (long n = blockIdx.x * (long)blockDim.x + threadIdx.x; n < n_nodes; n += (long)gridDim.x * blockDim.x) {
@@ -507,6 +517,7 @@ __global__ void __launch_bounds__(kRedThreads) k_mean_partials(long n_nodes, lon
 
 __global__ void __launch_bounds__(1024) k_mean_final(const double *partials, int nparts, double *out)
 {
+    pdl_enter();
     __shared__ double sh[1024];
     for (int c = 0; c < 4; ++c) {
         double v = 0.0;
@@ -531,6 +542,7 @@ template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(256) k_aos_to_soa(Geom g, const Tin *__restrict__ a, Tout *__restrict__ s,
                                                     unsigned long long *__restrict__ nonfinite)
 {
+    pdl_enter();
     __shared__ Tout tile[3][kTT][kTT + 1];
     const int n2 = blockIdx.z;
     const int n3_0 = blockIdx.x * kTT, n1_0 = blockIdx.y * kTT;
@@ -561,6 +573,7 @@ __global__ void __launch_bounds__(256) k_aos_to_soa(Geom g, const Tin *__restric
 template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(256) k_soa_to_aos(Geom g, const Tin *__restrict__ s, Tout *__restrict__ a)
 {
+    pdl_enter();
     __shared__ Tout tile[3][kTT][kTT + 1];
     const int n2 = blockIdx.z;
     const int n3_0 = blockIdx.x * kTT, n1_0 = blockIdx.y * kTT;
@@ -591,6 +604,7 @@ template <typename Tout>
 __global__ void k_cells_to_internal(Geom g, const double *__restrict__ a, int ncomp, double scale_by_Ms0,
                                     const double *__restrict__ Ms, Tout *__restrict__ s)
 {
+    pdl_enter();
     long c = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (c >= g.n_cells) return;
     const int c1 = (int)(c % g.N1);
@@ -605,6 +619,7 @@ __global__ void k_cells_to_internal(Geom g, const double *__restrict__ a, int nc
 template <typename Tin, typename Tout>
 __global__ void k_convert(long n, const Tin *__restrict__ a, Tout *__restrict__ b)
 {
+    pdl_enter();
     long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i < n) b[i] = (Tout)a[i];
 }
@@ -614,6 +629,7 @@ __global__ void k_convert(long n, const Tin *__restrict__ a, Tout *__restrict__ 
 template <typename T>
 __global__ void k_node_volume(Geom g, const double *__restrict__ Ms, double Ms0, double V8, T *vol)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= g.n_nodes) return;
     const int n1 = (int)(n % g.nn1);
@@ -662,11 +678,11 @@ void launch_stage_input(const Geom &g, const double *m, const KList &k, const St
     if constexpr (sizeof(T) == 4) {
         if (mf) {
             const long n4 = g.n_nodes >> 2;
-            k_stage_input_f4<<<div_up(n4 > 4 ? n4 : 4, 256), 256, 0, st>>>(g.n_nodes, g.ns, fk(k), ctl, (float *)y, mf);
+            launch_pdl(k_stage_input_f4, div_up(n4 > 4 ? n4 : 4, 256), 256, 0, st, g.n_nodes, g.ns, fk(k), ctl, (float *)y, mf);
             return;
         }
     }
-    k_stage_input<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, m, fk(k), ctl, y, mf);
+    launch_pdl(k_stage_input<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(k), ctl, y, mf);
 }
 
 int reduction_blocks(long n_nodes)
@@ -685,20 +701,20 @@ void launch_dp5_control(const Geom &g, const double *m, const KList &kb, const K
     const int nb = (int)(nbl > 4096 ? 4096 : (nbl < 1 ? 1 : nbl));
     if constexpr (sizeof(T) == 4) {
         if (f64_terms) {
-            k_dp5_err<T, true><<<nb, kRedThreads, 0, st>>>(g.n_nodes, g.ns, m, fk(kb), fk(ke), inv_mass, ctl,
+            launch_pdl(k_dp5_err<T, true>, nb, kRedThreads, 0, st, g.n_nodes, g.ns, m, fk(kb), fk(ke), inv_mass, ctl,
                                                            partials, nullptr);
-            k_dp5_ctl<<<1, 1024, 0, st>>>(partials, nb, n_active, ctl, max_rej);
+            launch_pdl(k_dp5_ctl, 1, 1024, 0, st, partials, nb, n_active, ctl, max_rej);
             return;
         }
         if (mf) {
-            k_dp5_err_f4<<<nb, kRedThreads, 0, st>>>(g.n_nodes, g.ns, fk(kb), fk(ke), (const float *)inv_mass, ctl,
+            launch_pdl(k_dp5_err_f4, nb, kRedThreads, 0, st, g.n_nodes, g.ns, fk(kb), fk(ke), (const float *)inv_mass, ctl,
                                                      partials, mf);
-            k_dp5_ctl<<<1, 1024, 0, st>>>(partials, nb, n_active, ctl, max_rej);
+            launch_pdl(k_dp5_ctl, 1, 1024, 0, st, partials, nb, n_active, ctl, max_rej);
             return;
         }
     }
-    k_dp5_err<T><<<nb, kRedThreads, 0, st>>>(g.n_nodes, g.ns, m, fk(kb), fk(ke), inv_mass, ctl, partials, mf);
-    k_dp5_ctl<<<1, 1024, 0, st>>>(partials, nb, n_active, ctl, max_rej);
+    launch_pdl(k_dp5_err<T>, nb, kRedThreads, 0, st, g.n_nodes, g.ns, m, fk(kb), fk(ke), inv_mass, ctl, partials, mf);
+    launch_pdl(k_dp5_ctl, 1, 1024, 0, st, partials, nb, n_active, ctl, max_rej);
 }
 
 template <typename T>
@@ -708,61 +724,61 @@ void launch_dp5_update(const Geom &g, double *m, const KList &kb, const T *k7, T
     if constexpr (sizeof(T) == 4) {
         if (mf) {
             const long n4 = g.n_nodes >> 2;
-            k_dp5_update_f4<<<div_up(n4 > 4 ? n4 : 4, 256), 256, 0, st>>>(g.n_nodes, g.ns, m, fk(kb), (const float *)k7,
+            launch_pdl(k_dp5_update_f4, div_up(n4 > 4 ? n4 : 4, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), (const float *)k7,
                                                                            (float *)k1, ctl, renorm, mf);
             return;
         }
     }
-    k_dp5_update<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, m, fk(kb), k7, k1, ctl, renorm, mf);
+    launch_pdl(k_dp5_update<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1, ctl, renorm, mf);
 }
 
 template <typename T>
 void launch_rk4_update(const Geom &g, double *m, const KList &kb, StepCtl *ctl, int renorm, cudaStream_t st,
                        float *mf)
 {
-    k_rk4_update<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, m, fk(kb), ctl, renorm, mf);
-    k_rk4_advance<<<1, 1, 0, st>>>(ctl);
+    launch_pdl(k_rk4_update<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), ctl, renorm, mf);
+    launch_pdl(k_rk4_advance, 1, 1, 0, st, ctl);
 }
 
 template <typename T>
 void launch_mean(const Geom &g, const double *m, const T *vol, double *partials, double *out, cudaStream_t st)
 {
     int nb = reduction_blocks(g.n_nodes);
-    k_mean_partials<T><<<nb, kRedThreads, 0, st>>>(g.n_nodes, g.ns, m, vol, partials);
-    k_mean_final<<<1, 1024, 0, st>>>(partials, nb, out);
+    launch_pdl(k_mean_partials<T>, nb, kRedThreads, 0, st, g.n_nodes, g.ns, m, vol, partials);
+    launch_pdl(k_mean_final, 1, 1024, 0, st, partials, nb, out);
 }
 
 template <typename Tin, typename Tout>
 void launch_aos_to_soa(const Geom &g, const Tin *a, Tout *s, cudaStream_t st, unsigned long long *nonfinite)
 {
     const dim3 grid(div_up(g.nn3, kTT), div_up(g.nn1, kTT), g.nn2);
-    k_aos_to_soa<Tin, Tout><<<grid, dim3(kTT, 8), 0, st>>>(g, a, s, nonfinite);
+    launch_pdl(k_aos_to_soa<Tin, Tout>, grid, dim3(kTT, 8), 0, st, g, a, s, nonfinite);
 }
 
 template <typename Tin, typename Tout>
 void launch_soa_to_aos(const Geom &g, const Tin *s, Tout *a, cudaStream_t st)
 {
     const dim3 grid(div_up(g.nn3, kTT), div_up(g.nn1, kTT), g.nn2);
-    k_soa_to_aos<Tin, Tout><<<grid, dim3(kTT, 8), 0, st>>>(g, s, a);
+    launch_pdl(k_soa_to_aos<Tin, Tout>, grid, dim3(kTT, 8), 0, st, g, s, a);
 }
 
 template <typename Tout>
 void launch_cells_to_internal(const Geom &g, const double *a, int ncomp, double scale_by_Ms0, const double *Ms,
                               Tout *s, cudaStream_t st)
 {
-    k_cells_to_internal<Tout><<<div_up(g.n_cells, 256), 256, 0, st>>>(g, a, ncomp, scale_by_Ms0, Ms, s);
+    launch_pdl(k_cells_to_internal<Tout>, div_up(g.n_cells, 256), 256, 0, st, g, a, ncomp, scale_by_Ms0, Ms, s);
 }
 
 template <typename Tin, typename Tout>
 void launch_convert(long n, const Tin *a, Tout *b, cudaStream_t st)
 {
-    k_convert<Tin, Tout><<<div_up(n, 256), 256, 0, st>>>(n, a, b);
+    launch_pdl(k_convert<Tin, Tout>, div_up(n, 256), 256, 0, st, n, a, b);
 }
 
 template <typename T>
 void launch_node_volume(const Geom &g, const double *Ms, double Ms0, double V, T *vol, cudaStream_t st)
 {
-    k_node_volume<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g, Ms, Ms0, V / 8.0, vol);
+    launch_pdl(k_node_volume<T>, div_up(g.n_nodes, 256), 256, 0, st, g, Ms, Ms0, V / 8.0, vol);
 }
 
 #define NM_INST(T)                                                                                             \

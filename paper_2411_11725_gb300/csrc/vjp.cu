@@ -8,6 +8,7 @@ template <typename T>
 __global__ void k_scale_inv_mass(long n_nodes, long ns, const T *__restrict__ v, const T *__restrict__ im,
                                  T *__restrict__ w)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     const T s = im[n];
@@ -18,6 +19,7 @@ template <typename T>
 __global__ void k_cell_moment(Geom g, const T *__restrict__ y, const T *__restrict__ Ms, T Ms0, T scale,
                               T *__restrict__ out)
 {
+    pdl_enter();
     long c = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (c >= g.n_cells) return;
     const int c1 = (int)(c % g.N1);
@@ -39,6 +41,7 @@ __global__ void k_cell_moment(Geom g, const T *__restrict__ y, const T *__restri
 template <typename T>
 __global__ void k_grad_Ms(Geom g, GradMsArgs a, const T *__restrict__ im, double *__restrict__ gMs)
 {
+    pdl_enter();
     long c = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (c >= g.n_cells) return;
     const int c1 = (int)(c % g.N1);
@@ -79,6 +82,7 @@ __global__ void k_llg_vjp_local(long n_nodes, long ns, const T *__restrict__ y, 
                                 const T *__restrict__ u, const T *__restrict__ im, T gam, T alpha,
                                 T *__restrict__ ybar, T *__restrict__ q)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     T yv[3], Hv[3], uv[3];
@@ -116,6 +120,7 @@ template <typename T>
 __global__ void k_axpby(long n_nodes, long ns, T a, const T *__restrict__ x, T b, const T *__restrict__ y,
                         T *__restrict__ out)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     for (int k = 0; k < 3; ++k) out[k * ns + n] = a * x[k * ns + n] + b * y[k * ns + n];
@@ -125,33 +130,33 @@ __global__ void k_axpby(long n_nodes, long ns, T a, const T *__restrict__ x, T b
 template <typename T>
 void launch_scale_inv_mass(const Geom &g, const T *v, const T *inv_mass, T *w, cudaStream_t st)
 {
-    k_scale_inv_mass<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, v, inv_mass, w);
+    launch_pdl(k_scale_inv_mass<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, v, inv_mass, w);
 }
 
 template <typename T>
 void launch_cell_moment(const Geom &g, const T *y, const T *Ms, T Ms0, T scale, T *out, cudaStream_t st)
 {
-    k_cell_moment<T><<<div_up(g.n_cells, 256), 256, 0, st>>>(g, y, Ms, Ms0, scale, out);
+    launch_pdl(k_cell_moment<T>, div_up(g.n_cells, 256), 256, 0, st, g, y, Ms, Ms0, scale, out);
 }
 
 template <typename T>
 void launch_grad_Ms(const Geom &g, const GradMsArgs &a, const T *inv_mass, double *gMs, cudaStream_t st)
 {
-    k_grad_Ms<T><<<div_up(g.n_cells, 256), 256, 0, st>>>(g, a, inv_mass, gMs);
+    launch_pdl(k_grad_Ms<T>, div_up(g.n_cells, 256), 256, 0, st, g, a, inv_mass, gMs);
 }
 
 template <typename T>
 void launch_llg_vjp_local(const Geom &g, const T *y, const T *H, const T *u, const T *inv_mass, double gam,
                           double alpha, T *ybar, T *q, cudaStream_t st)
 {
-    k_llg_vjp_local<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, y, H, u, inv_mass, (T)gam, (T)alpha,
+    launch_pdl(k_llg_vjp_local<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, y, H, u, inv_mass, (T)gam, (T)alpha,
                                                                  ybar, q);
 }
 
 template <typename T>
 void launch_axpby(const Geom &g, T a, const T *x, T b, const T *y, T *out, cudaStream_t st)
 {
-    k_axpby<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, a, x, b, y, out);
+    launch_pdl(k_axpby<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, a, x, b, y, out);
 }
 
 #define NM_VJP_INST(T)                                                                                          \
@@ -172,6 +177,7 @@ namespace nm {
 template <typename To>
 __global__ void k_cells_to_boundary(Geom g, const double *__restrict__ s, To *__restrict__ a)
 {
+    pdl_enter();
     long c = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (c >= g.n_cells) return;
     const int c1 = (int)(c % g.N1);
@@ -184,7 +190,7 @@ __global__ void k_cells_to_boundary(Geom g, const double *__restrict__ s, To *__
 template <typename To>
 void launch_cells_to_boundary(const Geom &g, const double *s, To *a, cudaStream_t st)
 {
-    k_cells_to_boundary<To><<<div_up(g.n_cells, 256), 256, 0, st>>>(g, s, a);
+    launch_pdl(k_cells_to_boundary<To>, div_up(g.n_cells, 256), 256, 0, st, g, s, a);
 }
 template void launch_cells_to_boundary<float>(const Geom &, const double *, float *, cudaStream_t);
 template void launch_cells_to_boundary<double>(const Geom &, const double *, double *, cudaStream_t);
@@ -196,6 +202,7 @@ namespace nm {
 template <typename T>
 __global__ void k_lincomb(long n_nodes, long ns, LinComb lc, T *__restrict__ out)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     for (int c = 0; c < 3; ++c) {
@@ -210,6 +217,7 @@ __global__ void k_lincomb(long n_nodes, long ns, LinComb lc, T *__restrict__ out
 template <typename T>
 __global__ void k_lincomb_d(long n_nodes, long ns, LinComb lc, double *__restrict__ out)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     for (int c = 0; c < 3; ++c) {
@@ -226,6 +234,7 @@ __global__ void k_renorm_adjoint(long n_nodes, long ns, const double *__restrict
                                  const double *__restrict__ lam, int renorm, double *__restrict__ lam_t,
                                  T *__restrict__ lam_tw)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     double mt[3], l[3];
@@ -256,6 +265,7 @@ __global__ void __launch_bounds__(256) k_loss_terms(long n_nodes, long ns, const
                                                     const double *__restrict__ W, const double *__restrict__ tg,
                                                     double *__restrict__ lam, double *__restrict__ partials)
 {
+    pdl_enter();
     __shared__ double sh[256];
     double acc = 0.0;
     for (long n = blockIdx.x * (long)blockDim.x + threadIdx.x; n < n_nodes; n += (long)gridDim.x * blockDim.x)
@@ -276,6 +286,7 @@ __global__ void __launch_bounds__(256) k_loss_terms(long n_nodes, long ns, const
 
 __global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict__ p, int n, double *out)
 {
+    pdl_enter();
     __shared__ double sh[1024];
     double v = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) v += p[i];
@@ -291,18 +302,18 @@ __global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict_
 template <typename T>
 void launch_lincomb(const Geom &g, const LinComb &lc, T *out, cudaStream_t st)
 {
-    k_lincomb<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, lc, out);
+    launch_pdl(k_lincomb<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, lc, out);
 }
 template <typename T>
 void launch_lincomb_d(const Geom &g, const LinComb &lc, double *out, cudaStream_t st)
 {
-    k_lincomb_d<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, lc, out);
+    launch_pdl(k_lincomb_d<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, lc, out);
 }
 template <typename T>
 void launch_renorm_adjoint(const Geom &g, const double *m, const LinComb &kb, double dt, const double *lam,
                            int renorm, double *lam_t, T *lam_t_w, cudaStream_t st)
 {
-    k_renorm_adjoint<T><<<div_up(g.n_nodes, 256), 256, 0, st>>>(g.n_nodes, g.ns, m, kb, dt, lam, renorm, lam_t,
+    launch_pdl(k_renorm_adjoint<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, kb, dt, lam, renorm, lam_t,
                                                                   lam_t_w);
 }
 int launch_loss_terms(const Geom &g, const double *m, const double *W, const double *target, double *lam,
@@ -310,17 +321,18 @@ int launch_loss_terms(const Geom &g, const double *m, const double *W, const dou
 {
     long b = (g.n_nodes + 255) / 256;
     int nb = (int)(b > 1024 ? 1024 : b);
-    k_loss_terms<<<nb, 256, 0, st>>>(g.n_nodes, g.ns, m, W, target, lam, partials);
+    launch_pdl(k_loss_terms, nb, 256, 0, st, g.n_nodes, g.ns, m, W, target, lam, partials);
     return nb;
 }
 void launch_sum_partials(const double *partials, int n, double *out, cudaStream_t st)
 {
-    k_sum_partials<<<1, 1024, 0, st>>>(partials, n, out);
+    launch_pdl(k_sum_partials, 1, 1024, 0, st, partials, n, out);
 }
 
 template <typename T>
 __global__ void k_accum_nodal(long n_nodes, long ns, const T *__restrict__ q, double scale, double *__restrict__ acc)
 {
+    pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     for (int c = 0; c < 3; ++c) acc[c * ns + n] += scale * (double)q[c * ns + n];
@@ -329,12 +341,13 @@ __global__ void k_accum_nodal(long n_nodes, long ns, const T *__restrict__ q, do
 template <typename T>
 void launch_accum_nodal(const Geom &g, const T *q, double scale, double *acc, cudaStream_t st)
 {
-    k_accum_nodal<T><<<(int)((g.n_nodes + 255) / 256), 256, 0, st>>>(g.n_nodes, g.ns, q, scale, acc);
+    launch_pdl(k_accum_nodal<T>, (int)((g.n_nodes + 255) / 256), 256, 0, st, g.n_nodes, g.ns, q, scale, acc);
 }
 
 __global__ void __launch_bounds__(256) k_sum_nodal3_partials(long n_nodes, long ns, const double *__restrict__ acc,
                                                               double *partials)
 {
+    pdl_enter();
     __shared__ double sh[3][256];
     double v[3] = {0.0, 0.0, 0.0};
     for (long n = blockIdx.x * (long)blockDim.x + threadIdx.x; n < n_nodes; n += (long)gridDim.x * blockDim.x)
@@ -354,8 +367,8 @@ void launch_sum_nodal3(const Geom &g, const double *acc, double *partials, doubl
 {
     long b = (g.n_nodes + 255) / 256;
     const int nb = (int)(b > 1024 ? 1024 : b);
-    k_sum_nodal3_partials<<<nb, 256, 0, st>>>(g.n_nodes, g.ns, acc, partials);
-    for (int c = 0; c < 3; ++c) k_sum_partials<<<1, 1024, 0, st>>>(partials + c * 1024, nb, out + c);
+    launch_pdl(k_sum_nodal3_partials, nb, 256, 0, st, g.n_nodes, g.ns, acc, partials);
+    for (int c = 0; c < 3; ++c) launch_pdl(k_sum_partials, 1, 1024, 0, st, partials + c * 1024, nb, out + c);
 }
 
 template void launch_accum_nodal<float>(const Geom &, const float *, double, double *, cudaStream_t);
