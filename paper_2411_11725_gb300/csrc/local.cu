@@ -162,13 +162,9 @@ struct NodeField {
     bool magnetic;
 };
 
-// Effective field at node (n1, n2, n3) = (x0 + tx, y0 + ty, z) from the shared planes.
-//   MODE 1 (interior, uniform material): every cell around the node exists, the 27 assembled weights
-//          are constants;
-//   MODE 2 (uniform material, any node): the weight of an offset is the per-pattern constant times the
-//          number of mesh cells holding both nodes, the product of per-axis counts;
-//   MODE 0 (general): the weights are summed over the adjacent cells' material values.
-template <typename T, int MODE>
+// Effective field at node (n1, n2, n3) = (x0 + tx, y0 + ty, z) from the shared planes: the weights are summed
+// over the adjacent cells' material values.
+template <typename T>
 __device__ __forceinline__ NodeField<T> node_field(const LocalParams<T> &p, const NodeSmem<T> &sm, int n1, int n2,
                                                    int n3, T im, int tx, int ty)
 {
@@ -185,112 +181,47 @@ __device__ __forceinline__ NodeField<T> node_field(const LocalParams<T> &p, cons
     }
     f.magnetic = im > T(0);
     T ex = 0, ey = 0, ez = 0, pe = 0;
-    if (MODE == 1) {
-        // sum_o w_o (m_{n+o} - m_n) = sum_{o != 0} w_o m_{n+o} - (sum w) m_n;  anisotropy: sum_o c_o m_{n+o}
-        T sx = 0, sy = 0, sz = 0, ax = 0, ay = 0, az = 0;
+    T a[8], ku[8];
 #pragma unroll
-        for (int o3 = -1; o3 <= 1; ++o3) {
-            const int slot = o3 < 0 ? szm : (o3 > 0 ? szp : sz0);
+    for (int i = 0; i < 8; ++i) {
+        const int c1 = n1 - ((i >> 2) & 1), c2 = n2 - ((i >> 1) & 1), c3 = n3 - (i & 1);
+        const bool valid = c1 >= 0 && c1 < g.N1 && c2 >= 0 && c2 < g.N2 && c3 >= 0 && c3 < g.N3;
+        const int c = valid ? (c3 * g.N2 + c2) * g.N1 + c1 : 0;
+        const T Ms = valid ? (p.Ms ? p.Ms[c] : p.Ms0) : T(0);
+        const bool mag = valid && Ms > T(0);
+        a[i] = (mag && (p.terms & NM_EXCH)) ? (p.A ? p.A[c] : p.A0) : T(0);
+        ku[i] = (mag && (p.terms & NM_ANIS)) ? (p.Ku ? p.Ku[c] : p.Ku0) : T(0);
+    }
 #pragma unroll
-            for (int o2 = -1; o2 <= 1; ++o2)
+    for (int o3 = -1; o3 <= 1; ++o3) {
+        const int slot = o3 < 0 ? szm : (o3 > 0 ? szp : sz0);
 #pragma unroll
-                for (int o1 = -1; o1 <= 1; ++o1) {
-                    const int k = (o3 + 1) * 9 + (o2 + 1) * 3 + (o1 + 1);
-                    const V4<T> q = sm.y.get(slot, cy0 + o2, cx0 + o1);
-                    if (k != 13) {
-                        sx += p.wex27[k] * q.x;
-                        sy += p.wex27[k] * q.y;
-                        sz += p.wex27[k] * q.z;
+        for (int o2 = -1; o2 <= 1; ++o2)
+#pragma unroll
+            for (int o1 = -1; o1 <= 1; ++o1) {
+                T S = 0, K = 0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int i1 = (i >> 2) & 1, i2 = (i >> 1) & 1, i3 = i & 1;
+                    const bool comp = (o1 == -1 ? i1 == 1 : (o1 == 1 ? i1 == 0 : true)) &&
+                                      (o2 == -1 ? i2 == 1 : (o2 == 1 ? i2 == 0 : true)) &&
+                                      (o3 == -1 ? i3 == 1 : (o3 == 1 ? i3 == 0 : true));
+                    if (comp) {
+                        S += a[i];
+                        K += ku[i];
                     }
-                    ax += p.wan27[k] * q.x;
-                    ay += p.wan27[k] * q.y;
-                    az += p.wan27[k] * q.z;
                 }
-        }
-        ex = sx - p.wex_sum * f.mx;
-        ey = sy - p.wex_sum * f.my;
-        ez = sz - p.wex_sum * f.mz;
-        pe = p.e0 * ax + p.e1 * ay + p.e2 * az;
-    } else if (MODE == 2) {
-        // cells n_k - 1 (pattern i_k = 1) and n_k (i_k = 0) along each axis
-        const int cm1 = n1 >= 1 && n1 - 1 < g.N1, cp1 = n1 < g.N1;
-        const int cm2 = n2 >= 1 && n2 - 1 < g.N2, cp2 = n2 < g.N2;
-        const int cm3 = n3 >= 1 && n3 - 1 < g.N3, cp3 = n3 < g.N3;
-        T sx = 0, sy = 0, sz = 0, ax = 0, ay = 0, az = 0, wsum = 0;
-#pragma unroll
-        for (int o3 = -1; o3 <= 1; ++o3) {
-            const int slot = o3 < 0 ? szm : (o3 > 0 ? szp : sz0);
-            const int k3 = o3 < 0 ? cm3 : (o3 > 0 ? cp3 : cm3 + cp3);
-#pragma unroll
-            for (int o2 = -1; o2 <= 1; ++o2) {
-                const int k23 = k3 * (o2 < 0 ? cm2 : (o2 > 0 ? cp2 : cm2 + cp2));
-#pragma unroll
-                for (int o1 = -1; o1 <= 1; ++o1) {
-                    const int cnt = k23 * (o1 < 0 ? cm1 : (o1 > 0 ? cp1 : cm1 + cp1));
-                    const int d = ((o1 != 0) << 2) | ((o2 != 0) << 1) | (o3 != 0);
-                    const T fc = (T)cnt;
-                    const V4<T> q = sm.y.get(slot, cy0 + o2, cx0 + o1);
-                    if (d != 0) {
-                        const T w = p.wexd[d] * fc;
-                        sx += w * q.x;
-                        sy += w * q.y;
-                        sz += w * q.z;
-                        wsum += w;
-                    }
-                    const T wa = p.wand[d] * fc;
-                    ax += wa * q.x;
-                    ay += wa * q.y;
-                    az += wa * q.z;
+                const int d = ((o1 != 0) << 2) | ((o2 != 0) << 1) | (o3 != 0);
+                const bool self = (o1 == 0 && o2 == 0 && o3 == 0);
+                const V4<T> q = sm.y.get(slot, cy0 + o2, cx0 + o1);
+                if (!self) {
+                    const T w = p.Wex[d] * S;
+                    ex += w * (q.x - f.mx);
+                    ey += w * (q.y - f.my);
+                    ez += w * (q.z - f.mz);
                 }
+                pe += p.Wm[d] * K * (p.e0 * q.x + p.e1 * q.y + p.e2 * q.z);
             }
-        }
-        ex = sx - wsum * f.mx;
-        ey = sy - wsum * f.my;
-        ez = sz - wsum * f.mz;
-        pe = p.e0 * ax + p.e1 * ay + p.e2 * az;
-    } else {
-        T a[8], ku[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c1 = n1 - ((i >> 2) & 1), c2 = n2 - ((i >> 1) & 1), c3 = n3 - (i & 1);
-            const bool valid = c1 >= 0 && c1 < g.N1 && c2 >= 0 && c2 < g.N2 && c3 >= 0 && c3 < g.N3;
-            const int c = valid ? (c3 * g.N2 + c2) * g.N1 + c1 : 0;
-            const T Ms = valid ? (p.Ms ? p.Ms[c] : p.Ms0) : T(0);
-            const bool mag = valid && Ms > T(0);
-            a[i] = (mag && (p.terms & NM_EXCH)) ? (p.A ? p.A[c] : p.A0) : T(0);
-            ku[i] = (mag && (p.terms & NM_ANIS)) ? (p.Ku ? p.Ku[c] : p.Ku0) : T(0);
-        }
-#pragma unroll
-        for (int o3 = -1; o3 <= 1; ++o3) {
-            const int slot = o3 < 0 ? szm : (o3 > 0 ? szp : sz0);
-#pragma unroll
-            for (int o2 = -1; o2 <= 1; ++o2)
-#pragma unroll
-                for (int o1 = -1; o1 <= 1; ++o1) {
-                    T S = 0, K = 0;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int i1 = (i >> 2) & 1, i2 = (i >> 1) & 1, i3 = i & 1;
-                        const bool comp = (o1 == -1 ? i1 == 1 : (o1 == 1 ? i1 == 0 : true)) &&
-                                          (o2 == -1 ? i2 == 1 : (o2 == 1 ? i2 == 0 : true)) &&
-                                          (o3 == -1 ? i3 == 1 : (o3 == 1 ? i3 == 0 : true));
-                        if (comp) {
-                            S += a[i];
-                            K += ku[i];
-                        }
-                    }
-                    const int d = ((o1 != 0) << 2) | ((o2 != 0) << 1) | (o3 != 0);
-                    const bool self = (o1 == 0 && o2 == 0 && o3 == 0);
-                    const V4<T> q = sm.y.get(slot, cy0 + o2, cx0 + o1);
-                    if (!self) {
-                        const T w = p.Wex[d] * S;
-                        ex += w * (q.x - f.mx);
-                        ey += w * (q.y - f.my);
-                        ez += w * (q.z - f.mz);
-                    }
-                    pe += p.Wm[d] * K * (p.e0 * q.x + p.e1 * q.y + p.e2 * q.z);
-                }
-        }
     }
     // -dE / mass: exchange and anisotropy
     T hx = -ex + T(2) * p.e0 * pe;
@@ -427,8 +358,6 @@ __global__ void __launch_bounds__(kTX *kTY<T>, sizeof(T) == 4 ? 6 : 3) k_node(Lo
     double dt = 0.0;
     if (STAGE) dt = sa.ctl ? sa.ctl->dt : 0.0;
     const float dtf = (float)dt;
-    // the tile's x-y footprint has all eight cells around every node (uniform material)
-    const bool tile_inner = p.uniform && x0 >= 1 && x0 + kTX <= g.N1 && y0 >= 1 && y0 + TY <= g.N2;
     for (int z = z0; z < z1; ++z) {
         // start the copies for the next plane (into the slots of planes z - 2 and cells z - 2, free since
         // the barrier that ended the previous iteration), then wait for everything but them
@@ -471,14 +400,11 @@ __global__ void __launch_bounds__(kTX *kTY<T>, sizeof(T) == 4 ? 6 : 3) k_node(Lo
         }
         asm volatile("cp.async.wait_group 1;\n" ::: "memory");
         __syncthreads();
-        const bool interior = tile_inner && z >= 1 && z <= g.N3 - 1;
         if constexpr (OWN) {
             if (active) im = (T)own_sm[z & 1][0][ty][tx];
         }
         if (active) {
-            NodeField<T> f = interior    ? node_field<T, 1>(p, sm, n1, n2, z, im, tx, ty)
-                             : p.uniform ? node_field<T, 2>(p, sm, n1, n2, z, im, tx, ty)
-                                         : node_field<T, 0>(p, sm, n1, n2, z, im, tx, ty);
+            NodeField<T> f = node_field<T>(p, sm, n1, n2, z, im, tx, ty);
             if (DMI) {
                 const T sc = p.raw ? T(1) : im;
                 f.hx += sc * dmx;
@@ -945,10 +871,14 @@ void launch_heff(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaSt
         launch_pdl(k_node1d<T, false>, p.g.nn1, kNode1dThreads, 0, st, p, y, h_out, nullptr, StageArgs{}, t);
         return;
     }
+    if (p.hdmi) launch_pdl(k_dmi<T>, div_up(p.g.n_nodes, 256), 256, 0, st, p, y, p.hdmi);
+    if (p.uniform) {
+        launch_heff_uniform<T>(p, y, h_out, t, st);
+        return;
+    }
     int nb;
     if (p.hdmi) {
         const NodeGrid ng = node_grid<T, false, true>(p.g, &nb);
-        launch_pdl(k_dmi<T>, div_up(p.g.n_nodes, 256), 256, 0, st, p, y, p.hdmi);
         launch_pdl(k_node<T, false, true>, nb, kTX * kTY<T>, 0, st, p, y, h_out, nullptr, StageArgs{}, t, ng);
         return;
     }
@@ -968,10 +898,14 @@ void launch_llg_stage(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, 
         launch_pdl(k_node1d<T, true>, p.g.nn1, kNode1dThreads, 0, st, p, y, k_out, y_next, sa, 0.0);
         return;
     }
+    if (p.hdmi) launch_pdl(k_dmi<T>, div_up(p.g.n_nodes, 256), 256, 0, st, p, y, p.hdmi);
+    if (p.uniform) {
+        launch_llg_stage_uniform<T>(p, y, k_out, y_next, sa, st);
+        return;
+    }
     int nb;
     if (p.hdmi) {
         const NodeGrid ng = node_grid<T, true, true>(p.g, &nb);
-        launch_pdl(k_dmi<T>, div_up(p.g.n_nodes, 256), 256, 0, st, p, y, p.hdmi);
         launch_pdl(k_node<T, true, true>, nb, kTX * kTY<T>, 0, st, p, y, k_out, y_next, sa, 0.0, ng);
         return;
     }

@@ -12,14 +12,10 @@ struct LocalParams {
     Geom g;
     T Wex[8];          // int_cell 2 grad(phi_i).grad(phi_i') for the pattern d (per unit A)
     T Wm[8];           // int_cell phi_i phi_i' for the pattern d
-    // Interior nodes of a uniform material (no cell maps, Ms0 > 0): the 27 assembled weights of the
-    // neighbour offsets o (index (o3+1)*9 + (o2+1)*3 + (o1+1)), exchange (self weight unused) and
-    // anisotropy, and the sum of the exchange weights.  uniform = 0 disables that path.
+    // Uniform material (no cell maps, Ms0 > 0; trilinear basis): node_uniform.cu.  2 A and 2 Ku (0 for terms
+    // that are off) times the constants of the one-dimensional element matrices, and 1 / (mu0 V/8 Ms0).
     int uniform;
-    T wex27[27], wan27[27], wex_sum;
-    // uniform material at any node: Wex[d] A and Wm[d] Ku (0 for terms that are off); the weight of an
-    // offset is this times the number of mesh cells that hold both nodes, a product of per-axis counts
-    T wexd[8], wand[8];
+    double ucx, ucy, ucz, uan, uim;
     T mu0V8;           // mu0 * V / 8
     // 2D basis (section "Low-Dimensional Geometries"): the in-plane pattern integrals per cell layer
     // (pattern d = 2 |o1| + |o2|), through the layer's thickness, and mu0 V / 4
@@ -73,6 +69,13 @@ void launch_heff(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaSt
 template <typename T>
 void launch_llg_stage(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa,
                       cudaStream_t st);
+
+// the same for a uniform material (p.uniform) on the trilinear basis; DMI reads the raw field p.hdmi
+template <typename T>
+void launch_heff_uniform(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaStream_t st);
+template <typename T>
+void launch_llg_stage_uniform(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa,
+                              cudaStream_t st);
 
 // lumped mass: inv_mass_n = 1 / (mu0 V/8 sum_{c∋n} Ms_c); counts magnetic nodes into *n_active (device)
 template <typename T>

@@ -1,0 +1,522 @@
+// Node kernel of the trilinear basis for a uniform material (no cell maps, Ms > 0): exchange, uniaxial
+// anisotropy, Zeeman and the cell->node demag average, divided by the lumped nodal mass (Eqs.
+// weak_form_impl_f, weak_form_impl, mass_lumping), followed by the LLG right-hand side (Eq. llg) and the next
+// Runge-Kutta stage input.
+//
+// With one A and one Ku on a box of cells the assembled operators are sums of tensor products of the
+// one-dimensional stiffness and mass matrices, which at a node with n adjacent cells along the axis (n = 2
+// inside, 1 at an end) act as
+//   K u = (n u0 - (u- + u+)) / dx,      M u = (2 n u0 + (u- + u+)) dx / 6,
+// with u = 0 beyond the ends.  The field is
+//   -dE_ex = -2 A (K1 M2 M3 + M1 K2 M3 + M1 M2 K3) m,   -dE_an = 2 Ku e (M1 M2 M3) (e . m),
+// evaluated axis by axis: along x and y for each node plane (9 neighbours), along z by carrying two partial
+// sums per component up the walk.  That is about 65 multiply-adds and 9 shared-memory vectors per node
+// instead of the 162 and 27 of the assembled 27-point form, and the boundary needs no case of its own.
+#include <type_traits>
+
+#include "local.cuh"
+
+namespace nm {
+
+// Tile of 32 x 4 nodes walked along z by 128 threads, eight FP32 blocks per SM at 64 registers.  Measured per
+// stage at 1024x1024x32 (FP32) / 512x512x16: this kernel 0.59 ms / 87 us, against 1.04 ms / 154 us for the
+// assembled 27-point form and 0.64 ms / 99 us with two rows per thread (96 registers, five blocks per SM).
+constexpr int kUX = 32, kUY = 4, kUThreads = kUX * kUY;
+constexpr int kUSlots = 3;
+
+// A 3-vector of the working precision.  FP32: x and y as one packed pair (fma.rn.f32x2: one instruction for
+// both, rounded as the scalar ones) and z apart, the layout of the shared planes.
+template <typename T>
+struct Vec {
+    T x, y, z;
+};
+template <>
+struct Vec<float> {
+    unsigned long long xy;
+    float z;
+};
+__device__ __forceinline__ unsigned long long pk(float a, float b)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpk(unsigned long long r, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> vadd(const Vec<T> &a, const Vec<T> &b)
+{
+    if constexpr (sizeof(T) == 4) {
+        Vec<float> r;
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.xy) : "l"(a.xy), "l"(b.xy));
+        r.z = a.z + b.z;
+        return r;
+    } else {
+        return Vec<T>{a.x + b.x, a.y + b.y, a.z + b.z};
+    }
+}
+// c v + w
+template <typename T>
+__device__ __forceinline__ Vec<T> vfma(T c, const Vec<T> &v, const Vec<T> &w)
+{
+    if constexpr (sizeof(T) == 4) {
+        Vec<float> r;
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.xy) : "l"(pk(c, c)), "l"(v.xy), "l"(w.xy));
+        r.z = fmaf(c, v.z, w.z);
+        return r;
+    } else {
+        return Vec<T>{fma(c, v.x, w.x), fma(c, v.y, w.y), fma(c, v.z, w.z)};
+    }
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> vmul(T c, const Vec<T> &v)
+{
+    if constexpr (sizeof(T) == 4) {
+        Vec<float> r;
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.xy) : "l"(pk(c, c)), "l"(v.xy));
+        r.z = c * v.z;
+        return r;
+    } else {
+        return Vec<T>{c * v.x, c * v.y, c * v.z};
+    }
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> vzero()
+{
+    if constexpr (sizeof(T) == 4) return Vec<float>{0ull, 0.f};
+    else return Vec<T>{T(0), T(0), T(0)};
+}
+template <typename T>
+__device__ __forceinline__ void vget(const Vec<T> &v, T &x, T &y, T &z)
+{
+    if constexpr (sizeof(T) == 4) {
+        unpk(v.xy, x, y);
+        z = v.z;
+    } else {
+        x = v.x;
+        y = v.y;
+        z = v.z;
+    }
+}
+
+// kUSlots planes of R x C 3-vectors in shared memory
+template <typename T, int R, int C>
+struct VPlanes {
+    T v[kUSlots][R * C][3];
+    __device__ __forceinline__ Vec<T> get(int s, int i) const { return Vec<T>{v[s][i][0], v[s][i][1], v[s][i][2]}; }
+    __device__ __forceinline__ T *p(int s, int i, int c) { return &v[s][i][c]; }
+};
+template <int R, int C>
+struct VPlanes<float, R, C> {
+    unsigned long long xy[kUSlots][R * C];
+    float z[kUSlots][R * C];
+    __device__ __forceinline__ Vec<float> get(int s, int i) const { return Vec<float>{xy[s][i], z[s][i]}; }
+    __device__ __forceinline__ float *p(int s, int i, int c)
+    {
+        return c == 2 ? &z[s][i] : reinterpret_cast<float *>(&xy[s][i]) + c;
+    }
+};
+
+template <typename T>
+struct NodeUSmem {
+    static constexpr int SX = kUX + 2, SY = kUY + 2, CX = kUX + 1, CY = kUY + 1;
+    VPlanes<T, SY, SX> y;  // node plane p in slot p mod 3 (counted from the first plane of the walk)
+    VPlanes<T, CY, CX> c;  // cell plane p - 1 (Ms_c H_c) beside node plane p
+    T hf[4];               // uniform applied field, time factor of the cell field
+};
+
+template <typename T>
+struct NodeUArgs {
+    int nn1, nn2, nn3, N1, N2, N3, ns, cs;
+    int bxn, full, chunks, zc;  // blocks b < full walk tile b over all planes; the other tiles are split into
+                                // `chunks` blocks of zc planes
+    T cx, cy, cz, can;          // 2 A x element constants of the three axes; 2 Ku V / 216
+    T e0, e1, e2;
+    T im1, mu0V8;               // 1 / (mu0 V/8 Ms); mu0 V/8
+    T gam, alpha;
+    const T *y, *MsH, *Msh, *hdmi;
+    T *out, *y_next;
+    const double *m;
+    const float *mf;
+    const T *k[4];              // earlier slopes with non-zero coefficients in the next stage input
+    T a[4], as;                 // their coefficients, and that of the slope being written
+    const StepCtl *ctl;
+    double c_s, t_fixed, hu0, hu1, hu2, hu_freq, hu_phase, hc_freq, hc_phase;
+    int raw, zee;
+};
+
+template <typename T>
+__device__ __forceinline__ double u_time_factor(double f, double ph, double t)
+{
+    return f == 0.0 ? 1.0 : sin(2.0 * 3.14159265358979323846 * f * t + ph);
+}
+
+// asynchronous copy of one value, or zero fill when !in
+template <typename T>
+__device__ __forceinline__ void cp_elem(T *dst, const T *src, bool in)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = in ? (int)sizeof(T) : 0;
+    if (sizeof(T) == 4)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+// What a kernel instance writes: the field (kHeff), the slope (kSlope), or the slope and the next stage input
+// formed from NK >= 0 earlier slopes.  M64: the next input is formed from the FP64 m (always in FP64, and in
+// FP32 where no FP32 copy of m is kept).
+constexpr int kHeff = -2, kSlope = -1;
+
+template <typename T, int NK, bool M64>
+__global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(const __grid_constant__ NodeUArgs<T> p)
+{
+    pdl_enter();
+    if (NK != kHeff && p.ctl && p.ctl->done) return;
+    using S = NodeUSmem<T>;
+    __shared__ S sm;
+    const int b = blockIdx.x, split = b >= p.full;
+    const int tile = split ? p.full + (b - p.full) / p.chunks : b;
+    const int z0 = split ? (b - p.full) % p.chunks * p.zc : 0, z1 = split ? min(p.nn3, z0 + p.zc) : p.nn3;
+    const int x0 = tile % p.bxn * kUX, y0 = tile / p.bxn * kUY;
+    const int tx = threadIdx.x % kUX, ty = threadIdx.x / kUX;
+    const int n1 = x0 + tx, n2 = y0 + ty;
+    if (threadIdx.x == 0) {
+        const double t = p.ctl ? p.ctl->t + p.c_s * p.ctl->dt : p.t_fixed;
+        const double su = u_time_factor<T>(p.hu_freq, p.hu_phase, t);
+        sm.hf[0] = (T)(p.hu0 * su);
+        sm.hf[1] = (T)(p.hu1 * su);
+        sm.hf[2] = (T)(p.hu2 * su);
+        sm.hf[3] = (T)u_time_factor<T>(p.hc_freq, p.hc_phase, t);
+    }
+    // the elements of every node and cell plane that this thread copies: offset within the plane, or -1
+    // outside the mesh (zero fill)
+    constexpr int EN = (S::SX * S::SY + kUThreads - 1) / kUThreads, EC = (S::CX * S::CY + kUThreads - 1) / kUThreads;
+    int no[EN], co[EC];
+#pragma unroll
+    for (int k = 0; k < EN; ++k) {
+        const int t = threadIdx.x + k * kUThreads, r = t / S::SX, c = t - r * S::SX;
+        const int i = x0 - 1 + c, j = y0 - 1 + r;
+        no[k] = (i >= 0 && i < p.nn1 && j >= 0 && j < p.nn2) ? j * p.nn1 + i : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < EC; ++k) {
+        const int t = threadIdx.x + k * kUThreads, r = t / S::CX, c = t - r * S::CX;
+        const int i = x0 - 1 + c, j = y0 - 1 + r;
+        co[k] = (i >= 0 && i < p.N1 && j >= 0 && j < p.N2) ? j * p.N1 + i : -1;
+    }
+    const int np = p.nn1 * p.nn2, ncp = p.N1 * p.N2;
+    // node plane q and cell plane q - 1 into slot s (planes outside the mesh are not read: their terms are
+    // skipped)
+    auto load_plane = [&](int q, int s) {
+        if (q >= 0 && q < p.nn3) {
+#pragma unroll
+            for (int k = 0; k < EN; ++k) {
+                const int t = threadIdx.x + k * kUThreads;
+                if (t < S::SX * S::SY) {
+                    const bool in = no[k] >= 0;
+                    const T *src = p.y + (in ? q * np + no[k] : 0);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) cp_elem(sm.y.p(s, t, c), src + c * p.ns, in);
+                }
+            }
+        }
+        if (p.MsH && q >= 1 && q - 1 < p.N3) {
+#pragma unroll
+            for (int k = 0; k < EC; ++k) {
+                const int t = threadIdx.x + k * kUThreads;
+                if (t < S::CX * S::CY) {
+                    const bool in = co[k] >= 0;
+                    const T *src = p.MsH + (in ? (q - 1) * ncp + co[k] : 0);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) cp_elem(sm.c.p(s, t, c), src + c * p.cs, in);
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    load_plane(z0 - 1, 0);
+    load_plane(z0, 1);
+    const T dt = NK >= 0 && p.ctl ? (T)p.ctl->dt : T(0);
+    const double dt64 = NK >= 0 && p.ctl ? p.ctl->dt : 0.0;
+    // cells on both sides of the node along x and y
+    const T nx = n1 >= 1 && n1 < p.N1 ? T(2) : T(1), ny = n2 >= 1 && n2 < p.N2 ? T(2) : T(1);
+    const bool active = n1 < p.nn1 && n2 < p.nn2;
+    // carried up the walk: the part of the node being completed that planes z - 1 and z gave, the share of
+    // plane z in the node above, m and the cell sum of plane z - 1
+    Vec<T> acc = vzero<T>(), up = acc, mc = acc, cc = acc;
+    T accR = 0, upR = 0;
+    int s = 0;
+    for (int q = z0 - 1; q <= z1; ++q) {
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncthreads();  // plane q has arrived for all; slot (s + 2) mod 3 (plane q - 1) is free
+        load_plane(q + 2 <= z1 ? q + 2 : -1, s + 2 >= kUSlots ? s + 2 - kUSlots : s + 2);
+        Vec<T> own = vzero<T>(), fin = own, mnew = own, ccur = own;
+        T ownR = 0, finR = 0;
+        if (q >= 0 && q < p.nn3) {
+            // row sums along x of rows n2 - 1 .. n2 + 1: a = 6 M1 m / dx, d = -dx K1 m
+            Vec<T> a[3], d[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const int i = (ty + r) * S::SX + tx;
+                const Vec<T> c = sm.y.get(s, i + 1), e = vadd(sm.y.get(s, i), sm.y.get(s, i + 2));
+                a[r] = vfma(T(2) * nx, c, e);
+                d[r] = vfma(-nx, c, e);
+                if (r == 1) mnew = c;
+            }
+            const T nz = q >= 1 && q < p.N3 ? T(2) : T(1);  // cells on both sides along z
+            const Vec<T> as = vadd(a[0], a[2]), ds = vadd(d[0], d[2]);
+            const Vec<T> P = vfma(T(2) * ny, a[1], as);     // M1 M2
+            const Vec<T> ka = vfma(-ny, a[1], as);          // -M1 K2
+            const Vec<T> kd = vfma(T(2) * ny, d[1], ds);    // -K1 M2
+            const Vec<T> Q = vfma(p.cx, kd, vmul(p.cy, ka));
+            fin = vfma(p.cz, P, Q);                         // share in the nodes of the planes beside
+            own = vfma(T(2) * nz, Q, vmul(-nz * p.cz, P));  // share in the plane's own node
+            T px, py, pz;
+            vget(P, px, py, pz);
+            finR = p.e0 * px + p.e1 * py + p.e2 * pz;
+            ownR = T(2) * nz * finR;
+        }
+        // Ms H over the four cells of plane q - 1 around the node
+        if (p.MsH && q >= 1 && q - 1 < p.N3) {
+            const int i = ty * S::CX + tx;
+            ccur = vadd(vadd(sm.c.get(s, i), sm.c.get(s, i + 1)),
+                        vadd(sm.c.get(s, i + S::CX), sm.c.get(s, i + S::CX + 1)));
+        }
+        const int z = q - 1;
+        if (z >= z0 && active) {
+            const int n = z * np + n2 * p.nn1 + n1;
+            T hx, hy, hz, dx, dy, dz, mx, my, mz;
+            vget(vadd(acc, fin), hx, hy, hz);
+            const T pe = p.can * (accR + finR);
+            hx += p.e0 * pe;
+            hy += p.e1 * pe;
+            hz += p.e2 * pe;
+            vget(vadd(cc, ccur), dx, dy, dz);
+            vget(mc, mx, my, mz);
+            if (p.Msh && p.zee) {
+                T sx = 0, sy = 0, sz = 0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int c1 = n1 - ((i >> 2) & 1), c2 = n2 - ((i >> 1) & 1), c3 = z - (i & 1);
+                    if (c1 >= 0 && c1 < p.N1 && c2 >= 0 && c2 < p.N2 && c3 >= 0 && c3 < p.N3) {
+                        const int c = (c3 * p.N2 + c2) * p.N1 + c1;
+                        sx += p.Msh[c];
+                        sy += p.Msh[p.cs + c];
+                        sz += p.Msh[2 * p.cs + c];
+                    }
+                }
+                dx += sm.hf[3] * sx;
+                dy += sm.hf[3] * sy;
+                dz += sm.hf[3] * sz;
+            }
+            hx += p.mu0V8 * dx;
+            hy += p.mu0V8 * dy;
+            hz += p.mu0V8 * dz;
+            if (p.hdmi) {
+                hx += p.hdmi[n];
+                hy += p.hdmi[p.ns + n];
+                hz += p.hdmi[2 * p.ns + n];
+            }
+            if (!p.raw) {
+                // 1 / mass: the node's cells number nx ny nz (a power of two)
+                const T im = p.im1 * (z >= 1 && z < p.N3 ? T(0.5) : T(1)) * (nx == T(2) ? T(0.5) : T(1)) *
+                             (ny == T(2) ? T(0.5) : T(1));
+                hx *= im;
+                hy *= im;
+                hz *= im;
+                if (p.zee) {
+                    hx += sm.hf[0];
+                    hy += sm.hf[1];
+                    hz += sm.hf[2];
+                }
+            }
+            if (NK == kHeff) {
+                p.out[n] = hx;
+                p.out[p.ns + n] = hy;
+                p.out[2 * p.ns + n] = hz;
+            } else {
+                // the next stage input's own values, all loads issued together
+                T kv[NK > 0 ? NK : 1][3], m0[3];
+                double md[3];
+                if (NK >= 0) {
+#pragma unroll
+                    for (int i = 0; i < NK; ++i)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) kv[i][c] = p.k[i][c * p.ns + n];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        if (M64) md[c] = p.m[c * p.ns + n];
+                        else m0[c] = (T)p.mf[c * p.ns + n];
+                    }
+                }
+                // k = -gamma' (m x H + alpha m x (m x H))
+                const T ax = my * hz - mz * hy, ay = mz * hx - mx * hz, az = mx * hy - my * hx;
+                const T bx = my * az - mz * ay, by = mz * ax - mx * az, bz = mx * ay - my * ax;
+                T kk[3];
+                kk[0] = -p.gam * (ax + p.alpha * bx);
+                kk[1] = -p.gam * (ay + p.alpha * by);
+                kk[2] = -p.gam * (az + p.alpha * bz);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) p.out[c * p.ns + n] = kk[c];
+                if (NK >= 0) {
+                    // y_{s+1} = m + dt sum_j a_j k_j, the slope combination in the working precision
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        T sum = 0;
+#pragma unroll
+                        for (int i = 0; i < NK; ++i) sum += p.a[i] * kv[i][c];
+                        sum += p.as * kk[c];
+                        p.y_next[c * p.ns + n] = M64 ? (T)(md[c] + dt64 * (double)sum) : m0[c] + dt * sum;
+                    }
+                }
+            }
+        }
+        acc = vadd(up, own);
+        accR = upR + ownR;
+        up = fin;
+        upR = finR;
+        mc = mnew;
+        cc = ccur;
+        s = s + 1 >= kUSlots ? 0 : s + 1;
+    }
+}
+
+// Split of the walk: cost in plane units of a grid whose tiles are cut into `chunks` pieces, from the latency
+// of one block (its planes, two more for the halo, and the start of the walk) and the planes an SM works
+// through when the blocks are dealt out evenly (about four planes of one block cost an SM as much time as the
+// latency of one).
+static void node_u_grid(int nn1, int nn2, int nn3, int sms, int *bxn, int *full, int *chunks, int *zc, int *blocks)
+{
+    *bxn = div_up(nn1, kUX);
+    const int tiles = *bxn * div_up(nn2, kUY);
+    double best = 1e300;
+    for (int f = 0; f < 2; ++f) {
+        const int fl = f ? tiles - tiles % sms : 0, rest = tiles - fl;
+        if (f && fl == 0) break;
+        for (int c = 1; c <= nn3; ++c) {
+            const int z = div_up(nn3, c), ch = div_up(nn3, z);
+            if (c > 1 && ch != c) continue;  // (the same split as fewer chunks)
+            const double work = (double)(fl / sms) * (nn3 + 2) + div_up((long)rest * ch, sms) * (double)(z + 2);
+            const double lat = 4.0 * ((fl ? nn3 : z) + 4);
+            const double cost = work > lat ? work : lat;
+            if (cost < best * 0.999) {
+                best = cost;
+                *full = fl;
+                *zc = z;
+                *chunks = ch;
+                *blocks = fl + rest * ch;
+            }
+        }
+    }
+}
+
+template <typename T, int NK, bool M64>
+static void launch_u(const NodeUArgs<T> &a, int blocks, cudaStream_t st)
+{
+    launch_pdl(k_node_u<T, NK, M64>, blocks, kUThreads, 0, st, a);
+}
+
+template <typename T>
+static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *y_next, const StageArgs *sa, double t,
+                                cudaStream_t st)
+{
+    const Geom &g = p.g;
+    NodeUArgs<T> a{};
+    a.nn1 = g.nn1; a.nn2 = g.nn2; a.nn3 = g.nn3;
+    a.N1 = g.N1; a.N2 = g.N2; a.N3 = g.N3;
+    a.ns = (int)g.ns;
+    a.cs = (int)g.cs;
+    int blocks = 0;
+    static int sms = 0;
+    if (sms == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
+    }
+    node_u_grid(g.nn1, g.nn2, g.nn3, sms, &a.bxn, &a.full, &a.chunks, &a.zc, &blocks);
+    a.cx = (T)p.ucx;
+    a.cy = (T)p.ucy;
+    a.cz = (T)p.ucz;
+    a.can = (T)p.uan;
+    a.e0 = p.e0; a.e1 = p.e1; a.e2 = p.e2;
+    a.im1 = (T)p.uim;
+    a.mu0V8 = p.mu0V8;
+    a.gam = p.gam_t;
+    a.alpha = p.alpha_t;
+    a.y = y;
+    a.MsH = (p.terms & NM_DEMAG) ? p.MsH : nullptr;
+    a.Msh = p.Msh;
+    a.hdmi = p.hdmi;
+    a.out = out;
+    a.y_next = y_next;
+    a.hu0 = p.hu0; a.hu1 = p.hu1; a.hu2 = p.hu2;
+    a.hu_freq = p.hu_freq; a.hu_phase = p.hu_phase;
+    a.hc_freq = p.hc_freq; a.hc_phase = p.hc_phase;
+    a.raw = p.raw;
+    a.zee = (p.terms & NM_ZEE) != 0;
+    a.t_fixed = t;
+    if (!sa) {
+        launch_u<T, kHeff, true>(a, blocks, st);
+        return;
+    }
+    a.ctl = sa->ctl;
+    a.c_s = sa->c_s;
+    a.t_fixed = sa->t_fixed;
+    if (!y_next) {
+        launch_u<T, kSlope, true>(a, blocks, st);
+        return;
+    }
+    a.m = sa->m;
+    a.mf = sa->mf;
+    a.as = sizeof(T) == 4 ? (T)sa->af_s : (T)sa->a_s;
+    int nk = 0;
+    for (int j = 0; j + 1 < sa->s && j < 7; ++j) {
+        const T c = sizeof(T) == 4 ? (T)sa->af[j] : (T)sa->a[j];
+        if (c == T(0)) continue;
+        a.k[nk] = (const T *)sa->k[j];
+        a.a[nk] = c;
+        ++nk;
+    }
+    const bool m64 = sizeof(T) == 8 || !sa->mf;
+    auto go = [&](auto n) {
+        constexpr int NK = decltype(n)::value;
+        if constexpr (sizeof(T) == 4) {
+            if (!m64) {
+                launch_u<T, NK, false>(a, blocks, st);
+                return;
+            }
+        }
+        launch_u<T, NK, true>(a, blocks, st);
+    };
+    switch (nk) {
+    case 0: go(std::integral_constant<int, 0>{}); break;
+    case 1: go(std::integral_constant<int, 1>{}); break;
+    case 2: go(std::integral_constant<int, 2>{}); break;
+    case 3: go(std::integral_constant<int, 3>{}); break;
+    default: go(std::integral_constant<int, 4>{}); break;
+    }
+}
+
+template <typename T>
+void launch_heff_uniform(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaStream_t st)
+{
+    launch_node_uniform<T>(p, y, h_out, nullptr, nullptr, t, st);
+}
+template <typename T>
+void launch_llg_stage_uniform(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa,
+                              cudaStream_t st)
+{
+    launch_node_uniform<T>(p, y, k_out, y_next, &sa, 0.0, st);
+}
+
+template void launch_heff_uniform<float>(const LocalParams<float> &, const float *, float *, double, cudaStream_t);
+template void launch_heff_uniform<double>(const LocalParams<double> &, const double *, double *, double, cudaStream_t);
+template void launch_llg_stage_uniform<float>(const LocalParams<float> &, const float *, float *, float *,
+                                              const StageArgs &, cudaStream_t);
+template void launch_llg_stage_uniform<double>(const LocalParams<double> &, const double *, double *, double *,
+                                               const StageArgs &, cudaStream_t);
+
+}  // namespace nm
