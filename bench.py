@@ -145,8 +145,8 @@ def algorithmic_bytes(name, stage, n, b, with_maps):
         return 2 * 3 * c * X * P2 * N3 + 6 * b * X * H2 * H3
     if name == "demag_y_inv":
         return 3 * c * X * P2 * N3 + 3 * c * X * N2 * N3
-    if name == "demag_y_conv":
-        return 2 * 3 * c * X * N2 + 6 * b * X * H2
+    if name == "demag_yz_conv":
+        return 2 * 3 * c * X * N2 * N3 + 6 * b * X * H2 * H3
     if name == "demag_x_inv":
         return 3 * c * X * N2 * N3 + ms + 3 * b * Nc
     # stage inputs and the error scale read the FP64 m (24 B/node), or in the FP32 path its FP32 copy

@@ -56,10 +56,12 @@ struct DemagPlan {
     size_t y_smem;
     int z_G, z_KY, z_threads;
     size_t z_smem;
-    bool z_reg;                // FP32, P3 <= 64: the register z convolution (two threads per line)
-    int yc_G, yc_threads;
-    size_t yc_smem;
+    bool z_reg;                // short lines: the register z convolution
     size_t yi_smem;            // y passes with a TMA tile (alignment slack and barrier)
+    bool yz;                   // one fused y-z convolution instead of the y and z passes
+    int yz_lgG, yz_nlp;        // log2 of its kx columns per block, row stride of its tile
+    unsigned yz_plan;          // log2 radices of its y stages, four bits each
+    size_t yz_smem;
 };
 template <typename T>
 DemagPlan demag_plan(const Geom &g);

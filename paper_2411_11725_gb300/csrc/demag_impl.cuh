@@ -1,8 +1,7 @@
 // Demag passes (section "Demagnetization Field"): node->cell averaging fused into a pruned
 // real-to-complex x transform, pruned y transforms, a z pass that fuses forward z, the pointwise
-// product with the symmetric tensor spectrum and inverse z (or, for one cell layer, a y pass that
-// fuses forward y, the product and inverse y), and a pruned complex-to-real x transform that writes
-// Ms_c H_c per cell.
+// product with the symmetric tensor spectrum and inverse z (or, for one cell layer and for small meshes, one
+// pass that fuses all of y and z), and a pruned complex-to-real x transform that writes Ms_c H_c per cell.
 //
 // Every kernel is instantiated per log2 transform length (the f3 engine), so the index arithmetic of
 // the FFT stages is resolved at compile time.  The x passes read their input in the first FFT stage
@@ -82,9 +81,6 @@ struct YTile {
 // x passes: radix-16 stages for FP32 lines of 2^10 complex values
 template <typename T, int LG>
 constexpr int kXEpt = (sizeof(T) == 4 && LG >= 10) ? 16 : 8;
-// the single-layer pass keeps up to 1024 threads (FP32) so that long y lines still fit one block
-template <typename T>
-constexpr int kMaxThreadsYC = sizeof(T) == 4 ? 1024 : 512;
 
 // Asynchronous global -> shared copies (cp.async): many in flight per thread without registers.
 __device__ __forceinline__ void cpa16(void *sm, const void *gm)
@@ -487,19 +483,6 @@ template <typename T>
 struct Ten6 {
     T xx, yy, zz, xy, xz, yz;
 };
-template <typename T>
-__device__ __forceinline__ Ten6<T> tensor_at(const Geom &g, const DemagBufs<T> &b, int kx, int a2, int kz)
-{
-    const int h3 = g.P3 >> 1;
-    const int a3 = kz <= h3 ? kz : g.P3 - kz;
-    const T s3 = kz <= h3 ? T(1) : T(-1);
-    const T *n = b.Nk + ((long)a3 * g.H2 + a2) * g.Xp + kx;
-    const long tc = g.t_comp;
-    Ten6<T> t;
-    t.xx = n[0]; t.yy = n[tc]; t.zz = n[2 * tc];
-    t.xy = n[3 * tc]; t.xz = n[4 * tc] * s3; t.yz = n[5 * tc] * s3;
-    return t;
-}
 // H^ = N~ M^ with N~ real symmetric; s2 = -1 on the mirrored frequency P2 - a2 (Nxy and Nyz odd in ky)
 template <typename T>
 __device__ __forceinline__ void tensor_mul(const Ten6<T> &t, T s2, Cx<T> *px, Cx<T> *py, Cx<T> *pz)
@@ -612,252 +595,468 @@ __global__ void __launch_bounds__(kMaxThreads<T>, kMinBlocks<T>) k_z_conv(Geom g
     f3::fft<T, LG, +1, true, true, false, Z::EPT, nl>(buf, nl, nlf, b.tw, g.twlg, P3, g.N3, f3::NoFn<T>(), dst);
 }
 
-// Register z convolution (FP32, P3 = 2^LG <= 64).  The z input is zero above N3 <= P3/2, so with
-// S threads per line (S = 2 or 4) and D = P3/S the spectrum splits into S interleaved parts:
+// Register z convolution.  A thread holds all three components of one (kx, ky) line, or of the part r of it
+// that a split over S threads leaves, so the tensor product needs no exchange.  The z input is zero above
+// N3 <= P3/2; with S threads per line and D = P3/S the spectrum splits into S interleaved parts
 //   X_{Sk+r} = sum_{m<D} e^{-2 pi i mk/D} w^{mr} sum_{j<S/2} w_S^{jr} x_{m+jD},
 // w = e^{-2 pi i/P3}, w_S = w^D, and the inverse kept for z = m + jD < N3 is
 //   y_{m+jD} = sum_r conj(w_S)^{jr} conj(w)^{mr} u_r[m],   u_r = length-D inverse transform of part r.
-// Thread r of a line forms its part and runs the whole length-D transform in registers: no
-// shared-memory exchange between FFT stages.  Shared layout: the tile of z_tile_load; after the forward
-// transform, kz = Sk + r of line l sits in row rD + k; the inverse leaves conj(w)^{mr} u_r[m] in the same
-// rows and the S threads of a line then share the sums over r.
-template <int LG, int S>
+// A warp is one part of 16 kx columns of an octant row a2 (lanes 0-15) and of its mirror P2 - a2 (lanes
+// 16-31), whose tensor reads coincide.
+//
+// Bound by latency and HBM together: four 128-thread blocks per SM at 128 registers (48 or 96 of them the spectrum).
+// The tensor slice is staged with cp.async while the forward transforms run; read straight from L2 inside the
+// product, its latency was exposed at every frequency (1.26 ms at 1024x1024x32).  Against the version that held one
+// component's line per thread and exchanged spectra through shared memory for the product (4x the shared traffic;
+// FP64 and P3 <= 4 had their own): 1.07 -> 1.01 ms at 1024x1024x32 (S = 4), 144 -> 107 us at 512x512x16 (S = 2),
+// 24.7 -> 16.5 us at 256x256x8 and FP64 53 -> 39 us at 128x128x4 (S = 1, no exchange at all).
+template <typename T, int LG>
 struct ZRTile {
-    static constexpr int P3 = 1 << LG, D = P3 / S, G = 16;
-    static constexpr int KY0 = pow2_floor_c(56 * 1024 / (6 * G * P3 * 8));
-    static constexpr int KY = KY0 < 1 ? 1 : (KY0 > 2 ? 2 : KY0);
-    static constexpr int NL = 6 * KY * G;  // lines (a multiple of 32: warps hold one part r)
-    static constexpr int THREADS = S * NL;
-    // the tensor slice goes through shared memory, except for 64-point lines: there the product reads it
-    // from global memory (L2), so that four blocks fit an SM
-    static constexpr bool TSM = LG < 6;
-    static constexpr size_t SMEM =
-        (size_t)NL * P3 * sizeof(Cx<float>) + (TSM ? (size_t)6 * (P3 / 2 + 1) * KY * G * sizeof(float) : 0);
-    static_assert(LG >= 2 && LG <= 6 && (S == 2 || S == 4) && D >= 2 && NL % 32 == 0 && THREADS <= 1024,
-                  "register z tile");
+    static constexpr int P3 = 1 << LG, G = 16, THREADS = 128;
+    static constexpr int DMAX = sizeof(T) == 4 ? 16 : 8;  // values per component that fit the registers
+    static constexpr int S = P3 <= DMAX ? 1 : P3 / DMAX, D = P3 / S;
+    static constexpr int KY = THREADS / 32 / S;  // octant rows per block
+    static constexpr bool STAGE = S == 4;        // inputs staged in shared memory: every part reads all of them
+    static constexpr int NZ = P3 / 2;
+    static constexpr size_t IN_BYTES = STAGE ? (size_t)3 * NZ * KY * 32 * sizeof(Cx<T>) : 0;
+    static constexpr size_t TEN_BYTES = (size_t)6 * (P3 / 2 + 1) * KY * G * sizeof(T);
+    static constexpr size_t EX_BYTES =  // over the inputs and the tensor, once they are consumed
+        S == 1 ? 0 : (size_t)3 * (S == 2 ? D : P3) * KY * 32 * sizeof(Cx<T>);
+    static constexpr size_t SMEM = IN_BYTES + TEN_BYTES > EX_BYTES ? IN_BYTES + TEN_BYTES : EX_BYTES;
+    static_assert(LG >= 2 && (S == 1 || S == 2 || S == 4), "register z tile");
 };
-// threads per line of the register z convolution: 2 (measured on 64-point lines: 1.21 ms against 1.59 ms
-// with 4 threads of 16-point transforms, although those fit twice the resident warps)
-template <int LG>
-constexpr int kZRSplit = 2;
+// longest register z line
+template <typename T>
+constexpr int kZRMaxLg = sizeof(T) == 4 ? 6 : 5;
 
-template <int LG>
-__global__ void __launch_bounds__(ZRTile<LG, kZRSplit<LG>>::THREADS, kZRSplit<LG> == 4 ? 3 : (LG >= 6 ? 4 : 2))
-    k_z_conv_r(Geom g, DemagBufs<float> b)
+// c v for a real c, c v + w
+__device__ __forceinline__ Cx<float> rmul(float c, Cx<float> v)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f3::pack2(cx<float>(c, c))), "l"(f3::pack2(v)));
+    return f3::unpack2(d);
+}
+__device__ __forceinline__ Cx<float> rfma(float c, Cx<float> v, Cx<float> w)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(d)
+        : "l"(f3::pack2(cx<float>(c, c))), "l"(f3::pack2(v)), "l"(f3::pack2(w)));
+    return f3::unpack2(d);
+}
+__device__ __forceinline__ Cx<double> rmul(double c, Cx<double> v) { return cx<double>(c * v.x, c * v.y); }
+__device__ __forceinline__ Cx<double> rfma(double c, Cx<double> v, Cx<double> w)
+{
+    return cx<double>(fma(c, v.x, w.x), fma(c, v.y, w.y));
+}
+
+// H^ = N~ M^ at the frequencies kz = Sk + r held in v[component][bitrev(k)]: N~ at a3 = kz or P3 - kz, xz and
+// yz odd in kz, xy and yz odd in ky (s2 = -1 on the mirrored row); the result is left in natural order, v[c][k].
+// n points at the tensor of (a3 = 0, a2, kx);
+// pl and tc are its strides in a3 and between components.
+template <typename T, int LG, int S>
+__device__ __forceinline__ void z_product(Cx<T> (&v)[3][(1 << LG) / S], const T *n, int pl, int tc, int r, T s2)
+{
+    constexpr int P3 = 1 << LG, D = P3 / S, H = P3 / 2;
+    auto mul = [&](int k, const Ten6<T> &t, T s3) {
+        Cx<T> &x = v[0][f3::bitrev<D>(k)], &y = v[1][f3::bitrev<D>(k)], &z = v[2][f3::bitrev<D>(k)];
+        const T xy = t.xy * s2, yz = t.yz * (s2 * s3), xz = t.xz * s3;
+        const Cx<T> a = rfma(xz, z, rfma(xy, y, rmul(t.xx, x)));
+        const Cx<T> c = rfma(yz, z, rfma(t.yy, y, rmul(xy, x)));
+        z = rfma(t.zz, z, rfma(yz, y, rmul(xz, x)));
+        x = a;
+        y = c;
+    };
+    auto load = [&](const T *p) {
+        Ten6<T> t;
+        t.xx = p[0];
+        t.yy = p[tc];
+        t.zz = p[2 * tc];
+        t.xy = p[3 * tc];
+        t.xz = p[4 * tc];
+        t.yz = p[5 * tc];
+        return t;
+    };
+    if constexpr (S == 1) {
+        // (kz and P3 - kz share a tensor value)
+#pragma unroll
+        for (int k = 0; k <= H; ++k) {
+            const Ten6<T> t = load(n + k * pl);
+            mul(k, t, T(1));
+            if (k > 0 && k < H) mul(P3 - k, t, T(-1));
+        }
+    } else {
+        const T *lo = n + r * pl, *hi = n + (P3 - r) * pl;  // a3 = Sk + r up to H, P3 - r - Sk above
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            // (kz = H itself, k = D/2 of part 0, counts as the lower half)
+            const Ten6<T> t = load(2 * k < D ? lo + S * k * pl : hi - S * k * pl);
+            mul(k, t, 2 * k < D ? T(1) : (2 * k == D && r == 0 ? T(1) : T(-1)));
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            const int j = f3::bitrev<D>(k);
+            if (j > k) {
+                const Cx<T> t = v[c][k];
+                v[c][k] = v[c][j];
+                v[c][j] = t;
+            }
+        }
+}
+
+template <typename T, int LG>
+__global__ void __launch_bounds__(ZRTile<T, LG>::THREADS, 4) k_z_conv_r(Geom g, DemagBufs<T> b)
 {
     pdl_enter();
-    using T = float;
-    constexpr int S = kZRSplit<LG>;
-    using Z = ZRTile<LG, S>;
     if (b.ctl && b.ctl->done) return;
-    constexpr int P3 = Z::P3, D = Z::D, H = P3 / 2, H3 = H + 1, G = Z::G, KY = Z::KY, R2 = 2 * KY, nl = Z::NL;
+    using Z = ZRTile<T, LG>;
+    constexpr int P3 = Z::P3, D = Z::D, S = Z::S, H = P3 / 2, KY = Z::KY, G = Z::G, NZ = Z::NZ;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx<T> *buf = reinterpret_cast<Cx<T> *>(smem_raw);
-    const int kx0 = blockIdx.x * G, a20 = blockIdx.y * KY;
-    z_tile_load<T, G, KY, P3, Z::TSM>(g, b, buf, kx0, a20);
-    const int r = threadIdx.x / nl, l = threadIdx.x - r * nl;
-    const int N3 = g.N3;
-    {
-        // forward: part r of the line's spectrum
-        Cx<T> v[D];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, r = wp % S, rw = wp / S;
+    const int h2 = g.P2 >> 1, N3 = g.N3;
+    const int mir = lane >> 4;
+    int a2 = blockIdx.y * KY + rw;
+    // rows past the octant and mirrors of the rows without one compute on row 0 and write nothing
+    const bool valid = a2 < g.H2 && (!mir || (a2 > 0 && a2 < h2));
+    if (a2 >= g.H2) a2 = 0;
+    const int kx = blockIdx.x * G + (lane & 15);
+    const int ky = valid && mir ? g.P2 - a2 : a2;
+    const int zs = g.P2 * g.Xp;
+    const int line = ky * g.Xp + kx, cstr = N3 * zs;
+    if constexpr (Z::STAGE) {
+        // rows of 32 lanes: element (c, z) of the block's row and mirror; zero above N3
+        const int kx0 = blockIdx.x * G;
+        constexpr int CP = G * (int)sizeof(Cx<T>) / 16;  // 16-byte copies per row of 16 columns
+        static_assert(KY == 1 && (2 * CP) % 16 == 0 && Z::THREADS % (2 * CP) == 0, "staging");
+        const int ch = threadIdx.x % (2 * CP), t0 = threadIdx.x / (2 * CP);
+        const int my = ch < CP ? a2 : ((a2 > 0 && a2 < h2) ? g.P2 - a2 : a2);
+        const char *src = (const char *)(b.S + my * g.Xp + kx0) + (ch % CP) * 16;
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_raw) + ch * 16;
 #pragma unroll
-        for (int m = 0; m < D; ++m) {
-            v[m] = m < N3 ? buf[m * nl + l] : cx<T>(T(0), T(0));
-            if (S == 4) {
-                // x_{m+D} w_S^r, w_S = -i (forward)
-                const Cx<T> x1 = m + D < N3 ? buf[(m + D) * nl + l] : cx<T>(T(0), T(0));
-                const Cx<T> t = r == 0 ? x1 : (r == 1 ? mul_si(x1, -1) : (r == 2 ? cx<T>(-x1.x, -x1.y) : mul_si(x1, 1)));
-                v[m] = f3::csum(v[m], t);
-            }
+        for (int i = 0; i < 3 * NZ * 2 * CP / Z::THREADS; ++i) {
+            const int t = t0 + i * (Z::THREADS / (2 * CP)), c = t / NZ, z = t % NZ;
+            const int n = z < N3 ? 16 : 0;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst + t * (unsigned)(32 * sizeof(Cx<T>))),
+                         "l"(src + (z < N3 ? (size_t)(c * cstr + z * zs) * sizeof(Cx<T>) : 0)), "r"(n)
+                         : "memory");
         }
-        __syncthreads();  // every part has read the input rows before any overwrites them
-        if (r > 0) {
-#pragma unroll
-            for (int m = 1; m < D; ++m) {
-                // w^{mr}: r is warp-uniform, the twiddle a compile-time constant per branch
-                if (r == 1) v[m] = f3::rot<T, P3, -1>(v[m], m);
-                else if (S == 4 && r == 2) v[m] = f3::rot<T, P3, -1>(v[m], 2 * m);
-                else if (S == 4 && r == 3) v[m] = f3::rot<T, P3, -1>(v[m], 3 * m);
-            }
-        }
-        f3::dft_reg<T, D, -1>(v);
-#pragma unroll
-        for (int k = 0; k < D; ++k) buf[(r * D + k) * nl + l] = v[f3::bitrev<D>(k)];
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
-    __syncthreads();
+    // the tensor slice [component][a3][row][kx] arrives while the forward transforms run
+    T *ten = reinterpret_cast<T *>(smem_raw + Z::IN_BYTES);
     {
-        // H^ = N~ M^ at every (kz, row, kx) of the tile; row q holds kz = S (q mod D) + q / D
-        const T *ten = reinterpret_cast<const T *>(buf + nl * P3);
-        constexpr int tstride = H3 * KY * G, npts = KY * G * P3;
-        const int h2 = g.P2 >> 1;
-        if constexpr (!Z::TSM) {
-            // the tensor comes from L2: all of a thread's tensor reads are issued before the products
-            constexpr int NPT = (npts + Z::THREADS - 1) / Z::THREADS;
-            Ten6<T> tv[NPT];
+        constexpr int CP = G * (int)sizeof(T) / 16, RT = Z::THREADS / CP, ROWS = 6 * (H + 1) * KY;
+        const int ch = threadIdx.x % CP, t0 = threadIdx.x / CP;
+        const T *src = b.Nk + blockIdx.x * G + ch * (16 / (int)sizeof(T));
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(ten) + ch * 16;
 #pragma unroll
-            for (int u = 0; u < NPT; ++u) {
-                const int t = threadIdx.x + u * Z::THREADS;
-                const int gg = t % G, qr = t / G, rr = qr % KY, q = qr / KY;
-                const int a2 = a20 + rr;
-                if (t >= npts || a2 >= g.H2) continue;
-                const int kz = S * (q % D) + q / D;
-                const int a3 = kz <= H ? kz : P3 - kz;
-                const T *tp = b.Nk + ((long)a3 * g.H2 + a2) * g.Xp + kx0 + gg;
-                const long tc = g.t_comp;
-                tv[u].xx = __ldg(tp);
-                tv[u].yy = __ldg(tp + tc);
-                tv[u].zz = __ldg(tp + 2 * tc);
-                tv[u].xy = __ldg(tp + 3 * tc);
-                tv[u].xz = __ldg(tp + 4 * tc);
-                tv[u].yz = __ldg(tp + 5 * tc);
-            }
-#pragma unroll
-            for (int u = 0; u < NPT; ++u) {
-                const int t = threadIdx.x + u * Z::THREADS;
-                const int gg = t % G, qr = t / G, rr = qr % KY, q = qr / KY;
-                const int a2 = a20 + rr;
-                if (t >= npts || a2 >= g.H2) continue;
-                const int kz = S * (q % D) + q / D;
-                const T s3 = kz <= H ? T(1) : T(-1);
-                Ten6<T> tt = tv[u];
-                tt.xz *= s3;
-                tt.yz *= s3;
-                Cx<T> *p = buf + q * nl + rr * G + gg;
-                tensor_mul(tt, T(1), p, p + R2 * G, p + 2 * R2 * G);
-                if (a2 > 0 && a2 < h2) {
-                    Cx<T> *pm = p + KY * G;
-                    tensor_mul(tt, T(-1), pm, pm + R2 * G, pm + 2 * R2 * G);
-                }
-            }
+        for (int i = 0; i < (ROWS + RT - 1) / RT; ++i) {
+            const int t = t0 + i * RT, rr = t % KY, q = t / KY, a3 = q % (H + 1), c = q / (H + 1);
+            const int aa = blockIdx.y * KY + rr;
+            if (t < ROWS)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + t * (unsigned)(G * sizeof(T))),
+                             "l"(src + c * (int)g.t_comp + (a3 * g.H2 + (aa < g.H2 ? aa : 0)) * g.Xp)
+                             : "memory");
         }
-#pragma unroll 2
-        for (int t = threadIdx.x; Z::TSM && t < npts; t += Z::THREADS) {
-            const int gg = t % G, qr = t / G, rr = qr % KY, q = qr / KY;
-            const int a2 = a20 + rr;
-            if (a2 >= g.H2) continue;
-            const int kz = S * (q % D) + q / D;
-            const int a3 = kz <= H ? kz : P3 - kz;
-            const T s3 = kz <= H ? T(1) : T(-1);
-            Ten6<T> tt;
-            if (Z::TSM) {
-                const T *tp = ten + (a3 * KY + rr) * G + gg;
-                tt.xx = tp[0];
-                tt.yy = tp[tstride];
-                tt.zz = tp[2 * tstride];
-                tt.xy = tp[3 * tstride];
-                tt.xz = tp[4 * tstride] * s3;
-                tt.yz = tp[5 * tstride] * s3;
-            } else {
-                const T *tp = b.Nk + ((long)a3 * g.H2 + a2) * g.Xp + kx0 + gg;
-                const long tc = g.t_comp;
-                tt.xx = __ldg(tp);
-                tt.yy = __ldg(tp + tc);
-                tt.zz = __ldg(tp + 2 * tc);
-                tt.xy = __ldg(tp + 3 * tc);
-                tt.xz = __ldg(tp + 4 * tc) * s3;
-                tt.yz = __ldg(tp + 5 * tc) * s3;
-            }
-            Cx<T> *p = buf + q * nl + rr * G + gg;
-            tensor_mul(tt, T(1), p, p + R2 * G, p + 2 * R2 * G);
-            if (a2 > 0 && a2 < h2) {
-                Cx<T> *pm = p + KY * G;
-                tensor_mul(tt, T(-1), pm, pm + R2 * G, pm + 2 * R2 * G);
-            }
-        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
-    __syncthreads();
-    {
-        // inverse of part r, twisted by conj(w)^{mr}, back into the part's own (consumed) rows
-        Cx<T> v[D];
-#pragma unroll
-        for (int k = 0; k < D; ++k) v[k] = buf[(r * D + k) * nl + l];
-        f3::dft_reg<T, D, +1>(v);
-#pragma unroll
-        for (int m = 0; m < D; ++m) {
-            Cx<T> u = v[f3::bitrev<D>(m)];
-            if (r == 1) u = f3::rot<T, P3, +1>(u, m);
-            else if (S == 4 && r == 2) u = f3::rot<T, P3, +1>(u, 2 * m);
-            else if (S == 4 && r == 3) u = f3::rot<T, P3, +1>(u, 3 * m);
-            buf[(r * D + m) * nl + l] = u;
-        }
+    if constexpr (Z::STAGE) {
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
         __syncthreads();
-        // z = r H/S + i, i < H/S (outputs z < H, shared by the S threads): z = m + jD
-        const int gg = l % G, q = l / G, rw = q % R2, c = q / R2;
-        const int ky = z_row_ky<KY>(g, a20, rw);
-        if (ky >= 0) {
-            Cx<T> *out = b.S + c * g.s_comp + (long)ky * g.Xp + kx0 + gg;
-            const long zs = (long)g.P2 * g.Xp;
-            constexpr int ZP = H / S;  // outputs per thread
+    }
+    Cx<T> v[3][D];
 #pragma unroll
-            for (int i = 0; i < ZP; ++i) {
-                const int z = r * ZP + i;
-                if (z >= N3) break;
-                const int m = z % D, j = z / D;  // j < S/2
-                Cx<T> y = buf[m * nl + l];
+    for (int c = 0; c < 3; ++c) {
+        const Cx<T> *in = b.S + line + c * cstr;
 #pragma unroll
-                for (int rr = 1; rr < S; ++rr) {
-                    const Cx<T> t = buf[(rr * D + m) * nl + l];
-                    // conj(w_S)^{j rr}: (+i)^{j rr} for S = 4, (-1)^{j rr} for S = 2 (j = 0 there)
-                    const int e = (j * rr) & (S - 1);
-                    const Cx<T> tt = S == 2 ? t : (e == 0 ? t : (e == 1 ? mul_si(t, 1) : (e == 2 ? cx<T>(-t.x, -t.y) : mul_si(t, -1))));
-                    y = f3::csum(y, tt);
+        for (int m = 0; m < D; ++m) {
+            if constexpr (Z::STAGE) {
+                const Cx<T> x0 = buf[(c * NZ + m) * 32 + lane], x1 = buf[(c * NZ + m + D) * 32 + lane];
+                // x_m + w_4^r x_{m+D}, w_4 = -i
+                const T p = r & 1 ? x1.y : x1.x, q = r & 1 ? x1.x : x1.y;
+                const T sp = r == 2 || r == 3 ? T(-1) : T(1), sq = r == 1 || r == 2 ? T(-1) : T(1);
+                v[c][m] = cx<T>(fma(sp, p, x0.x), fma(sq, q, x0.y));
+            } else {
+                v[c][m] = m < H && m < N3 ? in[m * zs] : cx<T>(T(0), T(0));
+            }
+        }
+    }
+    // twist by w^{mr}: r is the same for a whole warp, so the powers are constants of each branch
+    auto twist = [&](auto dir) {
+        constexpr int DIR = decltype(dir)::value;
+#pragma unroll
+        for (int rr = 1; rr < S; ++rr) {
+            if (r != rr) continue;
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int m = 1; m < D; ++m) {
+                    const int i = DIR < 0 ? m : f3::bitrev<D>(m);
+                    v[c][i] = f3::rot<T, P3, DIR>(v[c][i], m * rr);
                 }
-                out[z * zs] = y;
+        }
+    };
+    if constexpr (S > 1) twist(std::integral_constant<int, -1>{});
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f3::dft_reg<T, D, -1>(v[c]);
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    z_product<T, LG, S>(v, ten + rw * G + (lane & 15), KY * G, (H + 1) * KY * G, r, mir ? T(-1) : T(1));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f3::dft_reg<T, D, +1>(v[c]);
+    if constexpr (S > 1) twist(std::integral_constant<int, +1>{});
+    if constexpr (S == 1) {
+        if (!valid) return;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            Cx<T> *out = b.S + line + c * cstr;
+#pragma unroll
+            for (int m = 0; m < NZ; ++m)
+                if (m < N3) out[m * zs] = v[c][f3::bitrev<D>(m)];
+        }
+    } else if constexpr (S == 2) {
+        // part 0 writes z < D/2, part 1 the others: each sends the half that it does not write
+        constexpr int F = D / 2;
+        Cx<T> *ex = buf + (rw * 2) * (3 * F * 32) + lane;
+        __syncthreads();  // the tensor has been read
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int i = 0; i < F; ++i) {
+                const Cx<T> u0 = v[c][f3::bitrev<D>(i)], u1 = v[c][f3::bitrev<D>(i + F)];
+                ex[(r * 3 + c) * F * 32 + i * 32] = r == 0 ? u1 : u0;
+            }
+        __syncthreads();
+        if (!valid) return;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            Cx<T> *out = b.S + line + c * cstr;
+#pragma unroll
+            for (int i = 0; i < F; ++i) {
+                const Cx<T> u0 = v[c][f3::bitrev<D>(i)], u1 = v[c][f3::bitrev<D>(i + F)];
+                const Cx<T> own = r == 0 ? u0 : u1;
+                const int z = i + r * F;
+                if (z < N3) out[z * zs] = f3::csum(own, ex[((r ^ 1) * 3 + c) * F * 32 + i * 32]);
+            }
+        }
+    } else {
+        // thread r writes z = m and m + D for its quarter of the m: the four parts meet in shared memory
+        constexpr int F = D / 4;
+        __syncthreads();  // every part has read the staged inputs and the tensor
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int m = 0; m < D; ++m) buf[((c * 4 + r) * D + m) * 32 + lane] = v[c][f3::bitrev<D>(m)];
+        __syncthreads();
+        if (!valid) return;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            Cx<T> *out = b.S + line + c * cstr;
+#pragma unroll
+            for (int i = 0; i < F; ++i) {
+                const int m = r * F + i;
+                const Cx<T> *p = buf + (c * 4 * D + m) * 32 + lane;
+                const Cx<T> t0 = p[0], t1 = p[D * 32], t2 = p[2 * D * 32], t3 = p[3 * D * 32];
+                // j = 0: plain sum; j = 1: conj(w_4)^r = (i)^r
+                if (m < N3) out[m * zs] = f3::csum(f3::csum(t0, t2), f3::csum(t1, t3));
+                if (m + D < N3) out[(m + D) * zs] = f3::csum(f3::cdiff(t0, t2), mul_si(f3::cdiff(t1, t3), 1));
             }
         }
     }
 }
 
-// Single-layer variant (N3 == 1, P3 == 1): forward y, tensor product at kz = 0 (each octant row a2
-// read once and applied to ky = a2 and P2 - a2), inverse y.  Lines l = c * G + g; element y of line l
-// at buf[y * nl + l].  LG = 0 (N2 == 1): the product alone.
-template <typename T, int LG>
-__global__ void __launch_bounds__(kMaxThreadsYC<T>, 1) k_y_conv(Geom g, DemagBufs<T> b, int G)
+// Fused y-z convolution (FP32 P3 <= 16, FP64 P3 <= 8): one block holds all N3 planes of the three components of
+// G kx columns, P2 rows each, in shared memory and runs forward y, z convolution and inverse y on them, so
+// the spectrum padded along y never reaches global memory and three launches become one.
+//
+// One block of 512 threads (FP64: 256) works through its phases in turn, so their latencies bound it.  Against the
+// passes it replaces (for one layer a fused y pass that held a line's stage in registers, one column per block at
+// this length): 86 against 126 us at 1024x1024x1, 25 / 31 at 512x512x1, FP64 19 / 53 at 64x64x1 and 46 / 63 (three
+// launches) at 64x64x4.  (Events around each launch, about 5 us of each figure the gap between them.)
+//
+// The y transforms are in place: decimation in frequency forward (the frequencies end in digit-reversed
+// rows), decimation in time inverse (from digit-reversed rows back to natural ones), one barrier per stage
+// and any number of butterflies per thread.  The first stage reads the N2 input rows from global memory, the
+// last one writes the N2 output rows there.  In between a thread takes the three z lines of a (row, kx) into
+// registers for the z transforms and the product.
+// Row y at buf + y * nlp, line l = (c N3 + z) G + g within it; nlp = G x an odd number, so that the G columns
+// of consecutive rows fall into different banks.
+template <typename T>
+constexpr int kYZThreads = sizeof(T) == 4 ? 512 : 256;
+template <typename T>
+constexpr int kYZMaxLg3 = sizeof(T) == 4 ? 4 : 3;
+
+// One radix-2^LR stage over sub-transforms of 2^lgM rows (of 2^lgP rows in all) of nl lines.
+template <typename T, int LR, int DIR, typename Ld, typename St>
+__device__ __forceinline__ void yz_stage(int lgP, int lgM, int nl, const FastDiv &nlf, const Cx<T> *__restrict__ tw,
+                                         int twlg, const Ld &ld, const St &st)
+{
+    constexpr int R = 1 << LR;
+    const int lgq = lgM - LR, nb = nl << (lgP - LR), sh = twlg - lgM;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+        const int q = (int)nlf.div((unsigned)b), l = b - q * nl;
+        const int j = q & ((1 << lgq) - 1), row = ((q >> lgq) << lgM) + j;
+        Cx<T> v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = ld(l, row + (r << lgq));
+        Cx<T> w[R];
+        if (lgq > 0) {
+            const int jj = j << sh;
+            if constexpr (R == 16) {
+                // (powers from four table values: see f3::stage)
+                w[1] = tw[jj];
+                w[2] = tw[2 * jj];
+                w[4] = tw[4 * jj];
+                w[8] = tw[8 * jj];
+                w[3] = w[1] * w[2];
+                w[5] = w[4] * w[1];
+                w[6] = w[4] * w[2];
+                w[7] = w[4] * w[3];
+#pragma unroll
+                for (int r = 9; r < 16; ++r) w[r] = w[8] * w[r - 8];
+            } else {
+#pragma unroll
+                for (int r = 1; r < R; ++r) w[r] = tw[jj * r];
+            }
+        }
+        if (DIR > 0 && lgq > 0) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = f3::twmul<T, DIR>(v[r], w[r]);
+        }
+        f3::dft<T, R, DIR>(v);
+        if (DIR < 0 && lgq > 0) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[f3::bitrev<R>(r)] = f3::twmul<T, DIR>(v[f3::bitrev<R>(r)], w[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) st(l, row + (r << lgq), v[f3::bitrev<R>(r)]);
+    }
+}
+template <typename T, int DIR, typename Ld, typename St>
+__device__ __forceinline__ void yz_stage_any(int lr, int lgP, int lgM, int nl, const FastDiv &nlf,
+                                             const Cx<T> *__restrict__ tw, int twlg, const Ld &ld, const St &st)
+{
+    if (lr == 1) yz_stage<T, 1, DIR>(lgP, lgM, nl, nlf, tw, twlg, ld, st);
+    else if (lr == 2) yz_stage<T, 2, DIR>(lgP, lgM, nl, nlf, tw, twlg, ld, st);
+    else if (lr == 3) yz_stage<T, 3, DIR>(lgP, lgM, nl, nlf, tw, twlg, ld, st);
+    else if constexpr (sizeof(T) == 4) yz_stage<T, 4, DIR>(lgP, lgM, nl, nlf, tw, twlg, ld, st);
+}
+
+// plan: log2 radices of the forward stages, four bits each, first stage lowest
+template <typename T, int LG3>
+__global__ void __launch_bounds__(kYZThreads<T>, 1) k_yz_conv(Geom g, DemagBufs<T> b, int lgG, int nlp, FastDiv nlf, unsigned plan)
 {
     pdl_enter();
     if (b.ctl && b.ctl->done) return;
-    constexpr int P2 = 1 << LG;
+    constexpr int P3 = 1 << LG3, NZ = P3 > 1 ? P3 / 2 : 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx<T> *buf = reinterpret_cast<Cx<T> *>(smem_raw);
-    const int kx0 = blockIdx.x * G;
-    const int nl = 3 * G;
-    const int h2 = P2 >> 1;
-    auto gaddr = [&](int c, int y) -> long { return c * g.s_comp + (long)y * g.Xp + kx0; };
-    {
-        const int rowb = G * (int)sizeof(Cx<T>);
-        const int cb = rowb >= 16 ? 16 : rowb, lcpr = __ffs(rowb / cb) - 1;
-        const int nrow = g.N2 * 3;
-        for (int t = threadIdx.x; t < (nrow << lcpr); t += blockDim.x) {
-            const int rr = t >> lcpr, ch = t - (rr << lcpr);
-            const int y = rr / 3, c = rr - 3 * y;
-            cpa_chunk((char *)(buf + y * nl + c * G) + ch * cb, (const char *)(b.S + gaddr(c, y)) + ch * cb, cb);
-        }
-        cpa_wait_all();
+    const int G = 1 << lgG, N3 = g.N3, N2 = g.N2, lgP = g.lgP2, zs = g.P2 * g.Xp, Xp = g.Xp;
+    const int nl = 3 * N3 * G;
+    Cx<T> *S = b.S + (blockIdx.x << lgG);
+    auto gl = [&](int l, int y) { return (l >> lgG) * zs + (l & (G - 1)) + y * Xp; };
+    auto sld = [&](int l, int y) { return buf[y * nlp + l]; };
+    auto sst = [&](int l, int y, Cx<T> v) { buf[y * nlp + l] = v; };
+    auto gld = [&](int l, int y) { return y < N2 ? S[gl(l, y)] : cx<T>(T(0), T(0)); };
+    auto gst = [&](int l, int y, Cx<T> v) {
+        if (y < N2) S[gl(l, y)] = v;
+    };
+    if (lgP == 0) {
+        for (int l = threadIdx.x; l < nl; l += blockDim.x) sst(l, 0, gld(l, 0));
         __syncthreads();
     }
-    const FastDiv nlf((unsigned)nl);
-    if constexpr (LG > 0)
-        f3::fft<T, LG, -1, true, true, true>(buf, nl, nlf, b.tw, g.twlg, g.N2, P2, f3::NoFn<T>(), f3::NoFn<T>());
-    const int lG = __ffs(G) - 1;
-    for (int t = threadIdx.x; t < G * g.H2; t += blockDim.x) {
-        const int gg = t & (G - 1), a2 = t >> lG;
-        const Ten6<T> ten = tensor_at(g, b, kx0 + gg, a2, 0);
-        Cx<T> *p = buf + a2 * nl + gg;
-        tensor_mul(ten, T(1), p, p + G, p + 2 * G);
-        if (a2 > 0 && a2 < h2) {
-            Cx<T> *pm = buf + (P2 - a2) * nl + gg;
-            tensor_mul(ten, T(-1), pm, pm + G, pm + 2 * G);
+    {
+        int lgM = lgP;
+        for (unsigned p = plan; p; p >>= 4) {
+            const int lr = p & 15;
+            if (lgM == lgP) yz_stage_any<T, -1>(lr, lgP, lgM, nl, nlf, b.tw, g.twlg, gld, sst);
+            else yz_stage_any<T, -1>(lr, lgP, lgM, nl, nlf, b.tw, g.twlg, sld, sst);
+            lgM -= lr;
+            __syncthreads();
+        }
+    }
+    auto freq = [&](int row) {
+        int ky = 0, sh = 0, rem = lgP;
+        for (unsigned p = plan; p; p >>= 4) {
+            const int lr = p & 15;
+            rem -= lr;
+            ky |= ((row >> rem) & ((1 << lr) - 1)) << sh;
+            sh += lr;
+        }
+        return ky;
+    };
+    const T *nk = b.Nk + (int)(blockIdx.x << lgG);
+    const int tc = (int)g.t_comp, h2 = g.P2 >> 1;
+    if constexpr (P3 == 1) {
+        // one layer: the product alone, the tensor values of NB points in flight together
+        constexpr int NB = 4;
+        const int ni = G << lgP;
+        for (int i0 = threadIdx.x; i0 < ni; i0 += NB * blockDim.x) {
+            Ten6<T> t[NB];
+            T s2[NB];
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                const int i = i0 + u * blockDim.x;
+                if (i >= ni) break;
+                const int ky = freq(i >> lgG), a2 = ky > h2 ? g.P2 - ky : ky;
+                const T *q = nk + a2 * Xp + (i & (G - 1));
+                s2[u] = ky > h2 ? T(-1) : T(1);
+                t[u] = Ten6<T>{q[0], q[tc], q[2 * tc], q[3 * tc], q[4 * tc], q[5 * tc]};
+            }
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                const int i = i0 + u * blockDim.x;
+                if (i >= ni) break;
+                Cx<T> *p = buf + (i >> lgG) * nlp + (i & (G - 1));
+                tensor_mul(t[u], s2[u], p, p + G, p + 2 * G);
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < (G << lgP); i += blockDim.x) {
+            const int gg = i & (G - 1), row = i >> lgG, ky = freq(row);
+            const bool mir = ky > h2;
+            const int a2 = mir ? g.P2 - ky : ky;
+            Cx<T> *p = buf + row * nlp + gg;
+            Cx<T> v[3][P3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int m = 0; m < P3; ++m) v[c][m] = m < NZ && m < N3 ? p[(c * N3 + m) << lgG] : cx<T>(T(0), T(0));
+#pragma unroll
+            for (int c = 0; c < 3; ++c) f3::dft_reg<T, P3, -1>(v[c]);
+            z_product<T, LG3, 1>(v, nk + a2 * Xp + gg, g.H2 * Xp, tc, 0, mir ? T(-1) : T(1));
+#pragma unroll
+            for (int c = 0; c < 3; ++c) f3::dft_reg<T, P3, +1>(v[c]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int m = 0; m < NZ; ++m)
+                    if (m < N3) p[(c * N3 + m) << lgG] = v[c][f3::bitrev<P3>(m)];
         }
     }
     __syncthreads();
-    auto dst = [&](int l, int y, Cx<T> v) {
-        const int gg = l & (G - 1), c = l >> lG;
-        b.S[gaddr(c, y) + gg] = v;
-    };
-    if constexpr (LG > 0) {
-        f3::fft<T, LG, +1, true, true, false>(buf, nl, nlf, b.tw, g.twlg, P2, g.N2, f3::NoFn<T>(), dst);
-    } else {
-        for (int l = threadIdx.x; l < nl; l += blockDim.x) dst(l, 0, buf[l]);
+    if (lgP == 0) {
+        for (int l = threadIdx.x; l < nl; l += blockDim.x) gst(l, 0, sld(l, 0));
+        return;
+    }
+    {
+        // the stages in reverse order
+        int lgM = 0, ns = 0;
+        for (unsigned p = plan; p; p >>= 4) ++ns;
+        for (int s = ns - 1; s >= 0; --s) {
+            const int lr = (plan >> (4 * s)) & 15;
+            lgM += lr;
+            if (s > 0) {
+                yz_stage_any<T, +1>(lr, lgP, lgM, nl, nlf, b.tw, g.twlg, sld, sst);
+                __syncthreads();
+            } else {
+                yz_stage_any<T, +1>(lr, lgP, lgM, nl, nlf, b.tw, g.twlg, sld, gst);
+            }
+        }
     }
 }
 
@@ -883,28 +1082,37 @@ static void init_attributes_t()
         constexpr int LG = decltype(c)::value;
         set_smem((const void *)k_z_conv<T, LG>);
     });
-    if constexpr (sizeof(T) == 4) {
-        f3::lg_for_each<2, 6>([&](auto c) { set_smem((const void *)k_z_conv_r<decltype(c)::value>); });
+    f3::lg_for_each<2, kZRMaxLg<T>>([&](auto c) { set_smem((const void *)k_z_conv_r<T, decltype(c)::value>); });
+    f3::lg_for_each<0, kYZMaxLg3<T>>([&](auto c) { set_smem((const void *)k_yz_conv<T, decltype(c)::value>); });
+}
+
+
+// Tile of the fused y-z convolution.  Single-layer meshes always take it.  Meshes of several layers take it where
+// a column's tile is so small that the three launches it replaces cost more than its serial phases (FP32 steps,
+// fused against separate: 16x16x4 131 against 142 us, 64x32x4 143 / 150, 64x64x2 148 / 154, but 128x64x4 168 / 168
+// and 128x128x8 254 / 231; FP64: 64x64x4 611 / 657, 128x128x4 1253 / 1332).  G is the widest tile that leaves at
+// least 128 blocks: wider rows move whole sectors, narrower ones fill the GPU (FP32 steps with G = 1, 2, 4: 64x64x1
+// 142, 142, 146 us; 200x50x1 164, 144, 146; 512x512x1 536, 427, 357; 1024x1024x1 1491, 1289, 1122).
+template <typename T>
+static void plan_yz(const Geom &g, DemagPlan &p)
+{
+    constexpr long kMaxTile = sizeof(T) == 4 ? 768 : 4096;  // values of one column, several layers
+    p.yz = g.lgP3 <= kYZMaxLg3<T> && g.lgP2 <= 11 && (g.N3 == 1 || 3L * g.N3 * g.P2 <= kMaxTile);
+    if (!p.yz) return;
+    int lgG = sizeof(T) == 4 ? 2 : 1;
+    auto bytes = [&](int lg) { return ((size_t)((3L * g.N3) | 1) << lg) * g.P2 * sizeof(Cx<T>); };
+    while (lgG > 0 && (div_up(g.X, 1 << lgG) < 128 || bytes(lgG) > 200 * 1024)) --lgG;
+    p.yz_lgG = lgG;
+    p.yz_nlp = ((3 * g.N3) | 1) << lgG;
+    p.yz_smem = bytes(lgG);
+    // as few stages as radix 8 (FP64 and short lines) or 16 allows, split evenly, the larger radices first
+    const int RM = sizeof(T) == 4 && g.lgP2 > 7 ? 4 : 3;
+    p.yz_plan = 0;
+    for (int left = g.lgP2, s = 0, ns = div_up(left, RM); left > 0; ++s, --ns) {
+        const int lr = div_up(left, ns);
+        p.yz_plan |= (unsigned)lr << (4 * s);
+        left -= lr;
     }
-    f3::lg_for_each<0, 11>([&](auto c) {
-        constexpr int LG = decltype(c)::value;
-        set_smem((const void *)k_y_conv<T, LG>);
-    });
-}
-
-
-static int pow2_floor(long v)
-{
-    if (v < 1) return 0;
-    int p = 1;
-    while (2L * p <= v) p *= 2;
-    return p;
-}
-static int threads_for(long elems)
-{
-    long t = (elems + 7) / 8;
-    t = t < 32 ? 32 : t;
-    return (int)((t + 31) / 32 * 32);
 }
 
 // Launch shapes: every block transforms at most 8 complex values per thread; the y and z passes take
@@ -957,25 +1165,18 @@ DemagPlan demag_plan(const Geom &g)
             p.z_threads = Z::THREADS;
             p.z_smem = Z::SMEM;
         });
-        // FP32 lines of up to 64: the register z convolution
-        p.z_reg = sizeof(T) == 4 && g.lgP3 >= 2 && g.lgP3 <= 6 && 2 * g.N3 <= g.P3;
+        p.z_reg = g.lgP3 >= 2 && g.lgP3 <= kZRMaxLg<T> && 2 * g.N3 <= g.P3;
         if (p.z_reg) {
-            f3::lg_dispatch<2, 6>(g.lgP3, [&](auto c) {
-                using Z = ZRTile<decltype(c)::value, kZRSplit<decltype(c)::value>>;
+            f3::lg_dispatch<2, kZRMaxLg<T>>(g.lgP3, [&](auto c) {
+                using Z = ZRTile<T, decltype(c)::value>;
                 p.z_G = Z::G;
                 p.z_KY = Z::KY;
                 p.z_threads = Z::THREADS;
                 p.z_smem = Z::SMEM;
             });
         }
-    } else {
-        int G = pow2_floor(8L * kMaxThreadsYC<T> / (3L * g.P2));
-        G = G > 16 ? 16 : G;
-        if (G < 1 || g.lgP2 > 11) p.ok = false;
-        p.yc_G = G < 1 ? 1 : G;
-        p.yc_threads = threads_for(3L * p.yc_G * g.P2);
-        p.yc_smem = (size_t)3 * p.yc_G * g.P2 * cs;
     }
+    plan_yz<T>(g, p);
     // every block holds at most (values per thread) x (threads) values of its transforms
     if (g.P1 > 1) {
         const long xept = (sizeof(T) == 4 && g.lgQ >= 10) ? 16 : 8;
@@ -985,14 +1186,14 @@ DemagPlan demag_plan(const Geom &g)
         if (p.y_threads > kMaxThreads<T> * ((sizeof(T) == 4 && g.lgP2 >= 11) ? 2 : 1) ||
             p.z_threads > (p.z_reg ? 1024 : kMaxThreads<T>))
             p.ok = false;
-    } else if (3L * p.yc_G * g.P2 > 8L * p.yc_threads || p.yc_threads > kMaxThreadsYC<T>) {
+    } else if (!p.yz) {
         p.ok = false;
     }
     // the kx grouping divides Xp (a multiple of 16)
-    const int Gmax = g.N3 > 1 ? (p.y_G > p.z_G ? p.y_G : p.z_G) : p.yc_G;
+    const int Gmax = g.N3 > 1 ? (p.y_G > p.z_G ? p.y_G : p.z_G) : 1 << p.yz_lgG;
     if (g.Xp % Gmax != 0) p.ok = false;
     if (p.x_smem > 200 * 1024 || p.xi_smem > 200 * 1024 || p.y_smem > 200 * 1024 || p.yi_smem > 200 * 1024 ||
-        p.z_smem > 200 * 1024 || p.yc_smem > 200 * 1024)
+        p.z_smem > 200 * 1024 || (p.yz && p.yz_smem > 200 * 1024))
         p.ok = false;
     return p;
 }
@@ -1069,7 +1270,14 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
         });
     }
     b.mark("demag_x_fwd");
-    if (g.N3 > 1) {
+    if (p.yz) {
+        f3::lg_dispatch<0, kYZMaxLg3<T>>(g.lgP3, [&](auto c) {
+            constexpr int LG3 = decltype(c)::value;
+            launch_pdl(k_yz_conv<T, LG3>, div_up(g.X, 1 << p.yz_lgG), kYZThreads<T>, p.yz_smem, st, g, b, p.yz_lgG,
+                       p.yz_nlp, FastDiv((unsigned)((3 * g.N3) << p.yz_lgG)), p.yz_plan);
+        });
+        b.mark("demag_yz_conv");
+    } else {
         if (g.P2 > 1) {
             f3::lg_dispatch<1, 11>(g.lgP2, [&](auto c) {
                 constexpr int LG = decltype(c)::value;
@@ -1077,13 +1285,11 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
             });
             b.mark("demag_y_fwd");
         }
-        if constexpr (sizeof(T) == 4) {
-            if (p.z_reg) {
-                f3::lg_dispatch<2, 6>(g.lgP3, [&](auto c) {
-                    constexpr int LG = decltype(c)::value;
-                    launch_pdl(k_z_conv_r<LG>, dim3(g.Xp / p.z_G, div_up(g.H2, p.z_KY)), p.z_threads, p.z_smem, st, g, b);
-                });
-            }
+        if (p.z_reg) {
+            f3::lg_dispatch<2, kZRMaxLg<T>>(g.lgP3, [&](auto c) {
+                constexpr int LG = decltype(c)::value;
+                launch_pdl(k_z_conv_r<T, LG>, dim3(g.Xp / p.z_G, div_up(g.H2, p.z_KY)), p.z_threads, p.z_smem, st, g, b);
+            });
         }
         if (!p.z_reg) {
             f3::lg_dispatch<1, 7>(g.lgP3, [&](auto c) {
@@ -1099,12 +1305,6 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
             });
             b.mark("demag_y_inv");
         }
-    } else {
-        f3::lg_dispatch<0, 11>(g.lgP2, [&](auto c) {
-            constexpr int LG = decltype(c)::value;
-            launch_pdl(k_y_conv<T, LG>, g.Xp / p.yc_G, p.yc_threads, p.yc_smem, st, g, b, p.yc_G);
-        });
-        b.mark("demag_y_conv");
     }
     if (g.P1 == 1) {
         launch_pdl(k_x_inv1<T, CELL>, div_up(nlines, 256), 256, 0, st, g, b, out);
