@@ -863,6 +863,10 @@ template <typename T>
 void launch_heff(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaStream_t st)
 {
     if (p.g.basis == 2) {
+        if (p.uniform) {
+            launch_heff_uniform<T>(p, y, h_out, t, st);
+            return;
+        }
         launch_pdl(k_node2d<T, false>, dim3(div_up(p.g.nn1, 32), div_up(p.g.nn2, 8)), 256, 0, st, p, y, h_out, nullptr,
                                                                                           StageArgs{}, t);
         return;
@@ -890,6 +894,10 @@ template <typename T>
 void launch_llg_stage(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa, cudaStream_t st)
 {
     if (p.g.basis == 2) {
+        if (p.uniform) {
+            launch_llg_stage_uniform<T>(p, y, k_out, y_next, sa, st);
+            return;
+        }
         launch_pdl(k_node2d<T, true>, dim3(div_up(p.g.nn1, 32), div_up(p.g.nn2, 8)), 256, 0, st, p, y, k_out, y_next, sa,
                                                                                          0.0);
         return;

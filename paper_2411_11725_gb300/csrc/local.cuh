@@ -70,7 +70,7 @@ template <typename T>
 void launch_llg_stage(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa,
                       cudaStream_t st);
 
-// the same for a uniform material (p.uniform) on the trilinear basis; DMI reads the raw field p.hdmi
+// the same for a uniform material (p.uniform) on the trilinear or 2D basis; DMI reads the raw field p.hdmi
 template <typename T>
 void launch_heff_uniform(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaStream_t st);
 template <typename T>

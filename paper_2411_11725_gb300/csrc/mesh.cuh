@@ -219,7 +219,7 @@ inline LocalParams<T> local_params(nm_mesh M, unsigned terms)
     p.hu_freq = M->hu_freq; p.hu_phase = M->hu_phase;
     p.hc_freq = M->hc_freq; p.hc_phase = M->hc_phase;
     p.terms = terms;
-    p.uniform = (M->g.basis == 3 && !M->Ms_d && !M->A_d && !M->Ku_d && M->Ms0 > 0.0) ? 1 : 0;
+    p.uniform = (M->g.basis >= 2 && !M->Ms_d && !M->A_d && !M->Ku_d && M->Ms0 > 0.0) ? 1 : 0;
     if (p.uniform) {
         const double A = (terms & NM_EXCH) ? M->A0 : 0.0, Ku = (terms & NM_ANIS) ? M->Ku0 : 0.0;
         p.ucx = 2.0 * A * dx[1] * dx[2] / (36.0 * dx[0]);
@@ -227,6 +227,13 @@ inline LocalParams<T> local_params(nm_mesh M, unsigned terms)
         p.ucz = 2.0 * A * dx[0] * dx[1] / (36.0 * dx[2]);
         p.uan = 2.0 * Ku * V / 216.0;
         p.uim = 1.0 / (kMu0 * V / 8.0 * M->Ms0);
+        if (M->g.basis == 2) {
+            const double th = M->g.N3 * dx[2];
+            p.ucx = 2.0 * A * th * dx[1] / (6.0 * dx[0]);
+            p.ucy = 2.0 * A * th * dx[0] / (6.0 * dx[1]);
+            p.uan = 2.0 * Ku * th * dx[0] * dx[1] / 36.0;
+            p.uim = 1.0 / (kMu0 * th * dx[0] * dx[1] / 4.0 * M->Ms0);
+        }
     }
     p.gam = M->gamma / (1.0 + M->alpha * M->alpha);
     p.alpha = M->alpha;

@@ -1,4 +1,4 @@
-// Node kernel of the trilinear basis for a uniform material (no cell maps, Ms > 0): exchange, uniaxial
+// Node kernels of the trilinear and of the 2D basis for a uniform material (no cell maps, Ms > 0): exchange, uniaxial
 // anisotropy, Zeeman and the cell->node demag average, divided by the lumped nodal mass (Eqs.
 // weak_form_impl_f, weak_form_impl, mass_lumping), followed by the LLG right-hand side (Eq. llg) and the next
 // Runge-Kutta stage input.
@@ -132,9 +132,9 @@ struct NodeUArgs {
     int nn1, nn2, nn3, N1, N2, N3, ns, cs;
     int bxn, full, chunks, zc;  // blocks b < full walk tile b over all planes; the other tiles are split into
                                 // `chunks` blocks of zc planes
-    T cx, cy, cz, can;          // 2 A x element constants of the three axes; 2 Ku V / 216
+    T cx, cy, cz, can;          // 2 A x element constants of the axes; 2 Ku V / 216 (2D basis: / 36 per layer)
     T e0, e1, e2;
-    T im1, mu0V8;               // 1 / (mu0 V/8 Ms); mu0 V/8
+    T im1, mu0V8;               // 1 / (mu0 V/8 Ms), mu0 V/8 (2D basis: 1 / (mu0 V/4 Ms N3), mu0 V/4)
     T gam, alpha;
     const T *y, *MsH, *Msh, *hdmi;
     T *out, *y_next;
@@ -169,6 +169,53 @@ __device__ __forceinline__ void cp_elem(T *dst, const T *src, bool in)
 // formed from NK >= 0 earlier slopes.  M64: the next input is formed from the FP64 m (always in FP64, and in
 // FP32 where no FP32 copy of m is kept).
 constexpr int kHeff = -2, kSlope = -1;
+
+// The node's output from its field: H itself, or the LLG slope k and the next stage input
+template <typename T, int NK, bool M64>
+__device__ __forceinline__ void node_u_out(const NodeUArgs<T> &p, int n, T hx, T hy, T hz, T mx, T my, T mz, T dt,
+                                           double dt64)
+{
+    if (NK == kHeff) {
+        p.out[n] = hx;
+        p.out[p.ns + n] = hy;
+        p.out[2 * p.ns + n] = hz;
+    } else {
+        // the next stage input's own values, all loads issued together
+        T kv[NK > 0 ? NK : 1][3], m0[3];
+        double md[3];
+        if (NK >= 0) {
+#pragma unroll
+            for (int i = 0; i < NK; ++i)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) kv[i][c] = p.k[i][c * p.ns + n];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (M64) md[c] = p.m[c * p.ns + n];
+                else m0[c] = (T)p.mf[c * p.ns + n];
+            }
+        }
+        // k = -gamma' (m x H + alpha m x (m x H))
+        const T ax = my * hz - mz * hy, ay = mz * hx - mx * hz, az = mx * hy - my * hx;
+        const T bx = my * az - mz * ay, by = mz * ax - mx * az, bz = mx * ay - my * ax;
+        T kk[3];
+        kk[0] = -p.gam * (ax + p.alpha * bx);
+        kk[1] = -p.gam * (ay + p.alpha * by);
+        kk[2] = -p.gam * (az + p.alpha * bz);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) p.out[c * p.ns + n] = kk[c];
+        if (NK >= 0) {
+            // y_{s+1} = m + dt sum_j a_j k_j, the slope combination in the working precision
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                T sum = 0;
+#pragma unroll
+                for (int i = 0; i < NK; ++i) sum += p.a[i] * kv[i][c];
+                sum += p.as * kk[c];
+                p.y_next[c * p.ns + n] = M64 ? (T)(md[c] + dt64 * (double)sum) : m0[c] + dt * sum;
+            }
+        }
+    }
+}
 
 template <typename T, int NK, bool M64>
 __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(const __grid_constant__ NodeUArgs<T> p)
@@ -333,46 +380,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(co
                     hz += sm.hf[2];
                 }
             }
-            if (NK == kHeff) {
-                p.out[n] = hx;
-                p.out[p.ns + n] = hy;
-                p.out[2 * p.ns + n] = hz;
-            } else {
-                // the next stage input's own values, all loads issued together
-                T kv[NK > 0 ? NK : 1][3], m0[3];
-                double md[3];
-                if (NK >= 0) {
-#pragma unroll
-                    for (int i = 0; i < NK; ++i)
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) kv[i][c] = p.k[i][c * p.ns + n];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        if (M64) md[c] = p.m[c * p.ns + n];
-                        else m0[c] = (T)p.mf[c * p.ns + n];
-                    }
-                }
-                // k = -gamma' (m x H + alpha m x (m x H))
-                const T ax = my * hz - mz * hy, ay = mz * hx - mx * hz, az = mx * hy - my * hx;
-                const T bx = my * az - mz * ay, by = mz * ax - mx * az, bz = mx * ay - my * ax;
-                T kk[3];
-                kk[0] = -p.gam * (ax + p.alpha * bx);
-                kk[1] = -p.gam * (ay + p.alpha * by);
-                kk[2] = -p.gam * (az + p.alpha * bz);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) p.out[c * p.ns + n] = kk[c];
-                if (NK >= 0) {
-                    // y_{s+1} = m + dt sum_j a_j k_j, the slope combination in the working precision
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        T sum = 0;
-#pragma unroll
-                        for (int i = 0; i < NK; ++i) sum += p.a[i] * kv[i][c];
-                        sum += p.as * kk[c];
-                        p.y_next[c * p.ns + n] = M64 ? (T)(md[c] + dt64 * (double)sum) : m0[c] + dt * sum;
-                    }
-                }
-            }
+            node_u_out<T, NK, M64>(p, n, hx, hy, hz, mx, my, mz, dt, dt64);
         }
         acc = vadd(up, own);
         accR = upR + ownR;
@@ -382,6 +390,77 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(co
         cc = ccur;
         s = s + 1 >= kUSlots ? 0 : s + 1;
     }
+}
+
+// The same operators for the 2D nodal basis (one node layer, constant over the N3 cell layers): the field is
+//   -2 A (K1 M2 + M1 K2) m + 2 Ku e (M1 M2) (e . m), both times the film's thickness,
+// one thread per node, neighbours and cells through L1.  Bound by instruction issue and L1 latency: 26.6 us per stage
+// at 1024x1024x1 (events around each launch) against 52.4 us with the assembled 9-point weights of the general 2D
+// kernel, which sums A, Ku and the cell weights of every layer at every node.
+constexpr int kU2X = 32, kU2Y = 4;
+template <typename T, int NK, bool M64>
+__global__ void __launch_bounds__(kU2X *kU2Y) k_node2d_u(const __grid_constant__ NodeUArgs<T> p)
+{
+    pdl_enter();
+    if (NK != kHeff && p.ctl && p.ctl->done) return;
+    const int n1 = blockIdx.x * kU2X + threadIdx.x % kU2X, n2 = blockIdx.y * kU2Y + threadIdx.x / kU2X;
+    if (n1 >= p.nn1 || n2 >= p.nn2) return;
+    const int n = n2 * p.nn1 + n1;
+    const T dt = NK >= 0 && p.ctl ? (T)p.ctl->dt : T(0);
+    const double dt64 = NK >= 0 && p.ctl ? p.ctl->dt : 0.0;
+    const bool xl = n1 >= 1, xh = n1 < p.N1, yl = n2 >= 1, yh = n2 < p.N2;
+    const T nx = xl && xh ? T(2) : T(1), ny = yl && yh ? T(2) : T(1);
+    T h[3], m[3], P[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        // row sums along x of rows n2 - 1 .. n2 + 1: a = 6 M1 m / dx, d = -dx K1 m (zero beyond the ends)
+        const T *q = p.y + c * p.ns + n;
+        T a[3], d[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const bool in = r == 1 || (r == 0 ? yl : yh);
+            const T *qr = q + (r - 1) * p.nn1;
+            const T c0 = in ? qr[0] : T(0), e = (in && xl ? qr[-1] : T(0)) + (in && xh ? qr[1] : T(0));
+            a[r] = fma(T(2) * nx, c0, e);
+            d[r] = fma(-nx, c0, e);
+            if (r == 1) m[c] = c0;
+        }
+        const T as = a[0] + a[2];
+        P[c] = fma(T(2) * ny, a[1], as);
+        h[c] = p.cx * fma(T(2) * ny, d[1], d[0] + d[2]) + p.cy * fma(-ny, a[1], as);
+    }
+    const T pe = p.can * (p.e0 * P[0] + p.e1 * P[1] + p.e2 * P[2]);
+    h[0] += p.e0 * pe;
+    h[1] += p.e1 * pe;
+    h[2] += p.e2 * pe;
+    // Ms H (and the cell field) over the in-plane cells of every layer
+    auto cells = [&](const T *f, T s) {
+        T sum[3] = {0, 0, 0};
+        for (int c3 = 0; c3 < p.N3; ++c3) {
+            const T *q = f + (c3 * p.N2 + n2) * p.N1 + n1;
+#pragma unroll
+            for (int c = 0; c < 3; ++c, q += p.cs)
+                sum[c] += ((xl && yl ? q[-p.N1 - 1] : T(0)) + (xh && yl ? q[-p.N1] : T(0))) +
+                          ((xl && yh ? q[-1] : T(0)) + (xh && yh ? q[0] : T(0)));
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) h[c] += p.mu0V8 * s * sum[c];
+    };
+    const double t = NK != kHeff && p.ctl ? p.ctl->t + p.c_s * p.ctl->dt : p.t_fixed;
+    if (p.MsH) cells(p.MsH, T(1));
+    if (p.Msh && p.zee) cells(p.Msh, (T)u_time_factor<T>(p.hc_freq, p.hc_phase, t));
+    if (!p.raw) {
+        const T im = p.im1 * (nx == T(2) ? T(0.5) : T(1)) * (ny == T(2) ? T(0.5) : T(1));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) h[c] *= im;
+        if (p.zee) {
+            const double su = u_time_factor<T>(p.hu_freq, p.hu_phase, t);
+            h[0] += (T)(p.hu0 * su);
+            h[1] += (T)(p.hu1 * su);
+            h[2] += (T)(p.hu2 * su);
+        }
+    }
+    node_u_out<T, NK, M64>(p, n, h[0], h[1], h[2], m[0], m[1], m[2], dt, dt64);
 }
 
 // Split of the walk: cost in plane units of a grid whose tiles are cut into `chunks` pieces, from the latency
@@ -416,6 +495,10 @@ static void node_u_grid(int nn1, int nn2, int nn3, int sms, int *bxn, int *full,
 template <typename T, int NK, bool M64>
 static void launch_u(const NodeUArgs<T> &a, int blocks, cudaStream_t st)
 {
+    if (blocks == 0) {  // 2D basis
+        launch_pdl(k_node2d_u<T, NK, M64>, dim3(div_up(a.nn1, kU2X), div_up(a.nn2, kU2Y)), kU2X * kU2Y, 0, st, a);
+        return;
+    }
     launch_pdl(k_node_u<T, NK, M64>, blocks, kUThreads, 0, st, a);
 }
 
@@ -430,20 +513,22 @@ static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *
     a.ns = (int)g.ns;
     a.cs = (int)g.cs;
     int blocks = 0;
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
+    if (g.basis == 3) {
+        static int sms = 0;
+        if (sms == 0) {
+            int dev = 0, v = 0;
+            cudaGetDevice(&dev);
+            sms = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 152;
+        }
+        node_u_grid(g.nn1, g.nn2, g.nn3, sms, &a.bxn, &a.full, &a.chunks, &a.zc, &blocks);
     }
-    node_u_grid(g.nn1, g.nn2, g.nn3, sms, &a.bxn, &a.full, &a.chunks, &a.zc, &blocks);
     a.cx = (T)p.ucx;
     a.cy = (T)p.ucy;
     a.cz = (T)p.ucz;
     a.can = (T)p.uan;
     a.e0 = p.e0; a.e1 = p.e1; a.e2 = p.e2;
     a.im1 = (T)p.uim;
-    a.mu0V8 = p.mu0V8;
+    a.mu0V8 = g.basis == 3 ? p.mu0V8 : p.mu0V4;
     a.gam = p.gam_t;
     a.alpha = p.alpha_t;
     a.y = y;
