@@ -147,7 +147,7 @@ static void release(nm_mesh M)
     void *ptrs[] = {M->m, M->mf, M->y[0], M->y[1], M->hin, M->hout, M->inv_mass, M->vol, M->MsH, M->S, M->Nk, M->tw,
                     M->tw64, M->A_d, M->Ku_d, M->Ms_d, M->Ms64_d, M->Msh_d, M->hcell64_d, M->D_d, M->hdmi, M->ctl,
                     M->partials,
-                    M->mean_d, M->n_active_d, M->n_bad_d, M->vj_w, M->vj_h, M->vj_q, M->vj_g, M->vj_H, M->vj_HW, M->vj_M,
+                    M->mean_d, M->n_active_d, M->n_bad_d, M->vj_w, M->vj_h, M->vj_q, M->vj_g, M->vj_H, M->vj_HW,
                     M->vj_gMs};
     for (void *p : ptrs)
         if (p) cudaFree(p);

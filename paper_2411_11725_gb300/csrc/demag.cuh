@@ -66,14 +66,10 @@ struct DemagPlan {
 template <typename T>
 DemagPlan demag_plan(const Geom &g);
 
-// Demag of the nodal field y (SoA, real T): writes (Ms_c H_c) per cell into MsH (3 x cs).
+// Demag of the nodal field y (SoA, real T): writes (Ms_c H_c) per cell into MsH (3 x cs) and, when H is not
+// NULL, H_c itself there (3 x cs).
 template <typename T>
-void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cudaStream_t st);
-
-// Same pipeline with an explicit cell input: M (3 x cs, already Ms-weighted cell magnetisation)
-// replaces the node->cell averaging; output H (3 x cs) without the Ms factor.  Used by the adjoint.
-template <typename T>
-void demag_cells(const Geom &g, const DemagBufs<T> &b, const T *M, T *H, cudaStream_t st);
+void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cudaStream_t st, T *H = nullptr);
 
 // TMA descriptor of a y-pass tile over the spectrum buffer S (host work only; no device access).
 // Returns 0, or a non-zero code when the driver's encoder is unavailable or refuses the shape.

@@ -110,11 +110,11 @@ __device__ __forceinline__ void cpa_chunk(void *sm, const void *gm, int cb)
 // cell rows of one component, so the node rows they average overlap.  Offsets (elements, int32: every
 // supported size fits) of the line's start in the node array, the cell arrays and the spectrum.
 struct XInfo {
-    int in;    // node array (nodal input) or cell array (cell input / output), component included
+    int in;    // node array (forward pass) or cell array (inverse pass), component included
     int cell;  // cell index of the row start (Ms map)
     int spec;  // spectrum row start
 };
-__device__ __forceinline__ XInfo x_info(const Geom &g, const FastDiv &nrf, int L, bool cell_in)
+__device__ __forceinline__ XInfo x_info(const Geom &g, const FastDiv &nrf, int L, bool cell)
 {
     const int NR = g.N2 * g.N3;
     const int c = (int)nrf.div((unsigned)L);
@@ -123,7 +123,7 @@ __device__ __forceinline__ XInfo x_info(const Geom &g, const FastDiv &nrf, int L
     const int yy = row - zz * g.N2;
     XInfo x;
     x.cell = row * g.N1;
-    x.in = cell_in ? c * (int)g.cs + x.cell : c * (int)g.ns + zz * g.zsn + yy * g.ysn;
+    x.in = cell ? c * (int)g.cs + x.cell : c * (int)g.ns + zz * g.zsn + yy * g.ysn;
     x.spec = c * (int)g.s_comp + (zz * g.P2 + yy) * g.Xp;
     return x;
 }
@@ -149,8 +149,8 @@ __device__ __forceinline__ Cx<T> cell_M_pair(const T *__restrict__ p, int row, i
 }
 
 // Pass 1: x transform (R2C of length P1 = 2Q via a complex FFT of length Q = 2^LG on even/odd pairs).
-// One block holds `lpb` consecutive lines.  CELL_IN: the input is already a cell field.
-template <typename T, bool CELL_IN, int LG>
+// One block holds `lpb` consecutive lines.
+template <typename T, int LG>
 __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
     k_x_fwd(Geom g, DemagBufs<T> b, const T *__restrict__ in, int lpb)
 {
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
     const int l0 = blockIdx.x * lpb;
     const int nl = min(lpb, nlines - l0);
     if (nl <= 0) return;
-    if (threadIdx.x < nl) info[threadIdx.x] = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), l0 + threadIdx.x, CELL_IN);
+    if (threadIdx.x < nl) info[threadIdx.x] = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), l0 + threadIdx.x, false);
     __syncthreads();
     const int N1 = g.N1, row = g.ysn, plane = g.zsn;  // 2D (1D) basis: both z (y and z) corners are the node
     const T *Ms = b.Ms;
@@ -173,7 +173,6 @@ __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
         const int x = 2 * i;
         const XInfo xi = info[l];
         const T *p = in + xi.in + x;
-        if (CELL_IN) return cx<T>(p[0], x + 1 < N1 ? p[1] : T(0));
         return cell_M_pair<T>(p, row, plane, Ms, Ms0, xi.cell + x, x + 1 < N1);
     };
     f3::fft<T, LG, -1, false, false, true, kXEpt<T, LG>>(buf, nl, FastDiv(1u), b.tw, g.twlg, (N1 + 1) >> 1, Q, src,
@@ -209,7 +208,7 @@ __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
 }
 
 // N1 == 1 (P1 == 1): the x "transform" is a copy of the cell value (real) into kx = 0.
-template <typename T, bool CELL_IN>
+template <typename T>
 __global__ void k_x_fwd1(Geom g, DemagBufs<T> b, const T *__restrict__ in)
 {
     pdl_enter();
@@ -217,18 +216,16 @@ __global__ void k_x_fwd1(Geom g, DemagBufs<T> b, const T *__restrict__ in)
     const int nlines = 3 * g.N2 * g.N3;
     const int L = blockIdx.x * blockDim.x + threadIdx.x;
     if (L >= nlines) return;
-    const XInfo xi = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), L, CELL_IN);
-    T v;
-    if (CELL_IN) v = in[xi.in];
-    else v = cell_M_pair<T>(in + xi.in, g.ysn, g.zsn, b.Ms, b.Ms0, xi.cell, false).x;
+    const XInfo xi = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), L, false);
+    const T v = cell_M_pair<T>(in + xi.in, g.ysn, g.zsn, b.Ms, b.Ms0, xi.cell, false).x;
     b.S[xi.spec] = cx<T>(v, T(0));
 }
 
 // Pass 5: inverse x transform (C2R of length P1 via a complex FFT of length Q), keeping x < N1.
-// Output per cell: Ms_c H_c (or H_c when CELL_OUT).
-template <typename T, bool CELL_OUT, int LG>
+// Output per cell: Ms_c H_c and, when H is not NULL, H_c itself there.
+template <typename T, int LG>
 __global__ void __launch_bounds__(kXiThreads<T>, sizeof(T) == 4 ? 16 : 4)
-    k_x_inv(Geom g, DemagBufs<T> b, T *__restrict__ out, int lpb)
+    k_x_inv(Geom g, DemagBufs<T> b, T *__restrict__ out, T *__restrict__ H_out, int lpb)
 {
     pdl_enter();
     if (b.ctl && b.ctl->done) return;
@@ -288,18 +285,20 @@ __global__ void __launch_bounds__(kXiThreads<T>, sizeof(T) == 4 ? 16 : 4)
         const XInfo xi = info[l];
         const int x = 2 * j;
         T v0 = v.x, v1 = v.y;
-        if (!CELL_OUT) {
-            v0 *= Ms ? Ms[xi.cell + x] : Ms0;
-            if (x + 1 < N1) v1 *= Ms ? Ms[xi.cell + x + 1] : Ms0;
+        if (H_out) {
+            H_out[xi.in + x] = v0;
+            if (x + 1 < N1) H_out[xi.in + x + 1] = v1;
         }
+        v0 *= Ms ? Ms[xi.cell + x] : Ms0;
+        if (x + 1 < N1) v1 *= Ms ? Ms[xi.cell + x + 1] : Ms0;
         out[xi.in + x] = v0;
         if (x + 1 < N1) out[xi.in + x + 1] = v1;
     };
     f3::fft<T, LG, +1, false, true, false, kXEpt<T, LG>>(buf, nl, FastDiv(1u), b.tw, g.twlg, Q, (N1 + 1) >> 1, f3::NoFn<T>(), dst);
 }
 
-template <typename T, bool CELL_OUT>
-__global__ void k_x_inv1(Geom g, DemagBufs<T> b, T *__restrict__ out)
+template <typename T>
+__global__ void k_x_inv1(Geom g, DemagBufs<T> b, T *__restrict__ out, T *__restrict__ H_out)
 {
     pdl_enter();
     if (b.ctl && b.ctl->done) return;
@@ -308,7 +307,8 @@ __global__ void k_x_inv1(Geom g, DemagBufs<T> b, T *__restrict__ out)
     if (L >= nlines) return;
     const XInfo xi = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), L, true);
     T v = b.S[xi.spec].x;
-    if (!CELL_OUT) v *= b.Ms ? b.Ms[xi.cell] : b.Ms0;
+    if (H_out) H_out[xi.in] = v;
+    v *= b.Ms ? b.Ms[xi.cell] : b.Ms0;
     out[xi.in] = v;
 }
 
@@ -1068,10 +1068,8 @@ static void init_attributes_t()
 {
     f3::lg_for_each<1, 10>([&](auto c) {
         constexpr int LG = decltype(c)::value;
-        set_smem((const void *)k_x_fwd<T, false, LG>);
-        set_smem((const void *)k_x_fwd<T, true, LG>);
-        set_smem((const void *)k_x_inv<T, false, LG>);
-        set_smem((const void *)k_x_inv<T, true, LG>);
+        set_smem((const void *)k_x_fwd<T, LG>);
+        set_smem((const void *)k_x_inv<T, LG>);
     });
     f3::lg_for_each<1, 11>([&](auto c) {
         constexpr int LG = decltype(c)::value;
@@ -1253,8 +1251,8 @@ int demag_encode_ymap(const Geom &g, void *S, CUtensorMap *map)
     return r == CUDA_SUCCESS ? 0 : (int)r;
 }
 
-template <typename T, bool CELL>
-static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *out, cudaStream_t st)
+template <typename T>
+void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cudaStream_t st, T *H)
 {
     const DemagPlan p = demag_plan<T>(g);
     if (!p.ok) return;
@@ -1262,11 +1260,11 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
     if (g.N3 > 1 && g.P2 > 1 && !b.ymap) return;
     const int nlines = 3 * g.N2 * g.N3;
     if (g.P1 == 1) {
-        launch_pdl(k_x_fwd1<T, CELL>, div_up(nlines, 256), 256, 0, st, g, b, in);
+        launch_pdl(k_x_fwd1<T>, div_up(nlines, 256), 256, 0, st, g, b, y);
     } else {
         f3::lg_dispatch<1, 10>(g.lgQ, [&](auto c) {
             constexpr int LG = decltype(c)::value;
-            launch_pdl(k_x_fwd<T, CELL, LG>, div_up(nlines, p.x_lpb), p.x_threads, p.x_smem, st, g, b, in, p.x_lpb);
+            launch_pdl(k_x_fwd<T, LG>, div_up(nlines, p.x_lpb), p.x_threads, p.x_smem, st, g, b, y, p.x_lpb);
         });
     }
     b.mark("demag_x_fwd");
@@ -1307,26 +1305,15 @@ static void run_pipeline(const Geom &g, const DemagBufs<T> &b, const T *in, T *o
         }
     }
     if (g.P1 == 1) {
-        launch_pdl(k_x_inv1<T, CELL>, div_up(nlines, 256), 256, 0, st, g, b, out);
+        launch_pdl(k_x_inv1<T>, div_up(nlines, 256), 256, 0, st, g, b, MsH, H);
     } else {
         f3::lg_dispatch<1, 10>(g.lgQ, [&](auto c) {
             constexpr int LG = decltype(c)::value;
-            launch_pdl(k_x_inv<T, CELL, LG>, div_up(nlines, p.xi_lpb), p.xi_threads, p.xi_smem, st, g, b, out, p.xi_lpb);
+            launch_pdl(k_x_inv<T, LG>, div_up(nlines, p.xi_lpb), p.xi_threads, p.xi_smem, st, g, b, MsH, H,
+                       p.xi_lpb);
         });
     }
     b.mark("demag_x_inv");
-}
-
-template <typename T>
-void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cudaStream_t st)
-{
-    run_pipeline<T, false>(g, b, y, MsH, st);
-}
-
-template <typename T>
-void demag_cells(const Geom &g, const DemagBufs<T> &b, const T *M, T *H, cudaStream_t st)
-{
-    run_pipeline<T, true>(g, b, M, H, st);
 }
 
 }  // namespace nm

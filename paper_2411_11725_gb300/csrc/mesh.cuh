@@ -98,7 +98,7 @@ struct nm_mesh_s {
     cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};
     // adjoint workspaces (allocated on first use)
     void *vj_w = nullptr, *vj_h = nullptr, *vj_q = nullptr, *vj_g = nullptr;      // nodal 3 x ns
-    void *vj_H = nullptr, *vj_HW = nullptr, *vj_M = nullptr;                      // cells 3 x cs
+    void *vj_H = nullptr, *vj_HW = nullptr;                                            // cells 3 x cs
     double *vj_gMs = nullptr;                                                    // cells, FP64 accumulator
     double *vj_gh = nullptr;  // nodal FP64 accumulator of the uniform-field gradient (during nm_adjoint_run)
     std::vector<void *> extra;                                                   // further adjoint buffers

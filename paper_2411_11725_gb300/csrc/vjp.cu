@@ -16,29 +16,6 @@ __global__ void k_scale_inv_mass(long n_nodes, long ns, const T *__restrict__ v,
 }
 
 template <typename T>
-__global__ void k_cell_moment(Geom g, const T *__restrict__ y, const T *__restrict__ Ms, T Ms0, T scale,
-                              T *__restrict__ out)
-{
-    pdl_enter();
-    long c = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (c >= g.n_cells) return;
-    const int c1 = (int)(c % g.N1);
-    const long r = c / g.N1;
-    const int c2 = (int)(r % g.N2);
-    const int c3 = (int)(r / g.N2);
-    // corner offsets of the nodal basis: nn1 and nn1 nn2 for the trilinear basis; 0 along the directions
-    // in which the 2D or 1D basis is constant, where the 8-corner sum counts each node twice (or 4 times)
-    const long sy = g.ysn, sz = g.zsn;
-    const long n0 = (long)c3 * sz + (long)c2 * sy + c1;
-    const T ms = Ms ? Ms[c] : Ms0;
-    for (int k = 0; k < 3; ++k) {
-        const T *p = y + k * g.ns + n0;
-        T s = (p[0] + p[1]) + (p[sy] + p[sy + 1]) + (p[sz] + p[sz + 1]) + (p[sz + sy] + p[sz + sy + 1]);
-        out[k * g.cs + c] = ms * scale * s;
-    }
-}
-
-template <typename T>
 __global__ void k_grad_Ms(Geom g, GradMsArgs a, const T *__restrict__ im, double *__restrict__ gMs)
 {
     pdl_enter();
@@ -48,8 +25,8 @@ __global__ void k_grad_Ms(Geom g, GradMsArgs a, const T *__restrict__ im, double
     const long r = c / g.N1;
     const int c2 = (int)(r % g.N2);
     const int c3 = (int)(r / g.N2);
-    // corner offsets as in k_cell_moment: with the 2D and 1D bases the 8 corners collapse onto the
-    // cell's 4 (2) nodes, which gives the gradient of the restricted system (basis functions that are
+    // corner offsets of the nodal basis: nn1 and nn1 nn2 for the trilinear basis, 0 along the directions in
+    // which the 2D or 1D basis is constant, where the 8 corners collapse onto the cell's 4 (2) nodes, which gives the gradient of the restricted system (basis functions that are
     // sums of trilinear ones, integrals V/4 or V/2 per cell)
     const long sy = g.ysn, sz = g.zsn;
     const long n0 = (long)c3 * sz + (long)c2 * sy + c1;
@@ -69,7 +46,7 @@ __global__ void k_grad_Ms(Geom g, GradMsArgs a, const T *__restrict__ im, double
         double Hc = 0.0, HWc = 0.0;
         if (a.demag) {
             Hc = (double)((const T *)a.H)[k * g.cs + c];
-            HWc = (double)((const T *)a.HW)[k * g.cs + c];
+            HWc = 8.0 * (double)((const T *)a.Hw)[k * g.cs + c];
         }
         if (a.hcell) Hc += a.sc * a.hcell[k * g.cs + c];
         acc += W * Hc + mb * HWc - mass_term;
@@ -77,19 +54,25 @@ __global__ void k_grad_Ms(Geom g, GradMsArgs a, const T *__restrict__ im, double
     gMs[c] += a.weight * a.mu0V8 * acc;
 }
 
+// (the sums of stage cotangents, the division by the mass and the uniform-field accumulation ride along: each
+// was a launch of its own over the same nodes)
 template <typename T>
 __global__ void k_llg_vjp_local(long n_nodes, long ns, const T *__restrict__ y, const T *__restrict__ H,
-                                const T *__restrict__ u, const T *__restrict__ im, T gam, T alpha,
-                                T *__restrict__ ybar, T *__restrict__ q)
+                                const __grid_constant__ LinComb lu, const T *__restrict__ im, T gam, T alpha,
+                                T *__restrict__ ybar, T *__restrict__ w, double scale, double *__restrict__ acc)
 {
     pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
     T yv[3], Hv[3], uv[3];
     for (int k = 0; k < 3; ++k) {
-        yv[k] = y[k * ns + n];
-        Hv[k] = H[k * ns + n];
-        uv[k] = u[k * ns + n];
+        const long i = k * ns + n;
+        yv[k] = y[i];
+        Hv[k] = H[i];
+        double u = 0.0;
+        for (int j = 0; j < lu.nt; ++j) u += lu.at[j] * (double)((const T *)lu.pt[j])[i];
+        for (int j = 0; j < lu.nd; ++j) u += lu.ad[j] * lu.pd[j][i];
+        uv[k] = (T)u;
     }
     auto cross = [](const T *a, const T *b, T *c) {
         c[0] = a[1] * b[2] - a[2] * b[1];
@@ -97,7 +80,8 @@ __global__ void k_llg_vjp_local(long n_nodes, long ns, const T *__restrict__ y, 
         c[2] = a[0] * b[1] - a[1] * b[0];
     };
     T yb[3] = {0, 0, 0}, qv[3] = {0, 0, 0};
-    if (im[n] > T(0)) {
+    const T s = im[n];
+    if (s > T(0)) {
         T Hxu[3], yxH[3], yxHxu[3], uxy[3], Hxuxy[3], uxyxy[3];
         cross(Hv, uv, Hxu);
         cross(yv, Hv, yxH);
@@ -112,7 +96,36 @@ __global__ void k_llg_vjp_local(long n_nodes, long ns, const T *__restrict__ y, 
     }
     for (int k = 0; k < 3; ++k) {
         ybar[k * ns + n] = yb[k];
-        q[k * ns + n] = qv[k];
+        w[k * ns + n] = qv[k] * s;
+        if (acc) acc[k * ns + n] += scale * (double)qv[k];
+    }
+}
+
+template <typename T>
+__global__ void k_llg_slope(long n_nodes, long ns, const T *__restrict__ y, const T *__restrict__ h,
+                            const T *__restrict__ im, T gam, T alpha, T *__restrict__ k_out, T *__restrict__ y_next,
+                            const double *__restrict__ m, double dt, const __grid_constant__ LinComb e, double a_s)
+{
+    pdl_enter();
+    long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (n >= n_nodes) return;
+    const T mx = y[n], my = y[ns + n], mz = y[2 * ns + n], hx = h[n], hy = h[ns + n], hz = h[2 * ns + n];
+    T k[3] = {0, 0, 0};
+    if (im[n] > T(0)) {
+        const T ax = my * hz - mz * hy, ay = mz * hx - mx * hz, az = mx * hy - my * hx;
+        const T bx = my * az - mz * ay, by = mz * ax - mx * az, bz = mx * ay - my * ax;
+        k[0] = -gam * (ax + alpha * bx);
+        k[1] = -gam * (ay + alpha * by);
+        k[2] = -gam * (az + alpha * bz);
+    }
+    for (int c = 0; c < 3; ++c) {
+        const long i = c * ns + n;
+        k_out[i] = k[c];
+        if (!y_next) continue;
+        T sum = 0;
+        for (int j = 0; j < e.nt; ++j) sum += (T)e.at[j] * ((const T *)e.pt[j])[i];
+        sum += (T)a_s * k[c];
+        y_next[i] = (T)(m[i] + dt * (double)sum);
     }
 }
 
@@ -134,23 +147,25 @@ void launch_scale_inv_mass(const Geom &g, const T *v, const T *inv_mass, T *w, c
 }
 
 template <typename T>
-void launch_cell_moment(const Geom &g, const T *y, const T *Ms, T Ms0, T scale, T *out, cudaStream_t st)
-{
-    launch_pdl(k_cell_moment<T>, div_up(g.n_cells, 256), 256, 0, st, g, y, Ms, Ms0, scale, out);
-}
-
-template <typename T>
 void launch_grad_Ms(const Geom &g, const GradMsArgs &a, const T *inv_mass, double *gMs, cudaStream_t st)
 {
     launch_pdl(k_grad_Ms<T>, div_up(g.n_cells, 256), 256, 0, st, g, a, inv_mass, gMs);
 }
 
 template <typename T>
-void launch_llg_vjp_local(const Geom &g, const T *y, const T *H, const T *u, const T *inv_mass, double gam,
-                          double alpha, T *ybar, T *q, cudaStream_t st)
+void launch_llg_vjp_local(const Geom &g, const T *y, const T *H, const LinComb &lu, const T *inv_mass, double gam,
+                          double alpha, T *ybar, T *w, double scale, double *acc, cudaStream_t st)
 {
-    launch_pdl(k_llg_vjp_local<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, y, H, u, inv_mass, (T)gam, (T)alpha,
-                                                                 ybar, q);
+    launch_pdl(k_llg_vjp_local<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, y, H, lu, inv_mass, (T)gam,
+               (T)alpha, ybar, w, scale, acc);
+}
+
+template <typename T>
+void launch_llg_slope(const Geom &g, const T *y, const T *h, const T *inv_mass, double gam, double alpha, T *k_out,
+                      T *y_next, const double *m, double dt, const LinComb &earlier, double a_s, cudaStream_t st)
+{
+    launch_pdl(k_llg_slope<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, y, h, inv_mass, (T)gam, (T)alpha,
+               k_out, y_next, m, dt, earlier, a_s);
 }
 
 template <typename T>
@@ -161,10 +176,11 @@ void launch_axpby(const Geom &g, T a, const T *x, T b, const T *y, T *out, cudaS
 
 #define NM_VJP_INST(T)                                                                                          \
     template void launch_scale_inv_mass<T>(const Geom &, const T *, const T *, T *, cudaStream_t);               \
-    template void launch_cell_moment<T>(const Geom &, const T *, const T *, T, T, T *, cudaStream_t);            \
     template void launch_grad_Ms<T>(const Geom &, const GradMsArgs &, const T *, double *, cudaStream_t);         \
-    template void launch_llg_vjp_local<T>(const Geom &, const T *, const T *, const T *, const T *, double,      \
-                                          double, T *, T *, cudaStream_t);                                      \
+    template void launch_llg_vjp_local<T>(const Geom &, const T *, const T *, const LinComb &, const T *, double, \
+                                          double, T *, T *, double, double *, cudaStream_t);                     \
+    template void launch_llg_slope<T>(const Geom &, const T *, const T *, const T *, double, double, T *, T *,   \
+                                      const double *, double, const LinComb &, double, cudaStream_t);           \
     template void launch_axpby<T>(const Geom &, T, const T *, T, const T *, T *, cudaStream_t);
 NM_VJP_INST(float)
 NM_VJP_INST(double)
@@ -329,21 +345,6 @@ void launch_sum_partials(const double *partials, int n, double *out, cudaStream_
     launch_pdl(k_sum_partials, 1, 1024, 0, st, partials, n, out);
 }
 
-template <typename T>
-__global__ void k_accum_nodal(long n_nodes, long ns, const T *__restrict__ q, double scale, double *__restrict__ acc)
-{
-    pdl_enter();
-    long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (n >= n_nodes) return;
-    for (int c = 0; c < 3; ++c) acc[c * ns + n] += scale * (double)q[c * ns + n];
-}
-
-template <typename T>
-void launch_accum_nodal(const Geom &g, const T *q, double scale, double *acc, cudaStream_t st)
-{
-    launch_pdl(k_accum_nodal<T>, (int)((g.n_nodes + 255) / 256), 256, 0, st, g.n_nodes, g.ns, q, scale, acc);
-}
-
 __global__ void __launch_bounds__(256) k_sum_nodal3_partials(long n_nodes, long ns, const double *__restrict__ acc,
                                                               double *partials)
 {
@@ -370,9 +371,6 @@ void launch_sum_nodal3(const Geom &g, const double *acc, double *partials, doubl
     launch_pdl(k_sum_nodal3_partials, nb, 256, 0, st, g.n_nodes, g.ns, acc, partials);
     for (int c = 0; c < 3; ++c) launch_pdl(k_sum_partials, 1, 1024, 0, st, partials + c * 1024, nb, out + c);
 }
-
-template void launch_accum_nodal<float>(const Geom &, const float *, double, double *, cudaStream_t);
-template void launch_accum_nodal<double>(const Geom &, const double *, double, double *, cudaStream_t);
 
 #define NM_ADJ_INST(T)                                                                                          \
     template void launch_lincomb<T>(const Geom &, const LinComb &, T *, cudaStream_t);                          \
