@@ -68,6 +68,7 @@ static Geom make_geom(int n1, int n2, int n3, int basis = 3)
     g.s_comp = (long)n3 * g.P2 * g.Xp;
     g.t_comp = (long)g.H3 * g.H2 * g.Xp;
     g.n2f = FastDiv((unsigned)n2);
+    g.nrf = FastDiv((unsigned)(n2 * n3));
     return g;
 }
 
@@ -730,14 +731,25 @@ static void enqueue_stage(nm_mesh M, const LocalParams<T> &p, int s, double c_s,
     marker(M)("node_llg_stage");
 }
 
+// m as the input of a stage: m itself or its FP32 copy, which hold the same values in the same layout; the copy
+// into a stage input only where a FP32 mesh keeps none (during the adjoint runs)
+template <typename T>
+static const T *state_input(nm_mesh M, T *y)
+{
+    if (sizeof(T) == 8) return (const T *)M->m;
+    if (M->mf) return (const T *)M->mf;
+    KList none{};
+    launch_stage_input<T>(M->g, M->m, none, M->ctl, y, M->st, M->mf);
+    marker(M)("stage_input");
+    return y;
+}
+
 // k1 = f(m) at the resident time (first DP5 step after a state change)
 template <typename T>
 static void enqueue_k1(nm_mesh M)
 {
     const LocalParams<T> p = local_params<T>(M, M->terms);
-    KList none{};
-    launch_stage_input<T>(M->g, M->m, none, M->ctl, (T *)M->y[0], M->st, M->mf);
-    enqueue_stage<T>(M, p, 1, 0.0, (const T *)M->y[0], nullptr, nullptr, 0);
+    enqueue_stage<T>(M, p, 1, 0.0, state_input<T>(M, (T *)M->y[0]), nullptr, nullptr, 0);
 }
 
 template <typename T>
@@ -778,11 +790,9 @@ static void enqueue_rk4_step(nm_mesh M)
 {
     const LocalParams<T> p = local_params<T>(M, M->terms);
     const Geom &g = M->g;
-    KList none{};
-    launch_stage_input<T>(g, M->m, none, M->ctl, (T *)M->y[1], M->st, M->mf);  // y_1 = m
-    marker(M)("stage_input");
+    const T *y1 = state_input<T>(M, (T *)M->y[1]);
     for (int s = 1; s <= 4; ++s) {
-        const T *ys = (const T *)M->y[s % 2];
+        const T *ys = s == 1 ? y1 : (const T *)M->y[s % 2];
         T *yn = s < 4 ? (T *)M->y[(s + 1) % 2] : nullptr;
         enqueue_stage<T>(M, p, s, kRk4C[s - 1], ys, yn, s < 4 ? kRk4A[s] : nullptr, s < 4 ? s : 0);
     }

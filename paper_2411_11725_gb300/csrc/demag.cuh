@@ -28,6 +28,7 @@ struct Geom {
     long t_comp;               // component stride of the tensor spectrum = H3 * H2 * Xp
     FastDiv n2f;               // division by N2 (cell row -> (y, z))
     int ysn;                   // node offset between the y corners of a cell: nn1 (3D, 2D) or 0 (1D)
+    FastDiv nrf;               // division by N2 N3 (x line -> component)
 };
 
 template <typename T>

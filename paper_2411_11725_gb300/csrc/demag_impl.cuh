@@ -114,10 +114,10 @@ struct XInfo {
     int cell;  // cell index of the row start (Ms map)
     int spec;  // spectrum row start
 };
-__device__ __forceinline__ XInfo x_info(const Geom &g, const FastDiv &nrf, int L, bool cell)
+__device__ __forceinline__ XInfo x_info(const Geom &g, int L, bool cell)
 {
     const int NR = g.N2 * g.N3;
-    const int c = (int)nrf.div((unsigned)L);
+    const int c = (int)g.nrf.div((unsigned)L);
     const int row = L - c * NR;
     const int zz = (int)g.n2f.div((unsigned)row);
     const int yy = row - zz * g.N2;
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
     const int l0 = blockIdx.x * lpb;
     const int nl = min(lpb, nlines - l0);
     if (nl <= 0) return;
-    if (threadIdx.x < nl) info[threadIdx.x] = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), l0 + threadIdx.x, false);
+    if (threadIdx.x < nl) info[threadIdx.x] = x_info(g, l0 + threadIdx.x, false);
     __syncthreads();
     const int N1 = g.N1, row = g.ysn, plane = g.zsn;  // 2D (1D) basis: both z (y and z) corners are the node
     const T *Ms = b.Ms;
@@ -216,7 +216,7 @@ __global__ void k_x_fwd1(Geom g, DemagBufs<T> b, const T *__restrict__ in)
     const int nlines = 3 * g.N2 * g.N3;
     const int L = blockIdx.x * blockDim.x + threadIdx.x;
     if (L >= nlines) return;
-    const XInfo xi = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), L, false);
+    const XInfo xi = x_info(g, L, false);
     const T v = cell_M_pair<T>(in + xi.in, g.ysn, g.zsn, b.Ms, b.Ms0, xi.cell, false).x;
     b.S[xi.spec] = cx<T>(v, T(0));
 }
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kXiThreads<T>, sizeof(T) == 4 ? 16 : 4)
     const int l0 = blockIdx.x * lpb;
     const int nl = min(lpb, nlines - l0);
     if (nl <= 0) return;
-    if (threadIdx.x < nl) info[threadIdx.x] = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), l0 + threadIdx.x, true);
+    if (threadIdx.x < nl) info[threadIdx.x] = x_info(g, l0 + threadIdx.x, true);
     __syncthreads();
     // Z_k = (X_k + conj X_{Q-k}) + i conj(W^k) (X_k - conj X_{Q-k}), k < Q, into shared memory
     const int wsh = g.twlg - (LG + 1);
@@ -305,7 +305,7 @@ __global__ void k_x_inv1(Geom g, DemagBufs<T> b, T *__restrict__ out, T *__restr
     const int nlines = 3 * g.N2 * g.N3;
     const int L = blockIdx.x * blockDim.x + threadIdx.x;
     if (L >= nlines) return;
-    const XInfo xi = x_info(g, FastDiv((unsigned)(g.N2 * g.N3)), L, true);
+    const XInfo xi = x_info(g, L, true);
     T v = b.S[xi.spec].x;
     if (H_out) H_out[xi.in] = v;
     v *= b.Ms ? b.Ms[xi.cell] : b.Ms0;

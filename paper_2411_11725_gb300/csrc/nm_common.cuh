@@ -62,6 +62,7 @@ struct StepCtl {
     int status;      // NM_OK or an NM_ERR_* code set on the device
     int consecutive_rej;
     double rtol, atol;
+    unsigned ticket;  // blocks of the running reduction that have arrived (zero between launches)
 };
 
 // Optional per-launch hook, called after every kernel launch with the kernel's name (profiling).

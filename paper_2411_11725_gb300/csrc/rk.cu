@@ -6,6 +6,8 @@
 namespace nm {
 
 constexpr int kRedThreads = 256;
+// from here on the vector kernels (four nodes per thread) have two blocks for every SM
+constexpr long kVecNodes = 4L * 256 * 2 * 152;
 
 // y = m + dt * sum_j a_j k_j: slope combination in the working precision, addition in FP64
 // (with mf, the FP32 path forms y = fl32(m) + dt * sum in FP32: y is an FP32 quantity either way)
@@ -79,18 +81,112 @@ __device__ __forceinline__ double rsqrt_refined(double s)
     return r0 * (1.5 - 0.5 * s * r0 * r0);
 }
 
-template <typename T>
+// Sum over the block in a fixed order, the same value in every thread; sh holds 33 values.
 __device__ __forceinline__ double block_sum(double v, double *sh)
 {
-    sh[threadIdx.x] = v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if ((threadIdx.x & 31) == 0) sh[w] = v;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+    if (w == 0) {
+        v = (int)threadIdx.x < nw ? sh[threadIdx.x] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (threadIdx.x == 0) sh[32] = v;
     }
-    double r = sh[0];
+    __syncthreads();
+    const double r = sh[32];
     __syncthreads();
     return r;
+}
+
+// err^(-1/5) for err within [1e-4, 1e4]: the FP32 power and two Newton steps in FP64 (relative error 1e-6 ->
+// 1e-12 -> rounding), a dozen operations where the FP64 power takes hundreds at GB300's FP64 rate
+__device__ __forceinline__ double inv_fifth_root(double err)
+{
+    double r = (double)powf((float)err, -0.2f);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const double r2 = r * r;
+        r = r * (1.2 - 0.2 * err * r2 * r2 * r);
+    }
+    return r;
+}
+
+// Step control from s = the sum of the squared error terms (one thread): err = sqrt(s / (3 n_active)); accept
+// when err <= 1; new dt from dt * clamp(0.9 err^(-1/5), 0.2, 5); clipping to t_end; failure after too many
+// rejections.
+__device__ __forceinline__ void dp5_decide(double s, double n_active, StepCtl *ctl, int max_rej)
+{
+    const double err = n_active > 0 ? sqrt(s / (3.0 * n_active)) : 0.0;
+    const bool fin = isfinite(err), acc = fin && err <= 1.0;
+    // (below 1e-4 and above 1e4 the factor is at its bounds)
+    const double fac =
+        !fin || err > 1e4 ? 0.2 : (err < 1e-4 ? 5.0 : fmin(5.0, fmax(0.2, 0.9 * inv_fifth_root(err))));
+    const double dt = ctl->dt;
+    ctl->err = err;
+    ctl->accepted = acc;
+    ctl->dt_used = dt;
+    double t = ctl->t;
+    int rej = ctl->consecutive_rej;
+    if (acc) {
+        t += dt;
+        ctl->t = t;
+        ctl->n_acc += 1;
+        rej = 0;
+    } else {
+        ctl->n_rej += 1;
+        rej += 1;
+    }
+    ctl->consecutive_rej = rej;
+    double dtn = dt * fac;
+    ctl->dt_prop = dtn;
+    const double t_end = ctl->t_end;
+    bool done = false;
+    if (t_end > 0.0) {
+        const double rem = t_end - t;
+        if (rem <= 1e-12 * fmax(fabs(t_end), 1e-30)) done = true;
+        else if (dtn > rem) dtn = rem;
+    }
+    if (rej > max_rej || (!done && dtn < ctl->dt_min)) {
+        ctl->status = NM_ERR_STEP_UNDERFLOW;
+        done = true;
+    }
+    if (done) ctl->done = 1;
+    ctl->dt = dtn;
+}
+
+// End of an error kernel: the block's sum goes to partials, and the block that arrives last adds them up in
+// order and takes the step decision (a launch of its own before: on small meshes it took as long as a pass).
+// Every block has read what it needs of ctl before it arrives.
+__device__ __forceinline__ void dp5_finish(double acc, double *partials, double n_active, StepCtl *ctl, int max_rej,
+                                           double *sh)
+{
+    __shared__ bool last;
+    const double s = block_sum(acc, sh);
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double v = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(partials + i);
+    const double total = block_sum(v, sh);
+    if (threadIdx.x == 0) {
+        ctl->ticket = 0;
+        dp5_decide(total, n_active, ctl, max_rej);
+    }
+}
+// a finished integration: the attempt counts for nothing
+__device__ __forceinline__ bool dp5_idle(StepCtl *ctl)
+{
+    if (!ctl->done) return false;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->accepted = 0;
+    return true;
 }
 
 // Per-block partial sums of ((dt sum_i e_i k_i) / (atol + rtol max(|m|, |m5|)))^2 over magnetic
@@ -99,12 +195,12 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
 template <typename T, bool F64T = false>
 __global__ void __launch_bounds__(kRedThreads) k_dp5_err(long n_nodes, long ns, const double *__restrict__ m,
                                                           KList kb, KList ke, const T *__restrict__ inv_mass,
-                                                          const StepCtl *ctl, double *partials,
-                                                          const float *__restrict__ mf)
+                                                          StepCtl *ctl, double *partials, double n_active,
+                                                          int max_rej, const float *__restrict__ mf)
 {
     pdl_enter();
-    __shared__ double sh[kRedThreads];
-    if (ctl->done) return;
+    __shared__ double sh[33];
+    if (dp5_idle(ctl)) return;
     const double dt = ctl->dt, rtol = ctl->rtol, atol = ctl->atol;
     double acc = 0.0;
     // no early exit per node: all loads of an iteration are independent, so they are in flight together
@@ -160,8 +256,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dp5_err(long n_nodes, long ns, 
         }
         if (sizeof(T) == 4 && magnetic) acc += (double)part;
     }
-    double s = block_sum<T>(acc, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    dp5_finish(acc, partials, n_active, ctl, max_rej, sh);
 }
 
 // FP32 slopes with the FP32 copy of m: the same partial sums with four consecutive nodes per thread and
@@ -182,16 +277,49 @@ __device__ __forceinline__ float dp5_err_term(float m0, float sb, float se, floa
     return q * q;
 }
 
-__global__ void __launch_bounds__(kRedThreads) k_dp5_err_f4(long n_nodes, long ns, KList kb, KList ke,
-                                                             const float *__restrict__ inv_mass, const StepCtl *ctl,
-                                                             double *partials, const float *__restrict__ mf)
+// one node's terms
+__device__ __forceinline__ double dp5_err_node(long n, long ns, const KList &kb, const KList &ke,
+                                               const float *__restrict__ inv_mass, const float *__restrict__ mf,
+                                               float dtf, float rtol, float atol)
+{
+    const bool magnetic = inv_mass[n] > 0.f;
+    float part = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const long i = c * ns + n;
+        float sb = 0.f, se = 0.f, k1 = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (j >= kb.n) break;
+            const float kv = ((const float *)kb.p[j])[i];
+            sb += kb.af[j] * kv;
+            if (j == 0) k1 = kv;
+            else se += ke.af[j] * (kv - k1);
+        }
+        part += dp5_err_term(mf[i], sb, se, dtf, rtol, atol);
+    }
+    return magnetic ? (double)part : 0.0;
+}
+
+// V = 4: four consecutive nodes per thread and load; V = 1: one node, for meshes that four would leave short of
+// threads (kVecNodes)
+template <int V>
+__global__ void __launch_bounds__(kRedThreads) k_dp5_err_v(long n_nodes, long ns, const __grid_constant__ KList kb,
+                                                           const __grid_constant__ KList ke,
+                                                           const float *__restrict__ inv_mass, StepCtl *ctl,
+                                                           double *partials, double n_active, int max_rej,
+                                                           const float *__restrict__ mf)
 {
     pdl_enter();
-    __shared__ double sh[kRedThreads];
-    if (ctl->done) return;
+    __shared__ double sh[33];
+    if (dp5_idle(ctl)) return;
     const float dtf = (float)ctl->dt, rtol = (float)ctl->rtol, atol = (float)ctl->atol;
     double acc = 0.0;
-    const long n4 = n_nodes >> 2;
+    const long n4 = V == 4 ? n_nodes >> 2 : 0;
+    if constexpr (V == 1) {
+        for (long n = blockIdx.x * (long)blockDim.x + threadIdx.x; n < n_nodes; n += (long)gridDim.x * blockDim.x)
+            acc += dp5_err_node(n, ns, kb, ke, inv_mass, mf, dtf, rtol, atol);
+    }
     for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n4; q += (long)gridDim.x * blockDim.x) {
         const float4 im = reinterpret_cast<const float4 *>(inv_mass)[q];
         float4 part = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -221,72 +349,9 @@ __global__ void __launch_bounds__(kRedThreads) k_dp5_err_f4(long n_nodes, long n
                          (im.w > 0.f ? part.w : 0.f);
         acc += (double)s4;
     }
-    if (blockIdx.x == 0 && threadIdx.x < (n_nodes & 3)) {
-        const long n = 4 * n4 + threadIdx.x;
-        float part = 0.f;
-        for (int c = 0; c < 3; ++c) {
-            const long i = c * ns + n;
-            float sb = 0.f, se = 0.f, k1 = 0.f;
-            for (int j = 0; j < 8; ++j) {
-                if (j >= kb.n) break;
-                const float kv = ((const float *)kb.p[j])[i];
-                sb += kb.af[j] * kv;
-                if (j == 0) k1 = kv;
-                else se += ke.af[j] * (kv - k1);
-            }
-            part += dp5_err_term(mf[i], sb, se, dtf, rtol, atol);
-        }
-        if (inv_mass[n] > 0.f) acc += (double)part;
-    }
-    double s = block_sum<float>(acc, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// One block: err = sqrt(sum partials / (3 n_active)); accept when err <= 1; new dt from
-// dt * clamp(0.9 err^(-1/5), 0.2, 5); clipping to t_end; failure after too many rejections.
-__global__ void __launch_bounds__(1024) k_dp5_ctl(const double *partials, int nparts, double n_active, StepCtl *ctl,
-                                                  int max_rej)
-{
-    pdl_enter();
-    __shared__ double sh[1024];
-    if (ctl->done) {
-        if (threadIdx.x == 0) ctl->accepted = 0;
-        return;
-    }
-    double v = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) v += partials[i];
-    double s = block_sum<double>(v, sh);
-    if (threadIdx.x != 0) return;
-    double err = n_active > 0 ? sqrt(s / (3.0 * n_active)) : 0.0;
-    bool fin = isfinite(err);
-    bool acc = fin && err <= 1.0;
-    double fac = !fin ? 0.2 : (err == 0.0 ? 5.0 : fmin(5.0, fmax(0.2, 0.9 * pow(err, -0.2))));
-    ctl->err = err;
-    ctl->accepted = acc;
-    ctl->dt_used = ctl->dt;
-    if (acc) {
-        ctl->t += ctl->dt;
-        ctl->n_acc += 1;
-        ctl->consecutive_rej = 0;
-    } else {
-        ctl->n_rej += 1;
-        ctl->consecutive_rej += 1;
-    }
-    double dtn = ctl->dt * fac;
-    ctl->dt_prop = dtn;
-    if (ctl->t_end > 0.0) {
-        double rem = ctl->t_end - ctl->t;
-        if (rem <= 1e-12 * fmax(fabs(ctl->t_end), 1e-30)) {
-            ctl->done = 1;
-        } else if (dtn > rem) {
-            dtn = rem;
-        }
-    }
-    if (ctl->consecutive_rej > max_rej || (!ctl->done && dtn < ctl->dt_min)) {
-        ctl->status = NM_ERR_STEP_UNDERFLOW;
-        ctl->done = 1;
-    }
-    ctl->dt = dtn;
+    if (V == 4 && blockIdx.x == 0 && threadIdx.x < (n_nodes & 3))
+        acc += dp5_err_node(4 * n4 + threadIdx.x, ns, kb, ke, inv_mass, mf, dtf, rtol, atol);
+    dp5_finish(acc, partials, n_active, ctl, max_rej, sh);
 }
 
 // m + dt * sum_j b_j k_j, optionally renormalised (FP64 result; slope combination in the working
@@ -367,17 +432,20 @@ __device__ __forceinline__ void advance_f32(double v[3], const float d[3], int r
     for (int c = 0; c < 3; ++c) f[c] = d2f_int(v[c]);
 }
 
-// Accepted DP5 step of the FP32 path with the FP32 copy of m: four consecutive nodes per thread
-// (16-byte slope loads, two 16-byte FP64 loads per component); the ragged tail node by node.
-__global__ void k_dp5_update_f4(long n_nodes, long ns, double *__restrict__ m, KList kb, const float *__restrict__ k7,
-                                float *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf)
+// Accepted DP5 step of the FP32 path with the FP32 copy of m: V = 4, four consecutive nodes per thread
+// (16-byte slope loads, two 16-byte FP64 loads per component), the ragged tail node by node; V = 1, one node
+// per thread.
+template <int V>
+__global__ void k_dp5_update_v(long n_nodes, long ns, double *__restrict__ m, const __grid_constant__ KList kb,
+                               const float *__restrict__ k7,
+                               float *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf)
 {
     pdl_enter();
     const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (!ctl->accepted) return;
     const float dtf = (float)ctl->dt_used;
-    const long n4 = n_nodes >> 2;
-    if (q < n4) {
+    const long n4 = V == 4 ? n_nodes >> 2 : 0;
+    if (V == 4 && q < n4) {
         float d[3][4];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -419,13 +487,15 @@ __global__ void k_dp5_update_f4(long n_nodes, long ns, double *__restrict__ m, K
             reinterpret_cast<float4 *>(k1 + c * ns)[q] = reinterpret_cast<const float4 *>(k7 + c * ns)[q];
         }
     }
-    if (q < (n_nodes & 3)) {
+    if (V == 4 ? q < (n_nodes & 3) : q < n_nodes) {
         const long n = 4 * n4 + q;
         double w[3];
         float dd[3], ff[3];
+#pragma unroll
         for (int c = 0; c < 3; ++c) {
             const long i = c * ns + n;
             float sb = 0.f;
+#pragma unroll
             for (int j = 0; j < 8; ++j) {
                 if (j >= kb.n) break;
                 sb += kb.af[j] * ((const float *)kb.p[j])[i];
@@ -464,25 +534,24 @@ __global__ void k_dp5_update(long n_nodes, long ns, double *__restrict__ m, KLis
 
 // RK4 end of step: m <- m + dt/6 (k1 + 2 k2 + 2 k3 + k4), optional renormalisation.
 template <typename T>
-__global__ void k_rk4_update(long n_nodes, long ns, double *__restrict__ m, KList kb, const StepCtl *ctl, int renorm,
+__global__ void k_rk4_update(long n_nodes, long ns, double *__restrict__ m, KList kb, StepCtl *ctl, int renorm,
                              float *__restrict__ mf)
 {
     pdl_enter();
-    long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (n >= n_nodes) return;
     if (ctl->done) return;
-    double v[3];
-    advance_node<T>(n, ns, m, kb, ctl->dt, renorm, v);
-    for (int c = 0; c < 3; ++c) {
-        m[c * ns + n] = v[c];
-        if (mf) mf[c * ns + n] = (float)v[c];
+    const long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (n < n_nodes) {
+        double v[3];
+        advance_node<T>(n, ns, m, kb, ctl->dt, renorm, v);
+        for (int c = 0; c < 3; ++c) {
+            m[c * ns + n] = v[c];
+            if (mf) mf[c * ns + n] = (float)v[c];
+        }
     }
-}
-
-__global__ void k_rk4_advance(StepCtl *ctl)
-{
-    pdl_enter();
-    if (ctl->done) return;
+    // the block that arrives last (every thread of every block has read dt by then) advances the time
+    __syncthreads();
+    if (threadIdx.x != 0 || atomicAdd(&ctl->ticket, 1u) != gridDim.x - 1) return;
+    ctl->ticket = 0;
     ctl->t += ctl->dt;
     ctl->n_acc += 1;
     ctl->accepted = 1;
@@ -500,7 +569,7 @@ __global__ void __launch_bounds__(kRedThreads) k_mean_partials(long n_nodes, lon
                                                                 const T *__restrict__ vol, double *partials)
 {
     pdl_enter();
-    __shared__ double sh[kRedThreads];
+    __shared__ double sh[33];
     double a[4] = {0, 0, 0, 0};
     for (long n = blockIdx.x * (long)blockDim.x + threadIdx.x; n < n_nodes; n += (long)gridDim.x * blockDim.x) {
         double w = (double)vol[n];
@@ -510,7 +579,7 @@ __global__ void __launch_bounds__(kRedThreads) k_mean_partials(long n_nodes, lon
         a[3] += w;
     }
     for (int c = 0; c < 4; ++c) {
-        double s = block_sum<T>(a[c], sh);
+        double s = block_sum(a[c], sh);
         if (threadIdx.x == 0) partials[4 * blockIdx.x + c] = s;
     }
 }
@@ -518,12 +587,11 @@ __global__ void __launch_bounds__(kRedThreads) k_mean_partials(long n_nodes, lon
 __global__ void __launch_bounds__(1024) k_mean_final(const double *partials, int nparts, double *out)
 {
     pdl_enter();
-    __shared__ double sh[1024];
+    __shared__ double sh[33];
     for (int c = 0; c < 4; ++c) {
         double v = 0.0;
         for (int i = threadIdx.x; i < nparts; i += blockDim.x) v += partials[4 * i + c];
-        double s = block_sum<double>(v, sh);
-        if (threadIdx.x == 0) sh[0] = s;
+        double s = block_sum(v, sh);
         if (threadIdx.x == 0) out[c] = s;
         __syncthreads();
     }
@@ -697,24 +765,28 @@ void launch_dp5_control(const Geom &g, const double *m, const KList &kb, const K
                         const float *mf, bool f64_terms)
 {
     // up to 4096 partial sums (the mesh's partials buffer), so that enough loads are in flight
-    long nbl = (g.n_nodes + kRedThreads - 1) / kRedThreads;
+    const long nbl = (g.n_nodes + kRedThreads - 1) / kRedThreads;
     const int nb = (int)(nbl > 4096 ? 4096 : (nbl < 1 ? 1 : nbl));
     if constexpr (sizeof(T) == 4) {
         if (f64_terms) {
             launch_pdl(k_dp5_err<T, true>, nb, kRedThreads, 0, st, g.n_nodes, g.ns, m, fk(kb), fk(ke), inv_mass, ctl,
-                                                           partials, nullptr);
-            launch_pdl(k_dp5_ctl, 1, 1024, 0, st, partials, nb, n_active, ctl, max_rej);
+                       partials, n_active, max_rej, nullptr);
+            return;
+        }
+        if (mf && g.n_nodes < kVecNodes) {
+            launch_pdl(k_dp5_err_v<1>, nb, kRedThreads, 0, st, g.n_nodes, g.ns, fk(kb), fk(ke), (const float *)inv_mass,
+                       ctl, partials, n_active, max_rej, mf);
             return;
         }
         if (mf) {
-            launch_pdl(k_dp5_err_f4, nb, kRedThreads, 0, st, g.n_nodes, g.ns, fk(kb), fk(ke), (const float *)inv_mass, ctl,
-                                                     partials, mf);
-            launch_pdl(k_dp5_ctl, 1, 1024, 0, st, partials, nb, n_active, ctl, max_rej);
+            const int nb4 = div_up(g.n_nodes >> 2, kRedThreads);
+            launch_pdl(k_dp5_err_v<4>, nb4 > 4096 ? 4096 : nb4, kRedThreads, 0, st, g.n_nodes, g.ns, fk(kb), fk(ke),
+                       (const float *)inv_mass, ctl, partials, n_active, max_rej, mf);
             return;
         }
     }
-    launch_pdl(k_dp5_err<T>, nb, kRedThreads, 0, st, g.n_nodes, g.ns, m, fk(kb), fk(ke), inv_mass, ctl, partials, mf);
-    launch_pdl(k_dp5_ctl, 1, 1024, 0, st, partials, nb, n_active, ctl, max_rej);
+    launch_pdl(k_dp5_err<T>, nb, kRedThreads, 0, st, g.n_nodes, g.ns, m, fk(kb), fk(ke), inv_mass, ctl, partials, n_active,
+               max_rej, mf);
 }
 
 template <typename T>
@@ -723,9 +795,12 @@ void launch_dp5_update(const Geom &g, double *m, const KList &kb, const T *k7, T
 {
     if constexpr (sizeof(T) == 4) {
         if (mf) {
-            const long n4 = g.n_nodes >> 2;
-            launch_pdl(k_dp5_update_f4, div_up(n4 > 4 ? n4 : 4, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), (const float *)k7,
-                                                                           (float *)k1, ctl, renorm, mf);
+            if (g.n_nodes < kVecNodes)
+                launch_pdl(k_dp5_update_v<1>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb),
+                           (const float *)k7, (float *)k1, ctl, renorm, mf);
+            else
+                launch_pdl(k_dp5_update_v<4>, div_up(g.n_nodes >> 2, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb),
+                           (const float *)k7, (float *)k1, ctl, renorm, mf);
             return;
         }
     }
@@ -737,7 +812,6 @@ void launch_rk4_update(const Geom &g, double *m, const KList &kb, StepCtl *ctl, 
                        float *mf)
 {
     launch_pdl(k_rk4_update<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), ctl, renorm, mf);
-    launch_pdl(k_rk4_advance, 1, 1, 0, st, ctl);
 }
 
 template <typename T>
