@@ -159,13 +159,11 @@ def algorithmic_bytes(name, stage, n, b, with_maps):
             nk = {2: 1, 3: 2, 4: 3, 5: 4, 6: 4}[stage]
             base += mb * Nn + nk * 3 * b * Nn + 3 * b * Nn
         return base
-    if name == "stage_input":
-        return mb * Nn + 3 * b * Nn + 3 * b * Nn
     if name == "dp5_error_control":
         return mb * Nn + 6 * 3 * b * Nn + b * Nn
     if name == "dp5_update":
-        # m in and out (FP64), b_j k_j (j = 1, 3..6) and k7 in, k1 <- k7 out, FP32 copy of m out
-        return 24 * Nn + 6 * 3 * b * Nn + 24 * Nn + 3 * b * Nn + (3 * b * Nn if b == 4 else 0)
+        # m in and out (FP64), b_j k_j (j = 1, 3..6) and k7 in, k1 <- k7 and the next y_2 out, FP32 copy of m out
+        return 24 * Nn + 6 * 3 * b * Nn + 24 * Nn + 2 * 3 * b * Nn + (3 * b * Nn if b == 4 else 0)
     return 0
 
 

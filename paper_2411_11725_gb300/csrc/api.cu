@@ -609,6 +609,7 @@ extern "C" int nm_set_state(nm_mesh M, const double *m, int where, double t, dou
     CUDA_TRY(cudaMemcpyAsync(M->ctl, h, sizeof(StepCtl), cudaMemcpyHostToDevice, M->st));
     M->state_set = true;
     M->k1_valid = false;
+    M->y2_valid = false;
     M->mf_valid = false;
     return NM_OK;
 }
@@ -630,6 +631,7 @@ int pull_ctl(nm_mesh M)
 }
 int push_ctl(nm_mesh M)
 {
+    M->y2_valid = false;  // (formed with the step size that is replaced here)
     CUDA_TRY(cudaMemcpyAsync(M->ctl, M->hctl, sizeof(StepCtl), cudaMemcpyHostToDevice, M->st));
     return NM_OK;
 }
@@ -757,13 +759,7 @@ static void enqueue_dp5_step(nm_mesh M)
 {
     const LocalParams<T> p = local_params<T>(M, M->terms);
     const Geom &g = M->g;
-    KList k2in{};
-    k2in.p[0] = M->k[0];
-    k2in.a[0] = kDpA[1][0];
-    k2in.n = 1;
-    launch_stage_input<T>(g, M->m, k2in, M->ctl, (T *)M->y[0], M->st, M->mf);  // y_2
-    marker(M)("stage_input");
-    for (int s = 2; s <= 7; ++s) {
+    for (int s = 2; s <= 7; ++s) {  // (y_2 is in place: ensure_y2, or the update of the attempt before)
         const T *ys = (const T *)M->y[s % 2];
         T *yn = s < 7 ? (T *)M->y[(s + 1) % 2] : nullptr;
         enqueue_stage<T>(M, p, s, kDpC[s - 1], ys, yn, s < 7 ? kDpA[s] : nullptr, s < 7 ? s : 0);
@@ -781,7 +777,8 @@ static void enqueue_dp5_step(nm_mesh M)
     marker(M)("dp5_error_control");
     KList ku = kb;
     ku.n = 5;  // b7 = 0
-    launch_dp5_update<T>(g, M->m, ku, (const T *)M->k[6], (T *)M->k[0], M->ctl, M->renorm, M->st, M->mf);
+    launch_dp5_update<T>(g, M->m, ku, (const T *)M->k[6], (T *)M->k[0], M->ctl, M->renorm, M->st, M->mf, (T *)M->y[0],
+                         kDpA[1][0]);
     marker(M)("dp5_update");
 }
 
@@ -838,6 +835,7 @@ int launch_step(nm_mesh M, int method)
             return fail(NM_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
         }
     }
+    if ((rc0 = ensure_y2(M, method))) return rc0;
     CUDA_TRY(cudaGraphLaunch(gx, M->st));
     return NM_OK;
 }
@@ -851,6 +849,33 @@ int ensure_k1(nm_mesh M, int method)
     else enqueue_k1<float>(M);
     CHECK_LAUNCH();
     M->k1_valid = true;
+    M->y2_valid = false;
+    return NM_OK;
+}
+
+template <typename T>
+static void enqueue_y2(nm_mesh M)
+{
+    KList k2in{};
+    k2in.p[0] = M->k[0];
+    k2in.a[0] = kDpA[1][0];
+    k2in.n = 1;
+    launch_stage_input<T>(M->g, M->m, k2in, M->ctl, (T *)M->y[0], M->st, M->mf);
+}
+
+// The update of every Dormand-Prince attempt leaves the next one's y_2, so this launches only for the first attempt
+// after the host changed the state or the step control (and before every attempt of the adjoint's forward run).
+int ensure_y2(nm_mesh M, int method)
+{
+    if (method != NM_DP54) {
+        M->y2_valid = false;  // (RK4 stages use the buffer)
+        return NM_OK;
+    }
+    if (M->y2_valid) return NM_OK;
+    if (M->prec == NM_F64) enqueue_y2<double>(M);
+    else enqueue_y2<float>(M);
+    CHECK_LAUNCH();
+    M->y2_valid = true;
     return NM_OK;
 }
 
@@ -1031,6 +1056,7 @@ extern "C" int nm_profile_step(nm_mesh M, int method, int reps, double rtol, dou
     cudaEvent_t start;
     CUDA_TRY(cudaEventCreate(&start));
     for (int r = 0; r < reps; ++r) {
+        if ((rc = ensure_y2(M, method))) { cudaEventDestroy(start); return rc; }
         M->prof_on = true;
         M->prof_n = 0;
         cudaEventRecord(start, M->st);

@@ -89,6 +89,7 @@ struct nm_mesh_s {
     double hu[3] = {0, 0, 0}, hu_freq = 0, hu_phase = 0, hc_freq = 0, hc_phase = 0;
     bool has_hcell = false;
     bool material_set = false, state_set = false, k1_valid = false;
+    bool y2_valid = false;   // y[0] holds the first stage input of the next Dormand-Prince attempt
     unsigned terms = NM_ALL;
     int renorm = 1;
     double dt_min = 1e-22;
@@ -127,6 +128,7 @@ int check_step_args(nm_mesh M, int method, double rtol, double atol);
 int launch_step(nm_mesh M, int method);  // one step attempt of the captured step graph
 int ensure_mf(nm_mesh M);                // refresh the FP32 copy of m if m changed outside the steps
 int ensure_k1(nm_mesh M, int method);    // FSAL slope at the resident state when not valid
+int ensure_y2(nm_mesh M, int method);    // first stage input of a Dormand-Prince attempt when not valid
 
 // device buffer owned by the mesh (freed with it)
 inline int alloc_extra(nm_mesh M, void **p, size_t bytes)

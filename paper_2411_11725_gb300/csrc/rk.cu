@@ -434,17 +434,41 @@ __device__ __forceinline__ void advance_f32(double v[3], const float d[3], int r
 
 // Accepted DP5 step of the FP32 path with the FP32 copy of m: V = 4, four consecutive nodes per thread
 // (16-byte slope loads, two 16-byte FP64 loads per component), the ragged tail node by node; V = 1, one node
-// per thread.
+// per thread.  Accepted or not, y2 is the first stage input of the next attempt (m + dt a21 k1 with the new dt),
+// which a launch of its own formed before.
 template <int V>
 __global__ void k_dp5_update_v(long n_nodes, long ns, double *__restrict__ m, const __grid_constant__ KList kb,
                                const float *__restrict__ k7,
-                               float *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf)
+                               float *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf,
+                               float *__restrict__ y2, float a21)
 {
     pdl_enter();
     const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (!ctl->accepted) return;
-    const float dtf = (float)ctl->dt_used;
+    const bool accepted = ctl->accepted;
+    if (!accepted && ctl->done) return;
+    const float dtf = (float)ctl->dt_used, dt2 = (float)ctl->dt;
     const long n4 = V == 4 ? n_nodes >> 2 : 0;
+    if (!accepted) {
+        // the next attempt from the same state and slope
+        if (V == 4 && q < n4) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float4 f = reinterpret_cast<const float4 *>(mf + c * ns)[q];
+                const float4 k = reinterpret_cast<const float4 *>(k1 + c * ns)[q];
+                reinterpret_cast<float4 *>(y2 + c * ns)[q] =
+                    make_float4(f.x + dt2 * (a21 * k.x), f.y + dt2 * (a21 * k.y), f.z + dt2 * (a21 * k.z),
+                                f.w + dt2 * (a21 * k.w));
+            }
+        }
+        if (V == 4 ? q < (n_nodes & 3) : q < n_nodes) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const long i = c * ns + 4 * n4 + q;
+                y2[i] = mf[i] + dt2 * (a21 * k1[i]);
+            }
+        }
+        return;
+    }
     if (V == 4 && q < n4) {
         float d[3][4];
 #pragma unroll
@@ -484,7 +508,11 @@ __global__ void k_dp5_update_v(long n_nodes, long ns, double *__restrict__ m, co
             reinterpret_cast<double2 *>(m + c * ns)[2 * q] = make_double2(v[c][0], v[c][1]);
             reinterpret_cast<double2 *>(m + c * ns)[2 * q + 1] = make_double2(v[c][2], v[c][3]);
             reinterpret_cast<float4 *>(mf + c * ns)[q] = make_float4(f[c][0], f[c][1], f[c][2], f[c][3]);
-            reinterpret_cast<float4 *>(k1 + c * ns)[q] = reinterpret_cast<const float4 *>(k7 + c * ns)[q];
+            const float4 k = reinterpret_cast<const float4 *>(k7 + c * ns)[q];
+            reinterpret_cast<float4 *>(k1 + c * ns)[q] = k;
+            reinterpret_cast<float4 *>(y2 + c * ns)[q] =
+                make_float4(f[c][0] + dt2 * (a21 * k.x), f[c][1] + dt2 * (a21 * k.y), f[c][2] + dt2 * (a21 * k.z),
+                            f[c][3] + dt2 * (a21 * k.w));
         }
     }
     if (V == 4 ? q < (n_nodes & 3) : q < n_nodes) {
@@ -506,29 +534,37 @@ __global__ void k_dp5_update_v(long n_nodes, long ns, double *__restrict__ m, co
         advance_f32(w, dd, renorm, ff);
         for (int c = 0; c < 3; ++c) {
             const long i = c * ns + n;
+            const float k = k7[i];
             m[i] = w[c];
             mf[i] = ff[c];
-            k1[i] = k7[i];
+            k1[i] = k;
+            y2[i] = ff[c] + dt2 * (a21 * k);
         }
     }
 }
 
-// Accepted step: m <- m5 (optionally renormalised), k1 <- k7 (FSAL).  Rejected: nothing.
+// Accepted step: m <- m5 (optionally renormalised), k1 <- k7 (FSAL).  Either way y2 <- m + dt a21 k1 with the
+// next attempt's dt.
 template <typename T>
 __global__ void k_dp5_update(long n_nodes, long ns, double *__restrict__ m, KList kb, const T *__restrict__ k7,
-                             T *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf)
+                             T *__restrict__ k1, const StepCtl *ctl, int renorm, T *__restrict__ y2, T a21)
 {
     pdl_enter();
     long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (n >= n_nodes) return;
-    if (!ctl->accepted) return;
+    const bool accepted = ctl->accepted;
+    if (!accepted && ctl->done) return;
+    const double dt2 = ctl->dt;
     double v[3];
-    advance_node<T>(n, ns, m, kb, ctl->dt_used, renorm, v);
+    if (accepted) advance_node<T>(n, ns, m, kb, ctl->dt_used, renorm, v);
     for (int c = 0; c < 3; ++c) {
-        long i = c * ns + n;
-        m[i] = v[c];
-        if (mf) mf[i] = (float)v[c];
-        k1[i] = k7[i];
+        const long i = c * ns + n;
+        const T k = accepted ? k7[i] : k1[i];
+        if (accepted) {
+            m[i] = v[c];
+            k1[i] = k;
+        }
+        y2[i] = (T)((accepted ? v[c] : m[i]) + dt2 * (double)(a21 * k));
     }
 }
 
@@ -791,20 +827,21 @@ void launch_dp5_control(const Geom &g, const double *m, const KList &kb, const K
 
 template <typename T>
 void launch_dp5_update(const Geom &g, double *m, const KList &kb, const T *k7, T *k1, const StepCtl *ctl, int renorm,
-                       cudaStream_t st, float *mf)
+                       cudaStream_t st, float *mf, T *y2, double a21)
 {
     if constexpr (sizeof(T) == 4) {
         if (mf) {
             if (g.n_nodes < kVecNodes)
-                launch_pdl(k_dp5_update_v<1>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb),
-                           (const float *)k7, (float *)k1, ctl, renorm, mf);
+                launch_pdl(k_dp5_update_v<1>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1, ctl,
+                           renorm, mf, y2, (float)a21);
             else
-                launch_pdl(k_dp5_update_v<4>, div_up(g.n_nodes >> 2, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb),
-                           (const float *)k7, (float *)k1, ctl, renorm, mf);
+                launch_pdl(k_dp5_update_v<4>, div_up(g.n_nodes >> 2, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1,
+                           ctl, renorm, mf, y2, (float)a21);
             return;
         }
     }
-    launch_pdl(k_dp5_update<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1, ctl, renorm, mf);
+    launch_pdl(k_dp5_update<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1, ctl, renorm, y2,
+               (T)a21);
 }
 
 template <typename T>
@@ -861,7 +898,7 @@ void launch_node_volume(const Geom &g, const double *Ms, double Ms0, double V, T
     template void launch_dp5_control<T>(const Geom &, const double *, const KList &, const KList &, const T *,   \
                                         StepCtl *, double *, double, int, cudaStream_t, const float *, bool);                 \
     template void launch_dp5_update<T>(const Geom &, double *, const KList &, const T *, T *, const StepCtl *,  \
-                                       int, cudaStream_t, float *);                                                     \
+                                       int, cudaStream_t, float *, T *, double);                                                     \
     template void launch_rk4_update<T>(const Geom &, double *, const KList &, StepCtl *, int, cudaStream_t, float *);    \
     template void launch_mean<T>(const Geom &, const double *, const T *, double *, double *, cudaStream_t);     \
     template void launch_cells_to_internal<T>(const Geom &, const double *, int, double, const double *, T *,  \

@@ -33,9 +33,10 @@ template <typename T>
 void launch_dp5_control(const Geom &g, const double *m, const KList &kb, const KList &ke, const T *inv_mass,
                         StepCtl *ctl, double *partials, double n_active, int max_rej, cudaStream_t st,
                         const float *mf = nullptr, bool f64_terms = false);
+// end of a Dormand-Prince attempt; y2 = m + dt a21 k1 of the next one
 template <typename T>
 void launch_dp5_update(const Geom &g, double *m, const KList &kb, const T *k7, T *k1, const StepCtl *ctl, int renorm,
-                       cudaStream_t st, float *mf = nullptr);
+                       cudaStream_t st, float *mf, T *y2, double a21);
 template <typename T>
 void launch_rk4_update(const Geom &g, double *m, const KList &kb, StepCtl *ctl, int renorm, cudaStream_t st,
                        float *mf = nullptr);
