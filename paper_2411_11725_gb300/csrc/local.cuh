@@ -4,14 +4,14 @@
 
 namespace nm {
 
-// Per-mesh constants of the local terms.  The cell-local exchange and consistent-mass integrals of
-// the trilinear basis depend only on d = |i - i'| per direction (bit 2: direction 1, bit 1:
-// direction 2, bit 0: direction 3), so 8 numbers per term describe the 24x24 element matrices.
+// Per-mesh constants of the local terms.  The element integrals are tensor products of one-dimensional 2 x 2
+// stiffness and mass matrices; they depend only on d = |i - i'| per direction.
 template <typename T>
 struct LocalParams {
     Geom g;
-    T Wex[8];          // int_cell 2 grad(phi_i).grad(phi_i') for the pattern d (per unit A)
-    T Wm[8];           // int_cell phi_i phi_i' for the pattern d
+    // trilinear basis, by in-plane pattern d = 2 |o1| + |o2| (node_maps.cu): -2 (K1 M2 + M1 K2) dz/6 and
+    // -2 M1 M2 / dz per unit A, 2 M1 M2 dz/6 per unit Ku
+    T mP[4], mZ[4], mK[4];
     // Uniform material (no cell maps, Ms0 > 0; trilinear basis): node_uniform.cu.  2 A and 2 Ku (0 for terms
     // that are off) times the constants of the one-dimensional element matrices, and 1 / (mu0 V/8 Ms0).
     int uniform;
@@ -76,6 +76,13 @@ void launch_heff_uniform(const LocalParams<T> &p, const T *y, T *h_out, double t
 template <typename T>
 void launch_llg_stage_uniform(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa,
                               cudaStream_t st);
+
+// the same for cell maps on the trilinear basis
+template <typename T>
+void launch_heff_maps(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaStream_t st);
+template <typename T>
+void launch_llg_stage_maps(const LocalParams<T> &p, const T *y, T *k_out, T *y_next, const StageArgs &sa,
+                           cudaStream_t st);
 
 // lumped mass: inv_mass_n = 1 / (mu0 V/8 sum_{c∋n} Ms_c); counts magnetic nodes into *n_active (device)
 template <typename T>

@@ -170,18 +170,13 @@ inline LocalParams<T> local_params(nm_mesh M, unsigned terms)
     p.g = M->g;
     const double *dx = M->dx;
     const double V = dx[0] * dx[1] * dx[2];
-    for (int d = 0; d < 8; ++d) {
-        const int dd[3] = {(d >> 2) & 1, (d >> 1) & 1, d & 1};
-        double kk = 0.0, mm = V;
-        for (int k = 0; k < 3; ++k) mm *= dd[k] ? 1.0 / 6.0 : 1.0 / 3.0;
-        for (int k = 0; k < 3; ++k) {
-            double v = (dd[k] ? -1.0 : 1.0) / dx[k];
-            for (int l = 0; l < 3; ++l)
-                if (l != k) v *= dx[l] * (dd[l] ? 1.0 / 6.0 : 1.0 / 3.0);
-            kk += v;
-        }
-        p.Wex[d] = (T)(2.0 * kk);
-        p.Wm[d] = (T)mm;
+    for (int d = 0; d < 4; ++d) {
+        const int d1 = (d >> 1) & 1, d2 = d & 1;
+        const double M1x = dx[0] * (d1 ? 1.0 / 6.0 : 1.0 / 3.0), M1y = dx[1] * (d2 ? 1.0 / 6.0 : 1.0 / 3.0);
+        const double K1x = (d1 ? -1.0 : 1.0) / dx[0], K1y = (d2 ? -1.0 : 1.0) / dx[1];
+        p.mP[d] = (T)(-2.0 * (K1x * M1y + M1x * K1y) * dx[2] / 6.0);
+        p.mZ[d] = (T)(-2.0 * M1x * M1y / dx[2]);
+        p.mK[d] = (T)(2.0 * M1x * M1y * dx[2] / 6.0);
     }
     p.mu0V8 = (T)(kMu0 * V / 8.0);
     p.mu0V4 = (T)(kMu0 * V / 4.0);

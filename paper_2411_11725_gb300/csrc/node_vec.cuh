@@ -1,0 +1,313 @@
+// Shared parts of the node kernels: 3-vectors, rotating planes in shared memory, arguments, outputs and the split of
+// their walk along z.
+#pragma once
+#include <type_traits>
+
+#include "local.cuh"
+
+namespace nm {
+
+// tile of nodes walked along z by one block
+constexpr int kUX = 32, kUY = 4, kUThreads = kUX * kUY;
+
+// A 3-vector of the working precision.  FP32: x and y as one packed pair (fma.rn.f32x2: one instruction for
+// both, rounded as the scalar ones) and z apart, the layout of the shared planes.
+template <typename T>
+struct Vec {
+    T x, y, z;
+};
+template <>
+struct Vec<float> {
+    unsigned long long xy;
+    float z;
+};
+__device__ __forceinline__ unsigned long long pk(float a, float b)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpk(unsigned long long r, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> vadd(const Vec<T> &a, const Vec<T> &b)
+{
+    if constexpr (sizeof(T) == 4) {
+        Vec<float> r;
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.xy) : "l"(a.xy), "l"(b.xy));
+        r.z = a.z + b.z;
+        return r;
+    } else {
+        return Vec<T>{a.x + b.x, a.y + b.y, a.z + b.z};
+    }
+}
+// c v + w
+template <typename T>
+__device__ __forceinline__ Vec<T> vfma(T c, const Vec<T> &v, const Vec<T> &w)
+{
+    if constexpr (sizeof(T) == 4) {
+        Vec<float> r;
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.xy) : "l"(pk(c, c)), "l"(v.xy), "l"(w.xy));
+        r.z = fmaf(c, v.z, w.z);
+        return r;
+    } else {
+        return Vec<T>{fma(c, v.x, w.x), fma(c, v.y, w.y), fma(c, v.z, w.z)};
+    }
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> vmul(T c, const Vec<T> &v)
+{
+    if constexpr (sizeof(T) == 4) {
+        Vec<float> r;
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.xy) : "l"(pk(c, c)), "l"(v.xy));
+        r.z = c * v.z;
+        return r;
+    } else {
+        return Vec<T>{c * v.x, c * v.y, c * v.z};
+    }
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> vsub(const Vec<T> &a, const Vec<T> &b)
+{
+    if constexpr (sizeof(T) == 4) {
+        Vec<float> r;
+        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.xy) : "l"(a.xy), "l"(b.xy));
+        r.z = a.z - b.z;
+        return r;
+    } else {
+        return Vec<T>{a.x - b.x, a.y - b.y, a.z - b.z};
+    }
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> vzero()
+{
+    if constexpr (sizeof(T) == 4) return Vec<float>{0ull, 0.f};
+    else return Vec<T>{T(0), T(0), T(0)};
+}
+template <typename T>
+__device__ __forceinline__ void vget(const Vec<T> &v, T &x, T &y, T &z)
+{
+    if constexpr (sizeof(T) == 4) {
+        unpk(v.xy, x, y);
+        z = v.z;
+    } else {
+        x = v.x;
+        y = v.y;
+        z = v.z;
+    }
+}
+
+// NS planes of R x C 3-vectors in shared memory
+template <typename T, int R, int C, int NS>
+struct VPlanes {
+    T v[NS][R * C][3];
+    __device__ __forceinline__ Vec<T> get(int s, int i) const { return Vec<T>{v[s][i][0], v[s][i][1], v[s][i][2]}; }
+    __device__ __forceinline__ T *p(int s, int i, int c) { return &v[s][i][c]; }
+};
+template <int R, int C, int NS>
+struct VPlanes<float, R, C, NS> {
+    unsigned long long xy[NS][R * C];
+    float z[NS][R * C];
+    __device__ __forceinline__ Vec<float> get(int s, int i) const { return Vec<float>{xy[s][i], z[s][i]}; }
+    __device__ __forceinline__ float *p(int s, int i, int c)
+    {
+        return c == 2 ? &z[s][i] : reinterpret_cast<float *>(&xy[s][i]) + c;
+    }
+};
+
+template <typename T>
+struct NodeUArgs {
+    int nn1, nn2, nn3, N1, N2, N3, ns, cs;
+    int bxn, full, chunks, zc;  // blocks b < full walk tile b over all planes; the other tiles are split into
+                                // `chunks` blocks of zc planes
+    T cx, cy, cz, can;          // 2 A x element constants of the axes; 2 Ku V / 216 (2D basis: / 36 per layer)
+    T e0, e1, e2;
+    T im1, mu0V8;               // 1 / (mu0 V/8 Ms), mu0 V/8 (2D basis: 1 / (mu0 V/4 Ms N3), mu0 V/4)
+    T gam, alpha;
+    const T *y, *MsH, *Msh, *hdmi;
+    T *out, *y_next;
+    const double *m;
+    const float *mf;
+    const T *k[4];              // earlier slopes with non-zero coefficients in the next stage input
+    T a[4], as;                 // their coefficients, and that of the slope being written
+    const StepCtl *ctl;
+    double c_s, t_fixed, hu0, hu1, hu2, hu_freq, hu_phase, hc_freq, hc_phase;
+    int raw, zee, nk;
+};
+
+template <typename T>
+__device__ __forceinline__ double u_time_factor(double f, double ph, double t)
+{
+    return f == 0.0 ? 1.0 : sin(2.0 * 3.14159265358979323846 * f * t + ph);
+}
+
+// asynchronous copy of one value, or zero fill when !in
+template <typename T>
+__device__ __forceinline__ void cp_elem(T *dst, const T *src, bool in)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = in ? (int)sizeof(T) : 0;
+    if (sizeof(T) == 4)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+// What a kernel instance writes: the field (kHeff), the slope (kSlope), or the slope and the next stage input
+// formed from NK >= 0 earlier slopes.  M64: the next input is formed from the FP64 m (always in FP64, and in
+// FP32 where no FP32 copy of m is kept).
+constexpr int kHeff = -2, kSlope = -1;
+
+// The node's output from its field: H itself, or the LLG slope k (zero without magnetic material) and the next
+// stage input
+template <typename T, int NK, bool M64>
+__device__ __forceinline__ void node_u_out(const NodeUArgs<T> &p, int n, T hx, T hy, T hz, T mx, T my, T mz, T dt,
+                                           double dt64, bool magnetic = true)
+{
+    if (NK == kHeff) {
+        p.out[n] = hx;
+        p.out[p.ns + n] = hy;
+        p.out[2 * p.ns + n] = hz;
+    } else {
+        // the next stage input's own values, all loads issued together
+        T kv[NK > 0 ? NK : 1][3], m0[3];
+        double md[3];
+        if (NK >= 0) {
+#pragma unroll
+            for (int i = 0; i < NK; ++i)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) kv[i][c] = p.k[i][c * p.ns + n];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (M64) md[c] = p.m[c * p.ns + n];
+                else m0[c] = (T)p.mf[c * p.ns + n];
+            }
+        }
+        // k = -gamma' (m x H + alpha m x (m x H))
+        const T ax = my * hz - mz * hy, ay = mz * hx - mx * hz, az = mx * hy - my * hx;
+        const T bx = my * az - mz * ay, by = mz * ax - mx * az, bz = mx * ay - my * ax;
+        T kk[3];
+        kk[0] = -p.gam * (ax + p.alpha * bx);
+        kk[1] = -p.gam * (ay + p.alpha * by);
+        kk[2] = -p.gam * (az + p.alpha * bz);
+        if (!magnetic) kk[0] = kk[1] = kk[2] = T(0);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) p.out[c * p.ns + n] = kk[c];
+        if (NK >= 0) {
+            // y_{s+1} = m + dt sum_j a_j k_j, the slope combination in the working precision
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                T sum = 0;
+#pragma unroll
+                for (int i = 0; i < NK; ++i) sum += p.a[i] * kv[i][c];
+                sum += p.as * kk[c];
+                p.y_next[c * p.ns + n] = M64 ? (T)(md[c] + dt64 * (double)sum) : m0[c] + dt * sum;
+            }
+        }
+    }
+}
+
+// the arguments that both node kernels take from the mesh, the stage and the evaluation time
+template <typename T>
+inline NodeUArgs<T> node_u_args(const LocalParams<T> &p, const T *y, T *out, T *y_next, const StageArgs *sa, double t)
+{
+    const Geom &g = p.g;
+    NodeUArgs<T> a{};
+    a.nn1 = g.nn1; a.nn2 = g.nn2; a.nn3 = g.nn3;
+    a.N1 = g.N1; a.N2 = g.N2; a.N3 = g.N3;
+    a.ns = (int)g.ns;
+    a.cs = (int)g.cs;
+    a.e0 = p.e0; a.e1 = p.e1; a.e2 = p.e2;
+    a.mu0V8 = g.basis == 3 ? p.mu0V8 : p.mu0V4;
+    a.gam = p.gam_t;
+    a.alpha = p.alpha_t;
+    a.y = y;
+    a.MsH = (p.terms & NM_DEMAG) ? p.MsH : nullptr;
+    a.Msh = p.Msh;
+    a.hdmi = p.hdmi;
+    a.out = out;
+    a.y_next = y_next;
+    a.hu0 = p.hu0; a.hu1 = p.hu1; a.hu2 = p.hu2;
+    a.hu_freq = p.hu_freq; a.hu_phase = p.hu_phase;
+    a.hc_freq = p.hc_freq; a.hc_phase = p.hc_phase;
+    a.raw = p.raw;
+    a.zee = (p.terms & NM_ZEE) != 0;
+    a.t_fixed = t;
+    if (!sa) return a;
+    a.ctl = sa->ctl;
+    a.c_s = sa->c_s;
+    a.t_fixed = sa->t_fixed;
+    if (!y_next) return a;
+    a.m = sa->m;
+    a.mf = sa->mf;
+    a.as = sizeof(T) == 4 ? (T)sa->af_s : (T)sa->a_s;
+    for (int j = 0; j + 1 < sa->s && j < 7; ++j) {
+        const T c = sizeof(T) == 4 ? (T)sa->af[j] : (T)sa->a[j];
+        if (c == T(0)) continue;
+        a.k[a.nk] = (const T *)sa->k[j];
+        a.a[a.nk] = c;
+        ++a.nk;
+    }
+    return a;
+}
+
+// go(NK, M64) with the instance that the arguments need
+template <typename T, typename F>
+inline void node_u_dispatch(const NodeUArgs<T> &a, bool stage, F &&go)
+{
+    if (!stage) return go(std::integral_constant<int, kHeff>{}, std::true_type{});
+    if (!a.y_next) return go(std::integral_constant<int, kSlope>{}, std::true_type{});
+    auto slopes = [&](auto n) {
+        if constexpr (sizeof(T) == 4) {
+            if (a.mf) return go(n, std::false_type{});
+        }
+        go(n, std::true_type{});
+    };
+    switch (a.nk) {
+    case 0: return slopes(std::integral_constant<int, 0>{});
+    case 1: return slopes(std::integral_constant<int, 1>{});
+    case 2: return slopes(std::integral_constant<int, 2>{});
+    case 3: return slopes(std::integral_constant<int, 3>{});
+    default: return slopes(std::integral_constant<int, 4>{});
+    }
+}
+
+// Split of the walk: cost in plane units of a grid whose tiles are cut into `chunks` pieces, from the latency
+// of one block (its planes, two more for the halo, and the start of the walk) and the planes an SM works
+// through when the blocks are dealt out evenly (about four planes of one block cost an SM as much time as the
+// latency of one).
+inline void node_u_grid(int nn1, int nn2, int nn3, int *bxn, int *full, int *chunks, int *zc, int *blocks)
+{
+    static int sm_count = 0;
+    if (sm_count == 0) {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        sm_count = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 152;
+    }
+    const int sms = sm_count;
+    *bxn = div_up(nn1, kUX);
+    const int tiles = *bxn * div_up(nn2, kUY);
+    double best = 1e300;
+    for (int f = 0; f < 2; ++f) {
+        const int fl = f ? tiles - tiles % sms : 0, rest = tiles - fl;
+        if (f && fl == 0) break;
+        for (int c = 1; c <= nn3; ++c) {
+            const int z = div_up(nn3, c), ch = div_up(nn3, z);
+            if (c > 1 && ch != c) continue;  // (the same split as fewer chunks)
+            const double work = (double)(fl / sms) * (nn3 + 2) + div_up((long)rest * ch, sms) * (double)(z + 2);
+            const double lat = 4.0 * ((fl ? nn3 : z) + 4);
+            const double cost = work > lat ? work : lat;
+            if (cost < best * 0.999) {
+                best = cost;
+                *full = fl;
+                *zc = z;
+                *chunks = ch;
+                *blocks = fl + rest * ch;
+            }
+        }
+    }
+}
+
+}  // namespace nm
