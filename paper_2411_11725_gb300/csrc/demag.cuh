@@ -49,6 +49,7 @@ struct DemagBufs {
 // Launch shapes of the passes (lines per block bounded by the FFT engine's 16 values per thread).
 struct DemagPlan {
     bool ok;  // the grid fits the engine's per-block budget in this precision
+    int x_ept;                 // x passes: values per thread
     int x_lpb, x_threads;      // forward x pass
     size_t x_smem;
     int xi_lpb, xi_threads;    // inverse x pass

@@ -33,9 +33,11 @@ template <typename T, int LG = 0>
 constexpr int kMaxThreads = 512;
 template <typename T, int LG = 0>
 constexpr int kMinBlocks = sizeof(T) == 4 ? 2 : 1;
-// values per thread per FFT stage in the y passes: radix-16 stages for the long FP32 lines
+// values per thread per FFT stage in the y passes: radix-16 stages for the FP32 lengths where they save a stage
+// (2^10 and 2^11; 2^7 and 2^8: 12.3 against 14.8 us a pass at 512x100x8, 14.0 / 17.7 at 1000x60x12, 8.3 / 9.4 at
+// 131x67x5)
 template <typename T, int LG>
-constexpr int kYEpt = (sizeof(T) == 4 && LG >= 10) ? 16 : 8;
+constexpr int kYEpt = (sizeof(T) == 4 && (LG >= 10 || LG == 7 || LG == 8)) ? 16 : 8;
 constexpr int pow2_floor_c(int v)
 {
     int p = 1;
@@ -78,9 +80,21 @@ struct YTile {
     static_assert(TILE_BYTES % 8 == 0, "barrier alignment");
 };
 
-// x passes: radix-16 stages for FP32 lines of 2^10 complex values
-template <typename T, int LG>
-constexpr int kXEpt = (sizeof(T) == 4 && LG >= 10) ? 16 : 8;
+// x passes, values per thread: radix-16 stages (16) for FP32 lines of 2^10 complex values, and for those of 2^7 and 2^8,
+// where they save a stage, once the lines fill the GPU with half the threads (kXWide threads or more).  Steps: 256x256x8
+// (98k threads) 515 -> 491 us, but 256x256x4 (49k) 285 -> 300, 128x128x16 (49k) 292 -> 303, 200x50x1 (2k) 125 -> 152.
+constexpr long kXWide = 152 * 512;
+template <typename T>
+constexpr bool x_ept_choice(int LG)
+{
+    return sizeof(T) == 4 && (LG == 7 || LG == 8);
+}
+template <typename T>
+static int x_ept(const Geom &g)
+{
+    if (sizeof(T) == 4 && g.lgQ >= 10) return 16;
+    return x_ept_choice<T>(g.lgQ) && 3L * g.N2 * g.N3 * g.Q / 16 >= kXWide ? 16 : 8;
+}
 
 // Asynchronous global -> shared copies (cp.async): many in flight per thread without registers.
 __device__ __forceinline__ void cpa16(void *sm, const void *gm)
@@ -150,7 +164,7 @@ __device__ __forceinline__ Cx<T> cell_M_pair(const T *__restrict__ p, int row, i
 
 // Pass 1: x transform (R2C of length P1 = 2Q via a complex FFT of length Q = 2^LG on even/odd pairs).
 // One block holds `lpb` consecutive lines.
-template <typename T, int LG>
+template <typename T, int LG, int EPT>
 __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
     k_x_fwd(Geom g, DemagBufs<T> b, const T *__restrict__ in, int lpb)
 {
@@ -175,7 +189,7 @@ __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 8 : 4)
         const T *p = in + xi.in + x;
         return cell_M_pair<T>(p, row, plane, Ms, Ms0, xi.cell + x, x + 1 < N1);
     };
-    f3::fft<T, LG, -1, false, false, true, kXEpt<T, LG>>(buf, nl, FastDiv(1u), b.tw, g.twlg, (N1 + 1) >> 1, Q, src,
+    f3::fft<T, LG, -1, false, false, true, EPT>(buf, nl, FastDiv(1u), b.tw, g.twlg, (N1 + 1) >> 1, Q, src,
                                                          f3::NoFn<T>());
     // X_k = (Z_k + conj Z_{Q-k})/2 - (i/2) W^k (Z_k - conj Z_{Q-k}),  W = e^{-2 pi i / P1},  k = 0..Q;
     // thread (l, k) with k < Q/2 writes X_k and X_{Q-k}; k = 0 also writes X_{Q/2} (and X_0, X_Q)
@@ -223,7 +237,7 @@ __global__ void k_x_fwd1(Geom g, DemagBufs<T> b, const T *__restrict__ in)
 
 // Pass 5: inverse x transform (C2R of length P1 via a complex FFT of length Q), keeping x < N1.
 // Output per cell: Ms_c H_c and, when H is not NULL, H_c itself there.
-template <typename T, int LG>
+template <typename T, int LG, int EPT>
 __global__ void __launch_bounds__(kXiThreads<T>, sizeof(T) == 4 ? 16 : 4)
     k_x_inv(Geom g, DemagBufs<T> b, T *__restrict__ out, T *__restrict__ H_out, int lpb)
 {
@@ -294,7 +308,7 @@ __global__ void __launch_bounds__(kXiThreads<T>, sizeof(T) == 4 ? 16 : 4)
         out[xi.in + x] = v0;
         if (x + 1 < N1) out[xi.in + x + 1] = v1;
     };
-    f3::fft<T, LG, +1, false, true, false, kXEpt<T, LG>>(buf, nl, FastDiv(1u), b.tw, g.twlg, Q, (N1 + 1) >> 1, f3::NoFn<T>(), dst);
+    f3::fft<T, LG, +1, false, true, false, EPT>(buf, nl, FastDiv(1u), b.tw, g.twlg, Q, (N1 + 1) >> 1, f3::NoFn<T>(), dst);
 }
 
 template <typename T>
@@ -1068,8 +1082,13 @@ static void init_attributes_t()
 {
     f3::lg_for_each<1, 10>([&](auto c) {
         constexpr int LG = decltype(c)::value;
-        set_smem((const void *)k_x_fwd<T, LG>);
-        set_smem((const void *)k_x_inv<T, LG>);
+        constexpr int E = sizeof(T) == 4 && LG >= 10 ? 16 : 8;
+        set_smem((const void *)k_x_fwd<T, LG, E>);
+        set_smem((const void *)k_x_inv<T, LG, E>);
+        if constexpr (x_ept_choice<T>(LG)) {
+            set_smem((const void *)k_x_fwd<T, LG, 16>);
+            set_smem((const void *)k_x_inv<T, LG, 16>);
+        }
     });
     f3::lg_for_each<1, 11>([&](auto c) {
         constexpr int LG = decltype(c)::value;
@@ -1123,7 +1142,8 @@ DemagPlan demag_plan(const Geom &g)
     const size_t cs = sizeof(Cx<T>);
     const long budget = 8L * kMaxThreads<T>;
     if (g.P1 > 1) {
-        const int xept = (sizeof(T) == 4 && g.lgQ >= 10) ? 16 : 8;
+        const int xept = x_ept<T>(g);
+        p.x_ept = xept;
         int lpb = (int)((long)xept * kXThreads / g.Q);
         lpb = lpb > 64 ? 64 : lpb;
         if (lpb < 1 || g.lgQ > 10) p.ok = false;
@@ -1177,7 +1197,7 @@ DemagPlan demag_plan(const Geom &g)
     plan_yz<T>(g, p);
     // every block holds at most (values per thread) x (threads) values of its transforms
     if (g.P1 > 1) {
-        const long xept = (sizeof(T) == 4 && g.lgQ >= 10) ? 16 : 8;
+        const long xept = p.x_ept;
         if ((long)p.x_lpb * g.Q > xept * p.x_threads || (long)p.xi_lpb * g.Q > xept * p.xi_threads) p.ok = false;
     }
     if (g.N3 > 1) {
@@ -1263,8 +1283,12 @@ void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cud
         launch_pdl(k_x_fwd1<T>, div_up(nlines, 256), 256, 0, st, g, b, y);
     } else {
         f3::lg_dispatch<1, 10>(g.lgQ, [&](auto c) {
-            constexpr int LG = decltype(c)::value;
-            launch_pdl(k_x_fwd<T, LG>, div_up(nlines, p.x_lpb), p.x_threads, p.x_smem, st, g, b, y, p.x_lpb);
+            constexpr int LG = decltype(c)::value, E = sizeof(T) == 4 && LG >= 10 ? 16 : 8;
+            auto kernel = k_x_fwd<T, LG, E>;
+            if constexpr (x_ept_choice<T>(LG)) {
+                if (p.x_ept == 16) kernel = k_x_fwd<T, LG, 16>;
+            }
+            launch_pdl(kernel, div_up(nlines, p.x_lpb), p.x_threads, p.x_smem, st, g, b, y, p.x_lpb);
         });
     }
     b.mark("demag_x_fwd");
@@ -1308,9 +1332,12 @@ void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cud
         launch_pdl(k_x_inv1<T>, div_up(nlines, 256), 256, 0, st, g, b, MsH, H);
     } else {
         f3::lg_dispatch<1, 10>(g.lgQ, [&](auto c) {
-            constexpr int LG = decltype(c)::value;
-            launch_pdl(k_x_inv<T, LG>, div_up(nlines, p.xi_lpb), p.xi_threads, p.xi_smem, st, g, b, MsH, H,
-                       p.xi_lpb);
+            constexpr int LG = decltype(c)::value, E = sizeof(T) == 4 && LG >= 10 ? 16 : 8;
+            auto kernel = k_x_inv<T, LG, E>;
+            if constexpr (x_ept_choice<T>(LG)) {
+                if (p.x_ept == 16) kernel = k_x_inv<T, LG, 16>;
+            }
+            launch_pdl(kernel, div_up(nlines, p.xi_lpb), p.xi_threads, p.xi_smem, st, g, b, MsH, H, p.xi_lpb);
         });
     }
     b.mark("demag_x_inv");
