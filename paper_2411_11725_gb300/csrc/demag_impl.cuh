@@ -721,8 +721,9 @@ __device__ __forceinline__ void z_product(Cx<T> (&v)[3][(1 << LG) / S], const T 
         }
 }
 
+// (16-point FP32 lines spill at the 128 registers of four blocks: three blocks, 9.1 -> 8.6 us at 128x128x8)
 template <typename T, int LG>
-__global__ void __launch_bounds__(ZRTile<T, LG>::THREADS, 4) k_z_conv_r(Geom g, DemagBufs<T> b)
+__global__ void __launch_bounds__(ZRTile<T, LG>::THREADS, sizeof(T) == 4 && LG == 4 ? 3 : 4) k_z_conv_r(Geom g, DemagBufs<T> b)
 {
     pdl_enter();
     if (b.ctl && b.ctl->done) return;

@@ -287,7 +287,7 @@ static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *
     a.can = (T)p.uan;
     a.im1 = (T)p.uim;
     int blocks = 0;
-    if (g.basis == 3) node_u_grid(g.nn1, g.nn2, g.nn3, &a.bxn, &a.full, &a.chunks, &a.zc, &blocks);
+    if (g.basis == 3) node_u_grid(g.nn1, g.nn2, g.nn3, sizeof(T) == 8, &a.bxn, &a.full, &a.chunks, &a.zc, &blocks);
     node_u_dispatch<T>(a, sa != nullptr, [&](auto nk, auto m64) {
         constexpr int NK = decltype(nk)::value;
         constexpr bool M64 = decltype(m64)::value;
