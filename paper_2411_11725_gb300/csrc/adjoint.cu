@@ -166,16 +166,15 @@ struct AdjBufs {
     double *lam, *lamt, *partials, *scalar;
 };
 
+// t and dt of the next step, written on the device: no read-back, so the host enqueues the reverse sweep ahead of the GPU
+// (with a pull and a push of the control block per step, a gradient over 24 RK4 steps on 256x64x1 cells took 15.4 instead
+// of 14.3 ms)
 int set_ctl(nm_mesh M, double t, double dt)
 {
-    int rc = pull_ctl(M);
-    if (rc) return rc;
-    M->hctl->t = t;
-    M->hctl->dt = dt;
-    M->hctl->t_end = 0.0;
-    M->hctl->done = 0;
-    M->hctl->status = NM_OK;
-    return push_ctl(M);
+    M->y2_valid = false;
+    launch_set_ctl(M->ctl, t, dt, M->st);
+    CHECK_LAUNCH();
+    return NM_OK;
 }
 
 // Stage inputs and slopes of one step at the resident m (and FSAL k1), t and dt in ctl: y_s -> Y[s-1],
@@ -481,8 +480,7 @@ int adjoint_run_t(nm_mesh M, int method, double t_end, double rtol, double atol,
             const double tsamp = t0 + ks * sample_dt;
             if (tsamp < target_t) target_t = tsamp;
         }
-        while (true) {
-            ADJ_TRY(pull_ctl(M));
+        while (true) {  // (the mirror h is current: pulled before the loop and after every step)
             h->t = t;
             h->dt = method == NM_RK4 ? dt0 : dt;
             if (h->dt > target_t - t) h->dt = target_t - t;

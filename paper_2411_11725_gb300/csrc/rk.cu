@@ -599,6 +599,16 @@ __global__ void k_rk4_update(long n_nodes, long ns, double *__restrict__ m, KLis
     }
 }
 
+__global__ void k_set_ctl(StepCtl *ctl, double t, double dt)
+{
+    pdl_enter();
+    ctl->t = t;
+    ctl->dt = dt;
+    ctl->t_end = 0.0;
+    ctl->done = 0;
+    ctl->status = NM_OK;
+}
+
 // Volume-weighted mean of m: per-block partial sums of (w m_x, w m_y, w m_z, w).
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_mean_partials(long n_nodes, long ns, const double *__restrict__ m,
@@ -849,6 +859,11 @@ void launch_rk4_update(const Geom &g, double *m, const KList &kb, StepCtl *ctl, 
                        float *mf)
 {
     launch_pdl(k_rk4_update<T>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), ctl, renorm, mf);
+}
+
+void launch_set_ctl(StepCtl *ctl, double t, double dt, cudaStream_t st)
+{
+    launch_pdl(k_set_ctl, 1, 1, 0, st, ctl, t, dt);
 }
 
 template <typename T>
