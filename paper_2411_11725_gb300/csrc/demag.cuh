@@ -62,6 +62,7 @@ struct DemagPlan {
     size_t yi_smem;            // y passes with a TMA tile (alignment slack and barrier)
     bool yz;                   // one fused y-z convolution instead of the y and z passes
     int yz_lgG, yz_nlp;        // log2 of its kx columns per block, row stride of its tile
+    int yz_threads;
     unsigned yz_plan;          // log2 radices of its y stages, four bits each
     size_t yz_smem;
 };

@@ -890,7 +890,7 @@ __global__ void __launch_bounds__(ZRTile<T, LG>::THREADS, sizeof(T) == 4 && LG =
 //
 // One block of 512 threads (FP64: 256) works through its phases in turn, so their latencies bound it.  Against the
 // passes it replaces (for one layer a fused y pass that held a line's stage in registers, one column per block at
-// this length): 86 against 126 us at 1024x1024x1, 25 / 31 at 512x512x1, FP64 19 / 53 at 64x64x1 and 46 / 63 (three
+// this length): 76 against 126 us at 1024x1024x1, 23 / 31 at 512x512x1, FP64 19 / 53 at 64x64x1 and 46 / 63 (three
 // launches) at 64x64x4.  (Events around each launch, about 5 us of each figure the gap between them.)
 //
 // The y transforms are in place: decimation in frequency forward (the frequencies end in digit-reversed
@@ -912,6 +912,7 @@ __device__ __forceinline__ void yz_stage(int lgP, int lgM, int nl, const FastDiv
 {
     constexpr int R = 1 << LR;
     const int lgq = lgM - LR, nb = nl << (lgP - LR), sh = twlg - lgM;
+#pragma unroll 1  // (two butterflies at a time would not fit the registers)
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
         const int q = (int)nlf.div((unsigned)b), l = b - q * nl;
         const int j = q & ((1 << lgq) - 1), row = ((q >> lgq) << lgM) + j;
@@ -919,6 +920,7 @@ __device__ __forceinline__ void yz_stage(int lgP, int lgM, int nl, const FastDiv
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = ld(l, row + (r << lgq));
         Cx<T> w[R];
+        if (DIR < 0) f3::dft<T, R, DIR>(v);
         if (lgq > 0) {
             const int jj = j << sh;
             if constexpr (R == 16) {
@@ -942,7 +944,7 @@ __device__ __forceinline__ void yz_stage(int lgP, int lgM, int nl, const FastDiv
 #pragma unroll
             for (int r = 1; r < R; ++r) v[r] = f3::twmul<T, DIR>(v[r], w[r]);
         }
-        f3::dft<T, R, DIR>(v);
+        if (DIR > 0) f3::dft<T, R, DIR>(v);
         if (DIR < 0 && lgq > 0) {
 #pragma unroll
             for (int r = 1; r < R; ++r) v[f3::bitrev<R>(r)] = f3::twmul<T, DIR>(v[f3::bitrev<R>(r)], w[r]);
@@ -1123,6 +1125,9 @@ static void plan_yz(const Geom &g, DemagPlan &p)
     p.yz_lgG = lgG;
     p.yz_nlp = ((3 * g.N3) | 1) << lgG;
     p.yz_smem = bytes(lgG);
+    // as many threads as a radix-8 stage has butterflies
+    const int want = (((3 * g.N3) << lgG) * g.P2 / 8 + 31) / 32 * 32;
+    p.yz_threads = want < 128 ? 128 : (want > kYZThreads<T> ? kYZThreads<T> : want);
     // as few stages as radix 8 (FP64 and short lines) or 16 allows, split evenly, the larger radices first
     const int RM = sizeof(T) == 4 && g.lgP2 > 7 ? 4 : 3;
     p.yz_plan = 0;
@@ -1296,7 +1301,7 @@ void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cud
     if (p.yz) {
         f3::lg_dispatch<0, kYZMaxLg3<T>>(g.lgP3, [&](auto c) {
             constexpr int LG3 = decltype(c)::value;
-            launch_pdl(k_yz_conv<T, LG3>, div_up(g.X, 1 << p.yz_lgG), kYZThreads<T>, p.yz_smem, st, g, b, p.yz_lgG,
+            launch_pdl(k_yz_conv<T, LG3>, div_up(g.X, 1 << p.yz_lgG), p.yz_threads, p.yz_smem, st, g, b, p.yz_lgG,
                        p.yz_nlp, FastDiv((unsigned)((3 * g.N3) << p.yz_lgG)), p.yz_plan);
         });
         b.mark("demag_yz_conv");
