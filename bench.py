@@ -152,18 +152,23 @@ def algorithmic_bytes(name, stage, n, b, with_maps):
     # stage inputs and the error scale read the FP64 m (24 B/node), or in the FP32 path its FP32 copy
     mb = 3 * b if b == 4 else 24
     if name == "node_llg_stage":
-        # y_s, Ms*H_c, 1/mass in; k_s out; for s < 7 also m, the k_j with non-zero a_{s+1,j}
-        # (j < s), and y_{s+1} out
-        base = 3 * b * Nn + 3 * b * Nc + b * Nn + 3 * b * Nn
+        # y_s, Ms*H_c in (1/mass only with maps); k_s out; for s < 7 also m, the k_j with non-zero a_{s+1,j}
+        # (j < s), and y_{s+1} out; in FP32 (uniform material) stage 6 writes the step's increment and error so far,
+        # stage 7 reads m, k_1 and that error
+        base = 3 * b * Nn + 3 * b * Nc + (b * Nn if with_maps else 0) + 3 * b * Nn
         if stage < 7:
             nk = {2: 1, 3: 2, 4: 3, 5: 4, 6: 4}[stage]
             base += mb * Nn + nk * 3 * b * Nn + 3 * b * Nn
+        if b == 4 and not with_maps:
+            base += {6: 2 * 3 * b * Nn, 7: 3 * 3 * b * Nn}.get(stage, 0)
         return base
     if name == "dp5_error_control":
         return mb * Nn + 6 * 3 * b * Nn + b * Nn
     if name == "dp5_update":
-        # m in and out (FP64), b_j k_j (j = 1, 3..6) and k7 in, k1 <- k7 and the next y_2 out, FP32 copy of m out
-        return 24 * Nn + 6 * 3 * b * Nn + 24 * Nn + 2 * 3 * b * Nn + (3 * b * Nn if b == 4 else 0)
+        # m in and out (FP64), the increment (FP32, uniform material) or b_j k_j (j = 1, 3..6) and k7 in, k1 <- k7 and the
+        # next y_2 out, FP32 copy of m out
+        nin = 1 if b == 4 and not with_maps else 5
+        return 48 * Nn + (nin + 1) * 3 * b * Nn + 2 * 3 * b * Nn + (3 * b * Nn if b == 4 else 0)
     return 0
 
 

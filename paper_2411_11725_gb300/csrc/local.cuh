@@ -61,7 +61,19 @@ struct StageArgs {
     float af_s;
     const StepCtl *ctl;       // t, dt
     double t_fixed;           // time when ctl == NULL
+    // Dormand-Prince error (FP32, uniform materials): stage 6 also writes the increment dt sum_j b_j k_j of the step to
+    // dinc and its part of the error combination to se; stage 7 (y_next NULL) reads se and takes the step decision
+    float *se, *dinc;
+    float e[5];               // error weights of k_3 .. k_7
+    StepCtl *control;         // ctl, to be written by stage 7
+    double *partials;
+    double n_active;
+    int max_rej;
 };
+constexpr int kMaxPartials = 16384;  // partial sums of a reduction (the mesh's partials buffer)
+// whether the uniform node kernels can form the error of a step on this mesh: a partial sum per block has a place
+template <typename T>
+bool uniform_error_fits(const LocalParams<T> &p);
 
 template <typename T>
 void launch_heff(const LocalParams<T> &p, const T *y, T *h_out, double t, cudaStream_t st);

@@ -262,7 +262,7 @@ static void launch_node_maps(const LocalParams<T> &p, const T *y, T *out, T *y_n
     }
     int blocks = 0;
     node_u_grid(g.nn1, g.nn2, g.nn3, sizeof(T) == 8, &a.u.bxn, &a.u.full, &a.u.chunks, &a.u.zc, &blocks);
-    node_u_dispatch<T>(a.u, sa != nullptr, [&](auto nk, auto m64) {
+    node_u_dispatch<T, false>(a.u, sa != nullptr, [&](auto nk, auto m64) {
         launch_pdl(k_node_m<T, decltype(nk)::value, decltype(m64)::value>, blocks, kUThreads, 0, st, a);
     });
 }

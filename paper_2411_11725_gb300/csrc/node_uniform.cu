@@ -29,11 +29,17 @@ struct NodeUSmem {
     T hf[4];               // uniform applied field, time factor of the cell field
 };
 
+// (The instances of the last two Dormand-Prince stages take 72 registers, seven blocks: at 64 kLast spills and takes
+// 219 us at 512x512x16 where stage 5 takes 101; with 72 it takes 119 and kErr 94, against 63 without the error.)
 template <typename T, int NK, bool M64>
-__global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(const __grid_constant__ NodeUArgs<T> p)
+__global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK == kErr ? 7 : 8) : 4) k_node_u(const __grid_constant__ NodeUArgs<T> p)
 {
     pdl_enter();
-    if (NK != kHeff && p.ctl && p.ctl->done) return;
+    if constexpr (NK == kErr) {
+        if (dp5_idle(p.control)) return;
+    } else if (NK != kHeff && p.ctl && p.ctl->done) {
+        return;
+    }
     using S = NodeUSmem<T>;
     __shared__ S sm;
     const int b = blockIdx.x, split = b >= p.full;
@@ -98,7 +104,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(co
     };
     load_plane(z0 - 1, 0);
     load_plane(z0, 1);
-    const T dt = NK >= 0 && p.ctl ? (T)p.ctl->dt : T(0);
+    const T dt = (NK >= 0 || NK == kErr) && p.ctl ? (T)p.ctl->dt : T(0);
     const double dt64 = NK >= 0 && p.ctl ? p.ctl->dt : 0.0;
     // cells on both sides of the node along x and y
     const T nx = n1 >= 1 && n1 < p.N1 ? T(2) : T(1), ny = n2 >= 1 && n2 < p.N2 ? T(2) : T(1);
@@ -107,8 +113,13 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(co
     // plane z in the node above, m and the cell sum of plane z - 1
     Vec<T> acc = vzero<T>(), up = acc, mc = acc, cc = acc;
     T accR = 0, upR = 0;
+    double err = 0.0;  // (kErr; unused and gone otherwise)
     int s = 0;
     for (int q = z0 - 1; q <= z1; ++q) {
+        ErrIn ei;
+        if constexpr (NK == kErr) {
+            if (q - 1 >= z0 && active) ei = load_err<T>(p, (q - 1) * np + n2 * p.nn1 + n1);
+        }
         asm volatile("cp.async.wait_group 1;\n" ::: "memory");
         __syncthreads();  // plane q has arrived for all; slot (s + 2) mod 3 (plane q - 1) is free
         load_plane(q + 2 <= z1 ? q + 2 : -1, s + 2 >= kUSlots ? s + 2 - kUSlots : s + 2);
@@ -192,7 +203,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(co
                     hz += sm.hf[2];
                 }
             }
-            node_u_out<T, NK, M64>(p, n, hx, hy, hz, mx, my, mz, dt, dt64);
+            err += (double)node_u_out<T, NK, M64>(p, n, hx, hy, hz, mx, my, mz, dt, dt64, true, ei);
         }
         acc = vadd(up, own);
         accR = upR + ownR;
@@ -202,6 +213,10 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(co
         cc = ccur;
         s = s + 1 >= kUSlots ? 0 : s + 1;
     }
+    if constexpr (NK == kErr) {
+        __shared__ double sh[33];
+        dp5_finish(err, p.partials, p.n_active, p.control, p.max_rej, sh);
+    }
 }
 
 // The same operators for the 2D nodal basis (one node layer, constant over the N3 cell layers): the field is
@@ -210,15 +225,14 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 8 : 4) k_node_u(co
 // at 1024x1024x1 (events around each launch) against 52.4 us with the assembled 9-point weights of the general 2D
 // kernel, which sums A, Ku and the cell weights of every layer at every node.
 constexpr int kU2X = 32, kU2Y = 4;
+constexpr int kErrBlocks = 8 * 152;  // blocks of the error instance: eight per SM
 template <typename T, int NK, bool M64>
-__global__ void __launch_bounds__(kU2X *kU2Y) k_node2d_u(const __grid_constant__ NodeUArgs<T> p)
+__device__ __forceinline__ T node2d_u(const NodeUArgs<T> &p, int n1, int n2)
 {
-    pdl_enter();
-    if (NK != kHeff && p.ctl && p.ctl->done) return;
-    const int n1 = blockIdx.x * kU2X + threadIdx.x % kU2X, n2 = blockIdx.y * kU2Y + threadIdx.x / kU2X;
-    if (n1 >= p.nn1 || n2 >= p.nn2) return;
     const int n = n2 * p.nn1 + n1;
-    const T dt = NK >= 0 && p.ctl ? (T)p.ctl->dt : T(0);
+    ErrIn ei;
+    if constexpr (NK == kErr) ei = load_err<T>(p, n);
+    const T dt = (NK >= 0 || NK == kErr) && p.ctl ? (T)p.ctl->dt : T(0);
     const double dt64 = NK >= 0 && p.ctl ? p.ctl->dt : 0.0;
     const bool xl = n1 >= 1, xh = n1 < p.N1, yl = n2 >= 1, yh = n2 < p.N2;
     const T nx = xl && xh ? T(2) : T(1), ny = yl && yh ? T(2) : T(1);
@@ -272,8 +286,54 @@ __global__ void __launch_bounds__(kU2X *kU2Y) k_node2d_u(const __grid_constant__
             h[2] += (T)(p.hu2 * su);
         }
     }
-    node_u_out<T, NK, M64>(p, n, h[0], h[1], h[2], m[0], m[1], m[2], dt, dt64);
+    return node_u_out<T, NK, M64>(p, n, h[0], h[1], h[2], m[0], m[1], m[2], dt, dt64, true, ei);
 }
+template <typename T, int NK, bool M64>
+__global__ void __launch_bounds__(kU2X *kU2Y) k_node2d_u(const __grid_constant__ NodeUArgs<T> p)
+{
+    pdl_enter();
+    if constexpr (NK == kErr) {
+        if (dp5_idle(p.control)) return;
+    } else if (NK != kHeff && p.ctl && p.ctl->done) {
+        return;
+    }
+    auto node = [&](int tile) {
+        const int n1 = tile % p.bxn * kU2X + threadIdx.x % kU2X, n2 = tile / p.bxn * kU2Y + threadIdx.x / kU2X;
+        return n1 < p.nn1 && n2 < p.nn2 ? node2d_u<T, NK, M64>(p, n1, n2) : T(0);
+    };
+    if constexpr (NK == kErr) {
+        // (a block for every tile spends more on its part of the reduction than on its 128 nodes)
+        __shared__ double sh[33];
+        double err = 0.0;
+        for (int tile = blockIdx.x; tile < p.full; tile += gridDim.x) err += (double)node(tile);
+        dp5_finish(err, p.partials, p.n_active, p.control, p.max_rej, sh);
+    } else {
+        node(blockIdx.x);
+    }
+}
+
+template <typename T>
+static void uniform_grid(const Geom &g, NodeUArgs<T> &a, int *blocks)
+{
+    if (g.basis == 3) {
+        node_u_grid(g.nn1, g.nn2, g.nn3, sizeof(T) == 8, &a.bxn, &a.full, &a.chunks, &a.zc, blocks);
+    } else {
+        a.bxn = div_up(g.nn1, kU2X);
+        a.full = *blocks = a.bxn * div_up(g.nn2, kU2Y);
+    }
+}
+
+template <typename T>
+bool uniform_error_fits(const LocalParams<T> &p)
+{
+    if (!p.uniform) return false;
+    NodeUArgs<T> a{};
+    int blocks = 0;
+    uniform_grid<T>(p.g, a, &blocks);
+    return blocks <= kMaxPartials;
+}
+template bool uniform_error_fits<float>(const LocalParams<float> &);
+template bool uniform_error_fits<double>(const LocalParams<double> &);
 
 template <typename T>
 static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *y_next, const StageArgs *sa, double t,
@@ -287,14 +347,15 @@ static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *
     a.can = (T)p.uan;
     a.im1 = (T)p.uim;
     int blocks = 0;
-    if (g.basis == 3) node_u_grid(g.nn1, g.nn2, g.nn3, sizeof(T) == 8, &a.bxn, &a.full, &a.chunks, &a.zc, &blocks);
-    node_u_dispatch<T>(a, sa != nullptr, [&](auto nk, auto m64) {
+    uniform_grid<T>(g, a, &blocks);
+    node_u_dispatch<T, true>(a, sa != nullptr, [&](auto nk, auto m64) {
         constexpr int NK = decltype(nk)::value;
         constexpr bool M64 = decltype(m64)::value;
         if (g.basis == 3)
             launch_pdl(k_node_u<T, NK, M64>, blocks, kUThreads, 0, st, a);
         else
-            launch_pdl(k_node2d_u<T, NK, M64>, dim3(div_up(a.nn1, kU2X), div_up(a.nn2, kU2Y)), kU2X * kU2Y, 0, st, a);
+            launch_pdl(k_node2d_u<T, NK, M64>, NK == kErr && blocks > kErrBlocks ? kErrBlocks : blocks, kU2X * kU2Y, 0,
+                       st, a);
     });
 }
 

@@ -3,6 +3,7 @@
 #pragma once
 #include <type_traits>
 
+#include "dp5_control.cuh"
 #include "local.cuh"
 
 namespace nm {
@@ -135,6 +136,12 @@ struct NodeUArgs {
     const StepCtl *ctl;
     double c_s, t_fixed, hu0, hu1, hu2, hu_freq, hu_phase, hc_freq, hc_phase;
     int raw, zee, nk;
+    // error of a Dormand-Prince step (StageArgs)
+    float *se, *dinc;
+    float e[5];
+    StepCtl *control;
+    double *partials, n_active;
+    int max_rej;
 };
 
 template <typename T>
@@ -158,25 +165,49 @@ __device__ __forceinline__ void cp_elem(T *dst, const T *src, bool in)
 // What a kernel instance writes: the field (kHeff), the slope (kSlope), or the slope and the next stage input
 // formed from NK >= 0 earlier slopes.  M64: the next input is formed from the FP64 m (always in FP64, and in
 // FP32 where no FP32 copy of m is kept).
-constexpr int kHeff = -2, kSlope = -1;
+// kLast: the slope k_6, the next stage input from four earlier slopes, the step's increment and its error so far; kErr:
+// the slope k_7 and the error terms.
+constexpr int kHeff = -2, kSlope = -1, kErr = -3, kLast = 5;
+// earlier slopes that an instance combines
+constexpr int node_slopes(int NK) { return NK == kLast ? 4 : (NK > 0 ? NK : 0); }
+
+// what kErr reads of a node, loaded ahead of its field
+struct ErrIn {
+    float k1[3], se[3], m0[3];
+};
+
+template <typename T>
+__device__ __forceinline__ ErrIn load_err(const NodeUArgs<T> &p, int n)
+{
+    ErrIn e;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        e.k1[c] = p.k[0][c * p.ns + n];
+        e.se[c] = p.se[c * p.ns + n];
+        e.m0[c] = p.mf[c * p.ns + n];
+    }
+    return e;
+}
 
 // The node's output from its field: H itself, or the LLG slope k (zero without magnetic material) and the next
-// stage input
+// stage input.  Returns the node's error terms (kErr; 0 otherwise).
 template <typename T, int NK, bool M64>
-__device__ __forceinline__ void node_u_out(const NodeUArgs<T> &p, int n, T hx, T hy, T hz, T mx, T my, T mz, T dt,
-                                           double dt64, bool magnetic = true)
+__device__ __forceinline__ T node_u_out(const NodeUArgs<T> &p, int n, T hx, T hy, T hz, T mx, T my, T mz, T dt,
+                                     double dt64, bool magnetic = true, const ErrIn &ei = ErrIn())
 {
+    constexpr int NS = node_slopes(NK);
     if (NK == kHeff) {
         p.out[n] = hx;
         p.out[p.ns + n] = hy;
         p.out[2 * p.ns + n] = hz;
+        return T(0);
     } else {
         // the next stage input's own values, all loads issued together
-        T kv[NK > 0 ? NK : 1][3], m0[3];
+        T kv[NS > 0 ? NS : 1][3], m0[3];
         double md[3];
         if (NK >= 0) {
 #pragma unroll
-            for (int i = 0; i < NK; ++i)
+            for (int i = 0; i < NS; ++i)
 #pragma unroll
                 for (int c = 0; c < 3; ++c) kv[i][c] = p.k[i][c * p.ns + n];
 #pragma unroll
@@ -201,11 +232,31 @@ __device__ __forceinline__ void node_u_out(const NodeUArgs<T> &p, int n, T hx, T
             for (int c = 0; c < 3; ++c) {
                 T sum = 0;
 #pragma unroll
-                for (int i = 0; i < NK; ++i) sum += p.a[i] * kv[i][c];
+                for (int i = 0; i < NS; ++i) sum += p.a[i] * kv[i][c];
                 sum += p.as * kk[c];
+                if constexpr (NK == kLast) {
+                    // this sum is the step's increment; the error so far in difference form, operation by operation as
+                    // in dp5_err_node (the rounded slopes: no contraction into their last product)
+                    const T x = kv[0][c];
+                    T e = __fmul_rn(p.e[0], __fsub_rn(kv[1][c], x));
+                    e = __fmaf_rn(p.e[1], __fsub_rn(kv[2][c], x), e);
+                    e = __fmaf_rn(p.e[2], __fsub_rn(kv[3][c], x), e);
+                    p.se[c * p.ns + n] = __fmaf_rn(p.e[3], __fsub_rn(kk[c], x), e);
+                    p.dinc[c * p.ns + n] = dt * sum;
+                }
                 p.y_next[c * p.ns + n] = M64 ? (T)(md[c] + dt64 * (double)sum) : m0[c] + dt * sum;
             }
         }
+        T part = 0;
+        if constexpr (NK == kErr) {
+            // the stage's input is the step's result
+            const float m5[3] = {mx, my, mz}, rtol = (float)p.ctl->rtol, atol = (float)p.ctl->atol;
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                part += dp5_err_term5(ei.m0[c], m5[c], __fmaf_rn(p.e[4], __fsub_rn(kk[c], ei.k1[c]), ei.se[c]), dt, rtol,
+                                      atol);
+        }
+        return part;
     }
 }
 
@@ -239,9 +290,19 @@ inline NodeUArgs<T> node_u_args(const LocalParams<T> &p, const T *y, T *out, T *
     a.ctl = sa->ctl;
     a.c_s = sa->c_s;
     a.t_fixed = sa->t_fixed;
-    if (!y_next) return a;
-    a.m = sa->m;
+    a.se = sa->se;
+    a.dinc = sa->dinc;
+    for (int j = 0; j < 5; ++j) a.e[j] = sa->e[j];
+    a.control = sa->control;
+    a.partials = sa->partials;
+    a.n_active = sa->n_active;
+    a.max_rej = sa->max_rej;
     a.mf = sa->mf;
+    if (!y_next) {
+        a.k[0] = (const T *)sa->k[0];
+        return a;
+    }
+    a.m = sa->m;
     a.as = sizeof(T) == 4 ? (T)sa->af_s : (T)sa->a_s;
     for (int j = 0; j + 1 < sa->s && j < 7; ++j) {
         const T c = sizeof(T) == 4 ? (T)sa->af[j] : (T)sa->a[j];
@@ -253,12 +314,20 @@ inline NodeUArgs<T> node_u_args(const LocalParams<T> &p, const T *y, T *out, T *
     return a;
 }
 
-// go(NK, M64) with the instance that the arguments need
-template <typename T, typename F>
+// go(NK, M64) with the instance that the arguments need (ERR: kErr among them)
+template <typename T, bool ERR, typename F>
 inline void node_u_dispatch(const NodeUArgs<T> &a, bool stage, F &&go)
 {
     if (!stage) return go(std::integral_constant<int, kHeff>{}, std::true_type{});
-    if (!a.y_next) return go(std::integral_constant<int, kSlope>{}, std::true_type{});
+    if (!a.y_next) {
+        if constexpr (sizeof(T) == 4 && ERR) {
+            if (a.control) return go(std::integral_constant<int, kErr>{}, std::false_type{});
+        }
+        return go(std::integral_constant<int, kSlope>{}, std::true_type{});
+    }
+    if constexpr (sizeof(T) == 4 && ERR) {
+        if (a.se) return go(std::integral_constant<int, kLast>{}, std::false_type{});
+    }
     auto slopes = [&](auto n) {
         if constexpr (sizeof(T) == 4) {
             if (a.mf) return go(n, std::false_type{});
@@ -283,13 +352,11 @@ inline void node_u_dispatch(const NodeUArgs<T> &a, bool stage, F &&go)
 // both work on: its cost counts the planes a chunk really works on (128x128x4: 68 -> 46 us a stage, events around each launch).
 inline void node_u_grid(int nn1, int nn2, int nn3, bool fp64, int *bxn, int *full, int *chunks, int *zc, int *blocks)
 {
-    static int sm_count = 0;
-    if (sm_count == 0) {
+    static const int sms = [] {
         int dev = 0, v = 0;
         cudaGetDevice(&dev);
-        sm_count = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 152;
-    }
-    const int sms = sm_count;
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 152;
+    }();
     *bxn = div_up(nn1, kUX);
     const int tiles = *bxn * div_up(nn2, kUY);
     double best = 1e300;

@@ -1,7 +1,7 @@
 // Runge-Kutta bookkeeping kernels: stage inputs, Dormand-Prince error norm with a deterministic
 // two-level reduction, device-side step control, the accepted update with renormalisation, and the
 // boundary layout conversions.
-#include "rk.cuh"
+#include "dp5_control.cuh"
 
 namespace nm {
 
@@ -81,114 +81,6 @@ __device__ __forceinline__ double rsqrt_refined(double s)
     return r0 * (1.5 - 0.5 * s * r0 * r0);
 }
 
-// Sum over the block in a fixed order, the same value in every thread; sh holds 33 values.
-__device__ __forceinline__ double block_sum(double v, double *sh)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if ((threadIdx.x & 31) == 0) sh[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        v = (int)threadIdx.x < nw ? sh[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) sh[32] = v;
-    }
-    __syncthreads();
-    const double r = sh[32];
-    __syncthreads();
-    return r;
-}
-
-// err^(-1/5) for err within [1e-4, 1e4]: the FP32 power and two Newton steps in FP64 (relative error 1e-6 ->
-// 1e-12 -> rounding), a dozen operations where the FP64 power takes hundreds at GB300's FP64 rate
-__device__ __forceinline__ double inv_fifth_root(double err)
-{
-    double r = (double)powf((float)err, -0.2f);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const double r2 = r * r;
-        r = r * (1.2 - 0.2 * err * r2 * r2 * r);
-    }
-    return r;
-}
-
-// Step control from s = the sum of the squared error terms (one thread): err = sqrt(s / (3 n_active)); accept
-// when err <= 1; new dt from dt * clamp(0.9 err^(-1/5), 0.2, 5); clipping to t_end; failure after too many
-// rejections.
-__device__ __forceinline__ void dp5_decide(double s, double n_active, StepCtl *ctl, int max_rej)
-{
-    const double err = n_active > 0 ? sqrt(s / (3.0 * n_active)) : 0.0;
-    const bool fin = isfinite(err), acc = fin && err <= 1.0;
-    // (below 1e-4 and above 1e4 the factor is at its bounds)
-    const double fac =
-        !fin || err > 1e4 ? 0.2 : (err < 1e-4 ? 5.0 : fmin(5.0, fmax(0.2, 0.9 * inv_fifth_root(err))));
-    const double dt = ctl->dt;
-    ctl->err = err;
-    ctl->accepted = acc;
-    ctl->dt_used = dt;
-    double t = ctl->t;
-    int rej = ctl->consecutive_rej;
-    if (acc) {
-        t += dt;
-        ctl->t = t;
-        ctl->n_acc += 1;
-        rej = 0;
-    } else {
-        ctl->n_rej += 1;
-        rej += 1;
-    }
-    ctl->consecutive_rej = rej;
-    double dtn = dt * fac;
-    ctl->dt_prop = dtn;
-    const double t_end = ctl->t_end;
-    bool done = false;
-    if (t_end > 0.0) {
-        const double rem = t_end - t;
-        if (rem <= 1e-12 * fmax(fabs(t_end), 1e-30)) done = true;
-        else if (dtn > rem) dtn = rem;
-    }
-    if (rej > max_rej || (!done && dtn < ctl->dt_min)) {
-        ctl->status = NM_ERR_STEP_UNDERFLOW;
-        done = true;
-    }
-    if (done) ctl->done = 1;
-    ctl->dt = dtn;
-}
-
-// End of an error kernel: the block's sum goes to partials, and the block that arrives last adds them up in
-// order and takes the step decision (a launch of its own before: on small meshes it took as long as a pass).
-// Every block has read what it needs of ctl before it arrives.
-__device__ __forceinline__ void dp5_finish(double acc, double *partials, double n_active, StepCtl *ctl, int max_rej,
-                                           double *sh)
-{
-    __shared__ bool last;
-    const double s = block_sum(acc, sh);
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = s;
-        __threadfence();
-        last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double v = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(partials + i);
-    const double total = block_sum(v, sh);
-    if (threadIdx.x == 0) {
-        ctl->ticket = 0;
-        dp5_decide(total, n_active, ctl, max_rej);
-    }
-}
-// a finished integration: the attempt counts for nothing
-__device__ __forceinline__ bool dp5_idle(StepCtl *ctl)
-{
-    if (!ctl->done) return false;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->accepted = 0;
-    return true;
-}
-
 // Per-block partial sums of ((dt sum_i e_i k_i) / (atol + rtol max(|m|, |m5|)))^2 over magnetic
 // nodes, m5 = m + dt sum_i b_i k_i.  The per-node terms follow the working precision of the slopes
 // (F64T: in FP64 for FP32 slopes too, from the FP64 m and FP64 coefficients); the sums are FP64.
@@ -263,20 +155,6 @@ __global__ void __launch_bounds__(kRedThreads) k_dp5_err(long n_nodes, long ns, 
 // load (16-byte vectors; every component array starts on a 256-byte boundary), fewer and longer
 // requests for the 25 streams the norm reads.  Nodes past the last full group of four go through the
 // scalar terms of block 0.
-//
-// The error combination sum_j e_j k_j (e_j = b_j - b*_j, first slope k_1) is formed in FP32 as
-// sum_{j>1} e_j (k_j - k_1).  The weights sum to zero, so this is the same quantity; the slopes of one
-// step are close to each other, so their differences are exact in FP32 and the combination keeps its
-// relative accuracy when it is far smaller than the slopes (small steps), where the direct sum with
-// FP32-rounded weights would leave a residue of about 1e-8 |k_1|.
-__device__ __forceinline__ float dp5_err_term(float m0, float sb, float se, float dtf, float rtol, float atol)
-{
-    const float m5 = m0 + dtf * sb;
-    const float sc = atol + rtol * fmaxf(fabsf(m0), fabsf(m5));
-    const float q = __fdividef(dtf * se, sc);  // a weight of the norm: fast division
-    return q * q;
-}
-
 // one node's terms
 __device__ __forceinline__ double dp5_err_node(long n, long ns, const KList &kb, const KList &ke,
                                                const float *__restrict__ inv_mass, const float *__restrict__ mf,
@@ -434,13 +312,14 @@ __device__ __forceinline__ void advance_f32(double v[3], const float d[3], int r
 
 // Accepted DP5 step of the FP32 path with the FP32 copy of m: V = 4, four consecutive nodes per thread
 // (16-byte slope loads, two 16-byte FP64 loads per component), the ragged tail node by node; V = 1, one node
-// per thread.  Accepted or not, y2 is the first stage input of the next attempt (m + dt a21 k1 with the new dt),
+// per thread.  INC: d = dt sum_j b_j k_j comes from dinc (written with y_7 by the stage before) instead of from the
+// five slopes: 12 bytes a node instead of 60.  Accepted or not, y2 is the first stage input of the next attempt (m + dt a21 k1 with the new dt),
 // which a launch of its own formed before.
-template <int V>
+template <int V, bool INC>
 __global__ void k_dp5_update_v(long n_nodes, long ns, double *__restrict__ m, const __grid_constant__ KList kb,
                                const float *__restrict__ k7,
                                float *__restrict__ k1, const StepCtl *ctl, int renorm, float *__restrict__ mf,
-                               float *__restrict__ y2, float a21)
+                               float *__restrict__ y2, float a21, const float *__restrict__ dinc)
 {
     pdl_enter();
     const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -473,6 +352,11 @@ __global__ void k_dp5_update_v(long n_nodes, long ns, double *__restrict__ m, co
         float d[3][4];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
+            if constexpr (INC) {
+                const float4 v = reinterpret_cast<const float4 *>(dinc + c * ns)[q];
+                d[c][0] = v.x; d[c][1] = v.y; d[c][2] = v.z; d[c][3] = v.w;
+                continue;
+            }
             float4 sb = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -523,12 +407,14 @@ __global__ void k_dp5_update_v(long n_nodes, long ns, double *__restrict__ m, co
         for (int c = 0; c < 3; ++c) {
             const long i = c * ns + n;
             float sb = 0.f;
+            if constexpr (!INC) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (j >= kb.n) break;
-                sb += kb.af[j] * ((const float *)kb.p[j])[i];
+                for (int j = 0; j < 8; ++j) {
+                    if (j >= kb.n) break;
+                    sb += kb.af[j] * ((const float *)kb.p[j])[i];
+                }
             }
-            dd[c] = dtf * sb;
+            dd[c] = INC ? dinc[i] : dtf * sb;
             w[c] = m[i];
         }
         advance_f32(w, dd, renorm, ff);
@@ -837,16 +723,15 @@ void launch_dp5_control(const Geom &g, const double *m, const KList &kb, const K
 
 template <typename T>
 void launch_dp5_update(const Geom &g, double *m, const KList &kb, const T *k7, T *k1, const StepCtl *ctl, int renorm,
-                       cudaStream_t st, float *mf, T *y2, double a21)
+                       cudaStream_t st, float *mf, T *y2, double a21, const T *dinc)
 {
     if constexpr (sizeof(T) == 4) {
         if (mf) {
-            if (g.n_nodes < kVecNodes)
-                launch_pdl(k_dp5_update_v<1>, div_up(g.n_nodes, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1, ctl,
-                           renorm, mf, y2, (float)a21);
-            else
-                launch_pdl(k_dp5_update_v<4>, div_up(g.n_nodes >> 2, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1,
-                           ctl, renorm, mf, y2, (float)a21);
+            const int v = g.n_nodes < kVecNodes ? 1 : 4;
+            const auto kernel = v == 1 ? (dinc ? k_dp5_update_v<1, true> : k_dp5_update_v<1, false>)
+                                       : (dinc ? k_dp5_update_v<4, true> : k_dp5_update_v<4, false>);
+            launch_pdl(kernel, div_up(g.n_nodes / v, 256), 256, 0, st, g.n_nodes, g.ns, m, fk(kb), k7, k1, ctl, renorm, mf,
+                       y2, (float)a21, dinc);
             return;
         }
     }
@@ -913,7 +798,7 @@ void launch_node_volume(const Geom &g, const double *Ms, double Ms0, double V, T
     template void launch_dp5_control<T>(const Geom &, const double *, const KList &, const KList &, const T *,   \
                                         StepCtl *, double *, double, int, cudaStream_t, const float *, bool);                 \
     template void launch_dp5_update<T>(const Geom &, double *, const KList &, const T *, T *, const StepCtl *,  \
-                                       int, cudaStream_t, float *, T *, double);                                                     \
+                                       int, cudaStream_t, float *, T *, double, const T *);                                                     \
     template void launch_rk4_update<T>(const Geom &, double *, const KList &, StepCtl *, int, cudaStream_t, float *);    \
     template void launch_mean<T>(const Geom &, const double *, const T *, double *, double *, cudaStream_t);     \
     template void launch_cells_to_internal<T>(const Geom &, const double *, int, double, const double *, T *,  \

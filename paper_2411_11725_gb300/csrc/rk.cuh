@@ -33,10 +33,11 @@ template <typename T>
 void launch_dp5_control(const Geom &g, const double *m, const KList &kb, const KList &ke, const T *inv_mass,
                         StepCtl *ctl, double *partials, double n_active, int max_rej, cudaStream_t st,
                         const float *mf = nullptr, bool f64_terms = false);
-// end of a Dormand-Prince attempt; y2 = m + dt a21 k1 of the next one
+// end of a Dormand-Prince attempt; y2 = m + dt a21 k1 of the next one; dinc: dt sum_j b_j k_j of this one when a
+// stage has stored it, or NULL
 template <typename T>
 void launch_dp5_update(const Geom &g, double *m, const KList &kb, const T *k7, T *k1, const StepCtl *ctl, int renorm,
-                       cudaStream_t st, float *mf, T *y2, double a21);
+                       cudaStream_t st, float *mf, T *y2, double a21, const T *dinc);
 template <typename T>
 void launch_rk4_update(const Geom &g, double *m, const KList &kb, StepCtl *ctl, int renorm, cudaStream_t st,
                        float *mf = nullptr);
