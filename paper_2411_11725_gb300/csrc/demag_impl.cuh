@@ -1098,10 +1098,7 @@ static void init_attributes_t()
         set_smem((const void *)k_y_fwd<T, LG>);
         set_smem((const void *)k_y_inv<T, LG>);
     });
-    f3::lg_for_each<1, 7>([&](auto c) {
-        constexpr int LG = decltype(c)::value;
-        set_smem((const void *)k_z_conv<T, LG>);
-    });
+    f3::lg_for_each<kZRMaxLg<T> + 1, 7>([&](auto c) { set_smem((const void *)k_z_conv<T, decltype(c)::value>); });
     f3::lg_for_each<2, kZRMaxLg<T>>([&](auto c) { set_smem((const void *)k_z_conv_r<T, decltype(c)::value>); });
     f3::lg_for_each<0, kYZMaxLg3<T>>([&](auto c) { set_smem((const void *)k_yz_conv<T, decltype(c)::value>); });
 }
@@ -1181,15 +1178,15 @@ DemagPlan demag_plan(const Geom &g)
             p.y_smem = Y::SMEM;
             p.yi_smem = Y::SMEM_TMA;
         });
-        if (g.lgP3 < 1 || g.lgP3 > 7) p.ok = false;
-        f3::lg_dispatch<1, 7>(g.lgP3, [&](auto c) {
+        if (g.lgP3 < 2 || g.lgP3 > 7) p.ok = false;
+        f3::lg_dispatch<kZRMaxLg<T> + 1, 7>(g.lgP3, [&](auto c) {
             using Z = ZTile<T, decltype(c)::value>;
             p.z_G = Z::G;
             p.z_KY = Z::KY;
             p.z_threads = Z::THREADS;
             p.z_smem = Z::SMEM;
         });
-        p.z_reg = g.lgP3 >= 2 && g.lgP3 <= kZRMaxLg<T> && 2 * g.N3 <= g.P3;
+        p.z_reg = g.lgP3 <= kZRMaxLg<T>;
         if (p.z_reg) {
             f3::lg_dispatch<2, kZRMaxLg<T>>(g.lgP3, [&](auto c) {
                 using Z = ZRTile<T, decltype(c)::value>;
@@ -1320,7 +1317,7 @@ void demag_forward(const Geom &g, const DemagBufs<T> &b, const T *y, T *MsH, cud
             });
         }
         if (!p.z_reg) {
-            f3::lg_dispatch<1, 7>(g.lgP3, [&](auto c) {
+            f3::lg_dispatch<kZRMaxLg<T> + 1, 7>(g.lgP3, [&](auto c) {
                 constexpr int LG = decltype(c)::value;
                 launch_pdl(k_z_conv<T, LG>, dim3(g.Xp / p.z_G, div_up(g.H2, p.z_KY)), p.z_threads, p.z_smem, st, g, b);
             });
