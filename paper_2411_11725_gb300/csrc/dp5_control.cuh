@@ -1,5 +1,5 @@
-// Error terms, reduction and step control of a Dormand-Prince attempt: shared by the error kernels and by the node
-// kernels that form the error themselves.
+// Error terms, reduction and step control of a Dormand-Prince attempt, and the end of an RK4 step: shared by the kernels
+// of the Runge-Kutta bookkeeping and by the node kernels that do that work themselves.
 #pragma once
 #include "rk.cuh"
 
@@ -127,6 +127,43 @@ __device__ __forceinline__ float dp5_err_term5(float m0, float m5, float se, flo
 __device__ __forceinline__ float dp5_err_term(float m0, float sb, float se, float dtf, float rtol, float atol)
 {
     return dp5_err_term5(m0, m0 + dtf * sb, se, dtf, rtol, atol);
+}
+
+// 1/sqrt(s) for s > 0 in FP64 from an FP32 estimate and one Newton step (relative error ~1e-14), so
+// the FP32 path renormalises without FP64 division or square root.
+__device__ __forceinline__ double rsqrt_refined(double s)
+{
+    const double r0 = (double)rsqrtf((float)s);
+    return r0 * (1.5 - 0.5 * s * r0 * r0);
+}
+
+// v / |v| (v unchanged when zero): FP32 meshes through rsqrt_refined
+template <typename T>
+__device__ __forceinline__ void renormalise(double v[3])
+{
+    const double s = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    if (s > 0.0) {
+        const double r = sizeof(T) == 8 ? 1.0 / sqrt(s) : rsqrt_refined(s);
+        v[0] *= r; v[1] *= r; v[2] *= r;
+    }
+}
+
+// End of an RK4 step, called by every thread of the grid: the block that arrives last (every thread of every block has
+// read t and dt by then) advances the time
+__device__ __forceinline__ void rk4_finish(StepCtl *ctl)
+{
+    __syncthreads();
+    if (threadIdx.x != 0 || atomicAdd(&ctl->ticket, 1u) != gridDim.x - 1) return;
+    ctl->ticket = 0;
+    ctl->t += ctl->dt;
+    ctl->n_acc += 1;
+    ctl->accepted = 1;
+    ctl->dt_used = ctl->dt;
+    if (ctl->t_end > 0.0) {
+        double rem = ctl->t_end - ctl->t;
+        if (rem <= 1e-12 * fmax(fabs(ctl->t_end), 1e-30)) ctl->done = 1;
+        else if (ctl->dt > rem) ctl->dt = rem;
+    }
 }
 
 }  // namespace nm

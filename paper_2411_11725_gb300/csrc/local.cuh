@@ -65,7 +65,12 @@ struct StageArgs {
     // dinc and its part of the error combination to se; stage 7 (y_next NULL) reads se and takes the step decision
     float *se, *dinc;
     float e[5];               // error weights of k_3 .. k_7
-    StepCtl *control;         // ctl, to be written by stage 7
+    StepCtl *control;         // ctl, to be written by stage 7 (RK4: by stage 4)
+    // RK4 (node kernels of node_uniform.cu and node_maps.cu): stage 4 ends the step when m_out is set: a and a_s are then
+    // the weights b of the four slopes, m_out (= m) and its FP32 copy receive the new state, and the time advances
+    double *m_out;
+    float *mf_out;
+    int renorm;
     double *partials;
     double n_active;
     int max_rej;

@@ -237,6 +237,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? 6 : 4) k_node_m(co
         s1 = (s1 + 1) & 3;
         sc = sc + 1 >= kMCellSlots ? 0 : sc + 1;
     }
+    if constexpr (NK == kRk4) rk4_finish(p.control);
 }
 
 template <typename T>

@@ -32,7 +32,7 @@ struct NodeUSmem {
 // (The instances of the last two Dormand-Prince stages take 72 registers, seven blocks: at 64 kLast spills and takes
 // 219 us at 512x512x16 where stage 5 takes 101; with 72 it takes 119 and kErr 94, against 63 without the error.)
 template <typename T, int NK, bool M64>
-__global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK == kErr ? 7 : 8) : 4) k_node_u(const __grid_constant__ NodeUArgs<T> p)
+__global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK == kErr || NK == kRk4 ? 7 : 8) : 4) k_node_u(const __grid_constant__ NodeUArgs<T> p)
 {
     pdl_enter();
     if constexpr (NK == kErr) {
@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
         __shared__ double sh[33];
         dp5_finish(err, p.partials, p.n_active, p.control, p.max_rej, sh);
     }
+    if constexpr (NK == kRk4) rk4_finish(p.control);
 }
 
 // The same operators for the 2D nodal basis (one node layer, constant over the N3 cell layers): the field is
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
 // at 1024x1024x1 (events around each launch) against 52.4 us with the assembled 9-point weights of the general 2D
 // kernel, which sums A, Ku and the cell weights of every layer at every node.
 constexpr int kU2X = 32, kU2Y = 4;
-constexpr int kErrBlocks = 8 * 152;  // blocks of the error instance: eight per SM
+constexpr int kErrBlocks = 8 * 152;  // blocks of the instances that end a step: eight per SM
 template <typename T, int NK, bool M64>
 __device__ __forceinline__ T node2d_u(const NodeUArgs<T> &p, int n1, int n2)
 {
@@ -307,6 +308,9 @@ __global__ void __launch_bounds__(kU2X *kU2Y) k_node2d_u(const __grid_constant__
         double err = 0.0;
         for (int tile = blockIdx.x; tile < p.full; tile += gridDim.x) err += (double)node(tile);
         dp5_finish(err, p.partials, p.n_active, p.control, p.max_rej, sh);
+    } else if constexpr (NK == kRk4) {
+        for (int tile = blockIdx.x; tile < p.full; tile += gridDim.x) node(tile);
+        rk4_finish(p.control);
     } else {
         node(blockIdx.x);
     }
@@ -354,7 +358,7 @@ static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *
         if (g.basis == 3)
             launch_pdl(k_node_u<T, NK, M64>, blocks, kUThreads, 0, st, a);
         else
-            launch_pdl(k_node2d_u<T, NK, M64>, NK == kErr && blocks > kErrBlocks ? kErrBlocks : blocks, kU2X * kU2Y, 0,
+            launch_pdl(k_node2d_u<T, NK, M64>, (NK == kErr || NK == kRk4) && blocks > kErrBlocks ? kErrBlocks : blocks, kU2X * kU2Y, 0,
                        st, a);
     });
 }

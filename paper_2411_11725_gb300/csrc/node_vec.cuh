@@ -142,6 +142,10 @@ struct NodeUArgs {
     StepCtl *control;
     double *partials, n_active;
     int max_rej;
+    // end of an RK4 step (StageArgs)
+    double *m_out;
+    float *mf_out;
+    int renorm;
 };
 
 template <typename T>
@@ -167,9 +171,10 @@ __device__ __forceinline__ void cp_elem(T *dst, const T *src, bool in)
 // FP32 where no FP32 copy of m is kept).
 // kLast: the slope k_6, the next stage input from four earlier slopes, the step's increment and its error so far; kErr:
 // the slope k_7 and the error terms.
-constexpr int kHeff = -2, kSlope = -1, kErr = -3, kLast = 5;
+// kRk4: the new state of an RK4 step from three earlier slopes and k_4, which is not written.
+constexpr int kHeff = -2, kSlope = -1, kErr = -3, kLast = 5, kRk4 = 6;
 // earlier slopes that an instance combines
-constexpr int node_slopes(int NK) { return NK == kLast ? 4 : (NK > 0 ? NK : 0); }
+constexpr int node_slopes(int NK) { return NK == kLast ? 4 : (NK == kRk4 ? 3 : (NK > 0 ? NK : 0)); }
 
 // what kErr reads of a node, loaded ahead of its field
 struct ErrIn {
@@ -224,6 +229,24 @@ __device__ __forceinline__ T node_u_out(const NodeUArgs<T> &p, int n, T hx, T hy
         kk[1] = -p.gam * (ay + p.alpha * by);
         kk[2] = -p.gam * (az + p.alpha * bz);
         if (!magnetic) kk[0] = kk[1] = kk[2] = T(0);
+        if constexpr (NK == kRk4) {
+            double v[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                T sum = 0;
+#pragma unroll
+                for (int i = 0; i < NS; ++i) sum += p.a[i] * kv[i][c];
+                sum += p.as * kk[c];
+                v[c] = md[c] + dt64 * (double)sum;
+            }
+            if (p.renorm) renormalise<T>(v);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                p.m_out[c * p.ns + n] = v[c];
+                if (p.mf_out) p.mf_out[c * p.ns + n] = (float)v[c];
+            }
+            return T(0);
+        }
 #pragma unroll
         for (int c = 0; c < 3; ++c) p.out[c * p.ns + n] = kk[c];
         if (NK >= 0) {
@@ -298,7 +321,10 @@ inline NodeUArgs<T> node_u_args(const LocalParams<T> &p, const T *y, T *out, T *
     a.n_active = sa->n_active;
     a.max_rej = sa->max_rej;
     a.mf = sa->mf;
-    if (!y_next) {
+    a.m_out = sa->m_out;
+    a.mf_out = sa->mf_out;
+    a.renorm = sa->renorm;
+    if (!y_next && !sa->m_out) {
         a.k[0] = (const T *)sa->k[0];
         return a;
     }
@@ -319,6 +345,7 @@ template <typename T, bool ERR, typename F>
 inline void node_u_dispatch(const NodeUArgs<T> &a, bool stage, F &&go)
 {
     if (!stage) return go(std::integral_constant<int, kHeff>{}, std::true_type{});
+    if (a.m_out) return go(std::integral_constant<int, kRk4>{}, std::true_type{});
     if (!a.y_next) {
         if constexpr (sizeof(T) == 4 && ERR) {
             if (a.control) return go(std::integral_constant<int, kErr>{}, std::false_type{});

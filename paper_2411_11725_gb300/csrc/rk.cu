@@ -73,14 +73,6 @@ __global__ void k_stage_input_f4(long n_nodes, long ns, KList k, const StepCtl *
     }
 }
 
-// 1/sqrt(s) for s > 0 in FP64 from an FP32 estimate and one Newton step (relative error ~1e-14), so
-// the FP32 path renormalises without FP64 division or square root.
-__device__ __forceinline__ double rsqrt_refined(double s)
-{
-    const double r0 = (double)rsqrtf((float)s);
-    return r0 * (1.5 - 0.5 * s * r0 * r0);
-}
-
 // Per-block partial sums of ((dt sum_i e_i k_i) / (atol + rtol max(|m|, |m5|)))^2 over magnetic
 // nodes, m5 = m + dt sum_i b_i k_i.  The per-node terms follow the working precision of the slopes
 // (F64T: in FP64 for FP32 slopes too, from the FP64 m and FP64 coefficients); the sums are FP64.
@@ -248,13 +240,7 @@ __device__ __forceinline__ void advance_node(long n, long ns, const double *__re
         }
         v[c] = m[i] + dt * (double)sb;
     }
-    if (renorm) {
-        const double s = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-        if (s > 0.0) {
-            const double r = sizeof(T) == 8 ? 1.0 / sqrt(s) : rsqrt_refined(s);
-            v[0] *= r; v[1] *= r; v[2] *= r;
-        }
-    }
+    if (renorm) renormalise<T>(v);
 }
 
 // FP32 <-> FP64 conversions with integer operations, bit-identical to the hardware conversions in the
@@ -470,19 +456,7 @@ __global__ void k_rk4_update(long n_nodes, long ns, double *__restrict__ m, KLis
             if (mf) mf[c * ns + n] = (float)v[c];
         }
     }
-    // the block that arrives last (every thread of every block has read dt by then) advances the time
-    __syncthreads();
-    if (threadIdx.x != 0 || atomicAdd(&ctl->ticket, 1u) != gridDim.x - 1) return;
-    ctl->ticket = 0;
-    ctl->t += ctl->dt;
-    ctl->n_acc += 1;
-    ctl->accepted = 1;
-    ctl->dt_used = ctl->dt;
-    if (ctl->t_end > 0.0) {
-        double rem = ctl->t_end - ctl->t;
-        if (rem <= 1e-12 * fmax(fabs(ctl->t_end), 1e-30)) ctl->done = 1;
-        else if (ctl->dt > rem) ctl->dt = rem;
-    }
+    rk4_finish(ctl);
 }
 
 __global__ void k_set_ctl(StepCtl *ctl, double t, double dt)
