@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kMaxThreads<T>, kMinBlocks<T>) k_z_conv(Geom g
 // The tensor slice is staged with cp.async while the forward transforms run; read straight from L2 inside the
 // product, its latency was exposed at every frequency (1.26 ms at 1024x1024x32).  Against the version that held one
 // component's line per thread and exchanged spectra through shared memory for the product (4x the shared traffic;
-// FP64 and P3 <= 4 had their own): 1.07 -> 1.01 ms at 1024x1024x32 (S = 4), 144 -> 107 us at 512x512x16 (S = 2),
+// FP64 and P3 <= 4 had their own): 1.07 -> 0.89 ms at 1024x1024x32 (S = 4), 144 -> 107 us at 512x512x16 (S = 2),
 // 24.7 -> 16.5 us at 256x256x8 and FP64 53 -> 39 us at 128x128x4 (S = 1, no exchange at all).
 template <typename T, int LG>
 struct ZRTile {
@@ -800,18 +800,29 @@ __global__ void __launch_bounds__(ZRTile<T, LG>::THREADS, sizeof(T) == 4 && LG =
             }
         }
     }
-    // twist by w^{mr}: r is the same for a whole warp, so the powers are constants of each branch
+    // twist by w^{mr}; r is the same for a whole warp.  Two parts: constants for part 1.  Four parts: from the table, the
+    // same instructions for every part; with a branch of constants for each the kernel waited for its instructions more
+    // than for anything else (1.03 -> 0.89 ms at 1024x1024x32; two parts 107 -> 117 us at 512x512x16, so not there).
     auto twist = [&](auto dir) {
         constexpr int DIR = decltype(dir)::value;
+        if (r == 0) return;
+        if constexpr (S == 4) {
+            const Cx<T> *tw = b.tw;
+            const int step = r << (g.twlg - LG);
 #pragma unroll
-        for (int rr = 1; rr < S; ++rr) {
-            if (r != rr) continue;
+            for (int m = 1; m < D; ++m) {
+                const Cx<T> w = tw[m * step];
+                const int i = DIR < 0 ? m : f3::bitrev<D>(m);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) v[c][i] = f3::twmul<T, DIR>(v[c][i], w);
+            }
+        } else {
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
                 for (int m = 1; m < D; ++m) {
                     const int i = DIR < 0 ? m : f3::bitrev<D>(m);
-                    v[c][i] = f3::rot<T, P3, DIR>(v[c][i], m * rr);
+                    v[c][i] = f3::rot<T, P3, DIR>(v[c][i], m);
                 }
         }
     };
