@@ -222,9 +222,15 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
 
 // The same operators for the 2D nodal basis (one node layer, constant over the N3 cell layers): the field is
 //   -2 A (K1 M2 + M1 K2) m + 2 Ku e (M1 M2) (e . m), both times the film's thickness,
-// one thread per node, neighbours and cells through L1.  Bound by instruction issue and L1 latency: 26.6 us per stage
-// at 1024x1024x1 (events around each launch) against 52.4 us with the assembled 9-point weights of the general 2D
-// kernel, which sums A, Ku and the cell weights of every layer at every node.
+// one thread per node, neighbours and cells through L1.  Each operator is a combination of sums of differences to
+// the node itself, X of the neighbours along x, Y along y and C of the corners, in which an index beyond an end is
+// moved to the end (the weights take out what that adds):
+//   exchange w1 X + w2 Y + ws C,   36 M1 M2 u / (dx dy) = 9 nx ny u + (3 ny - 2) X + (3 nx - 2) Y + C.
+// Differences of close values are exact, so the exchange field keeps its relative accuracy on smooth states, where sums
+// of the values themselves cancel (FP32, 200x200 cells, a rotation by 0.01 rad a cell: relative error inside 6.8e-4
+// with such sums, 3.1e-7 here).  Bound by instruction issue and L1 latency: 30.2 us a stage of a Dormand-Prince step at
+// 1024x1024x1 (events around each launch; 29.7 us with sums of values), against 52.4 us with the assembled 9-point
+// weights of the general 2D kernel, which sums A, Ku and the cell weights of every layer at every node.
 constexpr int kU2X = 32, kU2Y = 4;
 constexpr int kErrBlocks = 8 * 152;  // blocks of the instances that end a step: eight per SM
 template <typename T, int NK, bool M64>
@@ -237,24 +243,17 @@ __device__ __forceinline__ T node2d_u(const NodeUArgs<T> &p, int n1, int n2)
     const double dt64 = NK >= 0 && p.ctl ? p.ctl->dt : 0.0;
     const bool xl = n1 >= 1, xh = n1 < p.N1, yl = n2 >= 1, yh = n2 < p.N2;
     const T nx = xl && xh ? T(2) : T(1), ny = yl && yh ? T(2) : T(1);
+    const int xm = xl ? -1 : 0, xp = xh ? 1 : 0, rm = yl ? -p.nn1 : 0, rp = yh ? p.nn1 : 0;
+    const T w1 = ny == T(2) ? p.w1[0] : p.w1[1], w2 = nx == T(2) ? p.w2[0] : p.w2[1];
     T h[3], m[3], P[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        // row sums along x of rows n2 - 1 .. n2 + 1: a = 6 M1 m / dx, d = -dx K1 m (zero beyond the ends)
         const T *q = p.y + c * p.ns + n;
-        T a[3], d[3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            const bool in = r == 1 || (r == 0 ? yl : yh);
-            const T *qr = q + (r - 1) * p.nn1;
-            const T c0 = in ? qr[0] : T(0), e = (in && xl ? qr[-1] : T(0)) + (in && xh ? qr[1] : T(0));
-            a[r] = fma(T(2) * nx, c0, e);
-            d[r] = fma(-nx, c0, e);
-            if (r == 1) m[c] = c0;
-        }
-        const T as = a[0] + a[2];
-        P[c] = fma(T(2) * ny, a[1], as);
-        h[c] = p.cx * fma(T(2) * ny, d[1], d[0] + d[2]) + p.cy * fma(-ny, a[1], as);
+        const T u = q[0], X = (q[xm] - u) + (q[xp] - u), Y = (q[rm] - u) + (q[rp] - u);
+        const T C = ((q[rm + xm] - u) + (q[rp + xp] - u)) + ((q[rm + xp] - u) + (q[rp + xm] - u));
+        m[c] = u;
+        h[c] = fma(p.ws, C, fma(w2, Y, w1 * X));
+        P[c] = fma(T(9) * nx * ny, u, fma(T(3) * nx - T(2), Y, fma(T(3) * ny - T(2), X, C)));
     }
     const T pe = p.can * (p.e0 * P[0] + p.e1 * P[1] + p.e2 * P[2]);
     h[0] += p.e0 * pe;
@@ -271,13 +270,14 @@ __device__ __forceinline__ T node2d_u(const NodeUArgs<T> &p, int n1, int n2)
                           ((xl && yh ? q[-1] : T(0)) + (xh && yh ? q[0] : T(0)));
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) h[c] += p.mu0V8 * s * sum[c];
+        for (int c = 0; c < 3; ++c) h[c] += p.im1 * (p.mu0V8 * s * sum[c]);
     };
     const double t = NK != kHeff && p.ctl ? p.ctl->t + p.c_s * p.ctl->dt : p.t_fixed;
     if (p.MsH) cells(p.MsH, T(1));
     if (p.Msh && p.zee) cells(p.Msh, (T)u_time_factor<T>(p.hc_freq, p.hc_phase, t));
     if (!p.raw) {
-        const T im = p.im1 * (nx == T(2) ? T(0.5) : T(1)) * (ny == T(2) ? T(0.5) : T(1));
+        // (the weights hold 1 / mass of a node with one cell column; the others have two or four)
+        const T im = (nx == T(2) ? T(0.5) : T(1)) * (ny == T(2) ? T(0.5) : T(1));
 #pragma unroll
         for (int c = 0; c < 3; ++c) h[c] *= im;
         if (p.zee) {
@@ -350,6 +350,17 @@ static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *
     a.cz = (T)p.ucz;
     a.can = (T)p.uan;
     a.im1 = (T)p.uim;
+    if (g.basis == 2) {
+        // one rounding for each constant
+        const double s = p.raw ? 1.0 : p.uim;
+        a.w1[0] = (T)(s * (4.0 * p.ucx - 2.0 * p.ucy));  // cells on both sides of the node along the other axis
+        a.w1[1] = (T)(s * (p.ucx - 2.0 * p.ucy));        // on one side
+        a.w2[0] = (T)(s * (4.0 * p.ucy - 2.0 * p.ucx));
+        a.w2[1] = (T)(s * (p.ucy - 2.0 * p.ucx));
+        a.ws = (T)(s * (p.ucx + p.ucy));
+        a.can = (T)(s * p.uan);
+        a.im1 = (T)s;
+    }
     int blocks = 0;
     uniform_grid<T>(g, a, &blocks);
     node_u_dispatch<T, true>(a, sa != nullptr, [&](auto nk, auto m64) {

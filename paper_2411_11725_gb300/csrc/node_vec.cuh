@@ -124,6 +124,8 @@ struct NodeUArgs {
     int bxn, full, chunks, zc;  // blocks b < full walk tile b over all planes; the other tiles are split into
                                 // `chunks` blocks of zc planes
     T cx, cy, cz, can;          // 2 A x element constants of the axes; 2 Ku V / 216 (2D basis: / 36 per layer)
+    T w1[2], w2[2], ws;         // 2D basis: exchange weights of the sums of differences (node_uniform.cu); these and can
+                                // are over the mass of a node with one cell column unless raw (im1 = 1 then)
     T e0, e1, e2;
     T im1, mu0V8;               // 1 / (mu0 V/8 Ms), mu0 V/8 (2D basis: 1 / (mu0 V/4 Ms N3), mu0 V/4)
     T gam, alpha;
