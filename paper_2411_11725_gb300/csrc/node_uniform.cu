@@ -6,19 +6,28 @@
 // With one A and one Ku on a box of cells the assembled operators are sums of tensor products of the
 // one-dimensional stiffness and mass matrices, which at a node with n adjacent cells along the axis (n = 2
 // inside, 1 at an end) act as
-//   K u = (n u0 - (u- + u+)) / dx,      M u = (2 n u0 + (u- + u+)) dx / 6,
-// with u = 0 beyond the ends.  The field is
-//   -dE_ex = -2 A (K1 M2 M3 + M1 K2 M3 + M1 M2 K3) m,   -dE_an = 2 Ku e (M1 M2 M3) (e . m),
-// evaluated axis by axis: along x and y for each node plane (9 neighbours), along z by carrying two partial
-// sums per component up the walk.  That is about 65 multiply-adds and 9 shared-memory vectors per node
-// instead of the 162 and 27 of the assembled 27-point form, and the boundary needs no case of its own.
+//   K u = -D u / dx,      M u = (3 n u0 + D u) dx / 6,      D u = the sum of u' - u0 over the neighbours u' (n of them).
+// The field is
+//   -dE_ex = -2 A (K1 M2 M3 + M1 K2 M3 + M1 M2 K3) m,   -dE_an = 2 Ku e (M1 M2 M3) (e . m).
+// A node at an end of the x or y axis has half the cells and half the mass of one inside, so its field is that of a node
+// inside whose missing neighbours mirror the ones it has; along z the ends keep their own weights.  In a node plane every
+// operator is a combination of sums of differences to the node itself, X of the neighbours along x, Y along y and C of
+// the corners; along z two partial sums per component and the node's own value are carried up the walk:
+//   exchange at z:  n3 (w1 X + w2 Y + ws C)(z) + sum over the planes z' beside of  (v1 X + v2 Y + vs C)(z') + vz (u0(z') - u0(z)),
+//   36 M1 M2 u / (dx dy) = 36 u0 + 4 X + 4 Y + C.
+// That is about 75 multiply-adds and 9 shared-memory vectors per node instead of the 162 and 27 of the assembled
+// 27-point form.  Differences of close values are exact, so the exchange field keeps its relative accuracy on smooth
+// states; sums of the values themselves cancel (FP32, 64x64x16 cells, a rotation by 0.01 rad a cell: relative error inside
+// 7.7e-4 with such sums, 1.6e-6 here; random state 7.1e-8, 5.3e-8).  FP64 keeps the sums: it is bound by the FP64 rate
+// (stage at 128x128x4: 54.5 us with differences, 48.5 us), and their rounding is 1e-16 of the values.
 #include "node_vec.cuh"
 
 namespace nm {
 
 // Tile of 32 x 4 nodes walked along z by 128 threads, eight FP32 blocks per SM at 64 registers.  Measured per
-// stage at 1024x1024x32 (FP32) / 512x512x16: this kernel 0.59 ms / 87 us, against 1.04 ms / 154 us for the
-// assembled 27-point form and 0.64 ms / 99 us with two rows per thread (96 registers, five blocks per SM).
+// stage at 1024x1024x32 (FP32) / 512x512x16, with sums of the values: 0.59 ms / 87 us, against 1.04 ms / 154 us for the
+// assembled 27-point form and 0.64 ms / 99 us with two rows per thread (96 registers, five blocks per SM).  The
+// differences cost 2 / 5 %: mean stage of a Dormand-Prince step, with its error terms, 0.644 -> 0.658 ms / 95 -> 100 us.
 constexpr int kUSlots = 3;
 
 template <typename T>
@@ -28,6 +37,9 @@ struct NodeUSmem {
     VPlanes<T, CY, CX, kUSlots> c;  // cell plane p - 1 (Ms_c H_c) beside node plane p
     T hf[4];               // uniform applied field, time factor of the cell field
 };
+
+// the node that stands for index i of an axis of n nodes: its mirror image beside an end, an end beyond that
+__device__ __forceinline__ int mirror(int i, int n) { return i < 0 ? 1 : (i < n ? i : (i == n ? n - 2 : n - 1)); }
 
 // (The instances of the last two Dormand-Prince stages take 72 registers, seven blocks: at 64 kLast spills and takes
 // 219 us at 512x512x16 where stage 5 takes 101; with 72 it takes 119 and kErr 94, against 63 without the error.)
@@ -56,15 +68,14 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
         sm.hf[2] = (T)(p.hu2 * su);
         sm.hf[3] = (T)u_time_factor<T>(p.hc_freq, p.hc_phase, t);
     }
-    // the elements of every node and cell plane that this thread copies: offset within the plane, or -1
-    // outside the mesh (zero fill)
+    // the elements of every node and cell plane that this thread copies: offset within the plane (outside the mesh: of the
+    // mirror node beside an end, of an end beyond that), or -1 outside the cells (zero fill)
     constexpr int EN = (S::SX * S::SY + kUThreads - 1) / kUThreads, EC = (S::CX * S::CY + kUThreads - 1) / kUThreads;
     int no[EN], co[EC];
 #pragma unroll
     for (int k = 0; k < EN; ++k) {
         const int t = threadIdx.x + k * kUThreads, r = t / S::SX, c = t - r * S::SX;
-        const int i = x0 - 1 + c, j = y0 - 1 + r;
-        no[k] = (i >= 0 && i < p.nn1 && j >= 0 && j < p.nn2) ? j * p.nn1 + i : -1;
+        no[k] = mirror(y0 - 1 + r, p.nn2) * p.nn1 + mirror(x0 - 1 + c, p.nn1);
     }
 #pragma unroll
     for (int k = 0; k < EC; ++k) {
@@ -81,10 +92,9 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
             for (int k = 0; k < EN; ++k) {
                 const int t = threadIdx.x + k * kUThreads;
                 if (t < S::SX * S::SY) {
-                    const bool in = no[k] >= 0;
-                    const T *src = p.y + (in ? q * np + no[k] : 0);
+                    const T *src = p.y + (q * np + no[k]);
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) cp_elem(sm.y.p(s, t, c), src + c * p.ns, in);
+                    for (int c = 0; c < 3; ++c) cp_elem(sm.y.p(s, t, c), src + c * p.ns, true);
                 }
             }
         }
@@ -107,10 +117,10 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
     const T dt = (NK >= 0 || NK == kErr) && p.ctl ? (T)p.ctl->dt : T(0);
     const double dt64 = NK >= 0 && p.ctl ? p.ctl->dt : 0.0;
     // cells on both sides of the node along x and y
-    const T nx = n1 >= 1 && n1 < p.N1 ? T(2) : T(1), ny = n2 >= 1 && n2 < p.N2 ? T(2) : T(1);
+    const bool bx = n1 >= 1 && n1 < p.N1, by = n2 >= 1 && n2 < p.N2;
     const bool active = n1 < p.nn1 && n2 < p.nn2;
-    // carried up the walk: the part of the node being completed that planes z - 1 and z gave, the share of
-    // plane z in the node above, m and the cell sum of plane z - 1
+    // carried up the walk: the part of the node being completed that planes z - 1 and z gave, the share of plane z in the
+    // node above, m and the cell sum of plane z
     Vec<T> acc = vzero<T>(), up = acc, mc = acc, cc = acc;
     T accR = 0, upR = 0;
     double err = 0.0;  // (kErr; unused and gone otherwise)
@@ -123,27 +133,41 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
         asm volatile("cp.async.wait_group 1;\n" ::: "memory");
         __syncthreads();  // plane q has arrived for all; slot (s + 2) mod 3 (plane q - 1) is free
         load_plane(q + 2 <= z1 ? q + 2 : -1, s + 2 >= kUSlots ? s + 2 - kUSlots : s + 2);
-        Vec<T> own = vzero<T>(), fin = own, mnew = own, ccur = own;
+        Vec<T> own = vzero<T>(), fin = own, mnew = own, ccur = own, dz = own;
+        T nz = 1;
         T ownR = 0, finR = 0;
         if (q >= 0 && q < p.nn3) {
-            // row sums along x of rows n2 - 1 .. n2 + 1: a = 6 M1 m / dx, d = -dx K1 m
-            Vec<T> a[3], d[3];
+            const int i = (ty + 1) * S::SX + tx + 1;
+            mnew = sm.y.get(s, i);
+            nz = q >= 1 && q < p.N3 ? T(2) : T(1);  // cells on both sides along z
+            Vec<T> P;                               // 36 M1 M2 m / (dx dy)
+            if constexpr (sizeof(T) == 4) {
+                auto diff = [&](int o) { return vsub(sm.y.get(s, i + o), mnew); };
+                const Vec<T> X = vadd(diff(-1), diff(1)), Y = vadd(diff(-S::SX), diff(S::SX));
+                const Vec<T> C = vadd(vadd(diff(-S::SX - 1), diff(S::SX + 1)), vadd(diff(1 - S::SX), diff(S::SX - 1)));
+                fin = vfma(p.vs, C, vfma(p.v2, Y, vmul(p.v1, X)));     // share in the nodes of the planes beside
+                own = vfma(p.ws, C, vfma(p.w2[0], Y, vmul(p.w1[0], X)));  // share in the plane's own node
+                if (q >= 1) {
+                    const Vec<T> d = vsub(mnew, mc);
+                    dz = vfma(p.vz, d, vmul(p.vzl, d));
+                }
+                P = vfma(T(36), mnew, vfma(T(4), vadd(X, Y), C));
+            } else {
+                // row sums along x of rows n2 - 1 .. n2 + 1: a = 6 M1 m / dx, d = -dx K1 m
+                Vec<T> a[3], d[3];
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const int i = (ty + r) * S::SX + tx;
-                const Vec<T> c = sm.y.get(s, i + 1), e = vadd(sm.y.get(s, i), sm.y.get(s, i + 2));
-                a[r] = vfma(T(2) * nx, c, e);
-                d[r] = vfma(-nx, c, e);
-                if (r == 1) mnew = c;
+                for (int r = 0; r < 3; ++r) {
+                    const int j = i + (r - 1) * S::SX;
+                    const Vec<T> c = sm.y.get(s, j), e = vadd(sm.y.get(s, j - 1), sm.y.get(s, j + 1));
+                    a[r] = vfma(T(4), c, e);
+                    d[r] = vfma(T(-2), c, e);
+                }
+                const Vec<T> as = vadd(a[0], a[2]), ds = vadd(d[0], d[2]);
+                P = vfma(T(4), a[1], as);
+                const Vec<T> Q = vfma(p.cx, vfma(T(4), d[1], ds), vmul(p.cy, vfma(T(-2), a[1], as)));
+                fin = vfma(p.cz, P, Q);
+                own = vfma(T(2), Q, vmul(-p.cz, P));
             }
-            const T nz = q >= 1 && q < p.N3 ? T(2) : T(1);  // cells on both sides along z
-            const Vec<T> as = vadd(a[0], a[2]), ds = vadd(d[0], d[2]);
-            const Vec<T> P = vfma(T(2) * ny, a[1], as);     // M1 M2
-            const Vec<T> ka = vfma(-ny, a[1], as);          // -M1 K2
-            const Vec<T> kd = vfma(T(2) * ny, d[1], ds);    // -K1 M2
-            const Vec<T> Q = vfma(p.cx, kd, vmul(p.cy, ka));
-            fin = vfma(p.cz, P, Q);                         // share in the nodes of the planes beside
-            own = vfma(T(2) * nz, Q, vmul(-nz * p.cz, P));  // share in the plane's own node
             T px, py, pz;
             vget(P, px, py, pz);
             finR = p.e0 * px + p.e1 * py + p.e2 * pz;
@@ -158,13 +182,13 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
         const int z = q - 1;
         if (z >= z0 && active) {
             const int n = z * np + n2 * p.nn1 + n1;
-            T hx, hy, hz, dx, dy, dz, mx, my, mz;
-            vget(vadd(acc, fin), hx, hy, hz);
+            T hx, hy, hz, cx, cy, cz, mx, my, mz;
+            vget(vadd(acc, sizeof(T) == 4 ? vadd(dz, fin) : fin), hx, hy, hz);
             const T pe = p.can * (accR + finR);
             hx += p.e0 * pe;
             hy += p.e1 * pe;
             hz += p.e2 * pe;
-            vget(vadd(cc, ccur), dx, dy, dz);
+            vget(vadd(cc, ccur), cx, cy, cz);
             vget(mc, mx, my, mz);
             if (p.Msh && p.zee) {
                 T sx = 0, sy = 0, sz = 0;
@@ -178,25 +202,29 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
                         sz += p.Msh[2 * p.cs + c];
                     }
                 }
-                dx += sm.hf[3] * sx;
-                dy += sm.hf[3] * sy;
-                dz += sm.hf[3] * sz;
+                cx += sm.hf[3] * sx;
+                cy += sm.hf[3] * sy;
+                cz += sm.hf[3] * sz;
             }
-            hx += p.mu0V8 * dx;
-            hy += p.mu0V8 * dy;
-            hz += p.mu0V8 * dz;
+            cx *= p.mu0V8;
+            cy *= p.mu0V8;
+            cz *= p.mu0V8;
             if (p.hdmi) {
-                hx += p.hdmi[n];
-                hy += p.hdmi[p.ns + n];
-                hz += p.hdmi[2 * p.ns + n];
+                cx += p.hdmi[n];
+                cy += p.hdmi[p.ns + n];
+                cz += p.hdmi[2 * p.ns + n];
             }
-            if (!p.raw) {
-                // 1 / mass: the node's cells number nx ny nz (a power of two)
-                const T im = p.im1 * (z >= 1 && z < p.N3 ? T(0.5) : T(1)) * (nx == T(2) ? T(0.5) : T(1)) *
-                             (ny == T(2) ? T(0.5) : T(1));
-                hx *= im;
-                hy *= im;
-                hz *= im;
+            // (powers of two: the share of the node's cells in those of a node inside, and its inverse)
+            if (p.raw) {
+                const T f = (bx ? T(1) : T(0.5)) * (by ? T(1) : T(0.5));
+                hx = f * hx + cx;
+                hy = f * hy + cy;
+                hz = f * hz + cz;
+            } else {
+                const T fz = z >= 1 && z < p.N3 ? T(1) : T(2), im = p.im1 * fz * (bx ? T(1) : T(2)) * (by ? T(1) : T(2));
+                hx = fz * hx + im * cx;
+                hy = fz * hy + im * cy;
+                hz = fz * hz + im * cz;
                 if (p.zee) {
                     hx += sm.hf[0];
                     hy += sm.hf[1];
@@ -205,7 +233,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
             }
             err += (double)node_u_out<T, NK, M64>(p, n, hx, hy, hz, mx, my, mz, dt, dt64, true, ei);
         }
-        acc = vadd(up, own);
+        acc = vfma(nz, own, sizeof(T) == 4 ? vsub(up, dz) : up);
         accR = upR + ownR;
         up = fin;
         upR = finR;
@@ -345,21 +373,31 @@ static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *
 {
     const Geom &g = p.g;
     NodeUArgs<T> a = node_u_args<T>(p, y, out, y_next, sa, t);
-    a.cx = (T)p.ucx;
-    a.cy = (T)p.ucy;
-    a.cz = (T)p.ucz;
-    a.can = (T)p.uan;
-    a.im1 = (T)p.uim;
-    if (g.basis == 2) {
-        // one rounding for each constant
-        const double s = p.raw ? 1.0 : p.uim;
-        a.w1[0] = (T)(s * (4.0 * p.ucx - 2.0 * p.ucy));  // cells on both sides of the node along the other axis
-        a.w1[1] = (T)(s * (p.ucx - 2.0 * p.ucy));        // on one side
-        a.w2[0] = (T)(s * (4.0 * p.ucy - 2.0 * p.ucx));
-        a.w2[1] = (T)(s * (p.ucy - 2.0 * p.ucx));
-        a.ws = (T)(s * (p.ucx + p.ucy));
-        a.can = (T)(s * p.uan);
-        a.im1 = (T)s;
+    // weights of the sums of differences, one rounding each
+    if (g.basis == 3) {
+        const double f = p.raw ? 1.0 : p.uim / 8.0, cx = f * p.ucx, cy = f * p.ucy, cz = f * p.ucz;
+        a.cx = (T)cx;
+        a.cy = (T)cy;
+        a.cz = (T)cz;
+        a.w1[0] = (T)(8.0 * cx - 4.0 * cy - 4.0 * cz);
+        a.w2[0] = (T)(8.0 * cy - 4.0 * cx - 4.0 * cz);
+        a.ws = (T)(2.0 * cx + 2.0 * cy - cz);
+        a.v1 = (T)(4.0 * cx - 2.0 * cy + 4.0 * cz);
+        a.v2 = (T)(4.0 * cy - 2.0 * cx + 4.0 * cz);
+        a.vs = (T)(cx + cy + cz);
+        a.vz = (T)(36.0 * cz);
+        a.vzl = (T)(36.0 * cz - (double)a.vz);
+        a.can = (T)(f * p.uan);
+        a.im1 = (T)f;
+    } else {
+        const double f = p.raw ? 1.0 : p.uim, cx = f * p.ucx, cy = f * p.ucy;
+        a.w1[0] = (T)(4.0 * cx - 2.0 * cy);  // cells on both sides of the node along the other axis
+        a.w1[1] = (T)(cx - 2.0 * cy);        // on one side
+        a.w2[0] = (T)(4.0 * cy - 2.0 * cx);
+        a.w2[1] = (T)(cy - 2.0 * cx);
+        a.ws = (T)(cx + cy);
+        a.can = (T)(f * p.uan);
+        a.im1 = (T)f;
     }
     int blocks = 0;
     uniform_grid<T>(g, a, &blocks);

@@ -123,11 +123,15 @@ struct NodeUArgs {
     int nn1, nn2, nn3, N1, N2, N3, ns, cs;
     int bxn, full, chunks, zc;  // blocks b < full walk tile b over all planes; the other tiles are split into
                                 // `chunks` blocks of zc planes
-    T cx, cy, cz, can;          // 2 A x element constants of the axes; 2 Ku V / 216 (2D basis: / 36 per layer)
-    T w1[2], w2[2], ws;         // 2D basis: exchange weights of the sums of differences (node_uniform.cu); these and can
-                                // are over the mass of a node with one cell column unless raw (im1 = 1 then)
+    // uniform materials (node_uniform.cu), over a nodal mass unless raw.  2D basis, of a node with one cell column: exchange
+    // weights w of the sums of differences, by the cells along the other axis.  3D basis, of a node inside: FP32 the same
+    // in the node's own plane (w, index 0) and in the planes beside it (v), and of the difference along z (vz, and vzl:
+    // what its rounding left); FP64 2 A x element constants of the axes (c)
+    T w1[2], w2[2], ws;
+    T can;                      // 2 Ku V / 216 (2D basis: / 36 per layer)
+    T v1, v2, vs, vz, vzl, cx, cy, cz;
     T e0, e1, e2;
-    T im1, mu0V8;               // 1 / (mu0 V/8 Ms), mu0 V/8 (2D basis: 1 / (mu0 V/4 Ms N3), mu0 V/4)
+    T im1, mu0V8;               // 1 / (mu0 V/8 Ms) or 1 when raw, mu0 V/8 (2D basis: 1 / (mu0 V/4 Ms N3), mu0 V/4)
     T gam, alpha;
     const T *y, *MsH, *Msh, *hdmi;
     T *out, *y_next;

@@ -49,3 +49,12 @@ def test_2d_basis(oracle_mod, nmgb, shape, dx, theta):
     p = inp.random_problem(np.random.default_rng(1), shape, dx=dx, heterogeneous=False)
     err = _errors(nmgb, oracle_mod, p, (shape[0] + 1, shape[1] + 1, 1), theta, 2)
     _check(err, max(dx[0] / dx[1], dx[1] / dx[0]) ** 2, theta)
+
+
+@pytest.mark.parametrize("theta", [0.1, 0.01, 0.003])
+@pytest.mark.parametrize("shape, dx", [((70, 9, 5), (3e-9, 3e-9, 3e-9)), ((40, 30, 2), (5e-9, 5e-9, 1e-9)),
+                                       ((33, 20, 40), (2e-9, 2.5e-9, 3e-9)), ((60, 40, 1), (2.5e-9, 2.5e-9, 3e-9))])
+def test_3d_basis(oracle_mod, nmgb, shape, dx, theta):
+    p = inp.random_problem(np.random.default_rng(2), shape, dx=dx, heterogeneous=False)
+    err = _errors(nmgb, oracle_mod, p, p.nodes, theta, 3)
+    _check(err, (max(dx) / min(dx)) ** 2, theta)
