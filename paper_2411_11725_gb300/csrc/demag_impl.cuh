@@ -34,7 +34,7 @@ constexpr int kMaxThreads = 512;
 template <typename T, int LG = 0>
 constexpr int kMinBlocks = sizeof(T) == 4 ? 2 : 1;
 // values per thread per FFT stage in the y passes: radix-16 stages for the FP32 lengths where they save a stage
-// (2^10 and 2^11; 2^7 and 2^8: 12.3 against 14.8 us a pass at 512x100x8, 14.0 / 17.7 at 1000x60x12, 8.3 / 9.4 at
+// (2^10 and 2^11; 2^7 and 2^8: 12.5 against 14.8 us a pass at 512x100x8, 14.2 / 17.7 at 1000x60x12, 8.5 / 9.4 at
 // 131x67x5)
 template <typename T, int LG>
 constexpr int kYEpt = (sizeof(T) == 4 && (LG >= 10 || LG == 7 || LG == 8)) ? 16 : 8;
@@ -827,13 +827,14 @@ __global__ void __launch_bounds__(ZRTile<T, LG>::THREADS, sizeof(T) == 4 && LG =
         }
     };
     if constexpr (S > 1) twist(std::integral_constant<int, -1>{});
+    // (two parts: the radix-4 first level takes 116 instead of 107 us at 512x512x16)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) f3::dft_reg<T, D, -1>(v[c]);
+    for (int c = 0; c < 3; ++c) f3::dft_reg<T, D, -1, S != 2>(v[c]);
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
     z_product<T, LG, S>(v, ten + rw * G + (lane & 15), KY * G, (H + 1) * KY * G, r, mir ? T(-1) : T(1));
 #pragma unroll
-    for (int c = 0; c < 3; ++c) f3::dft_reg<T, D, +1>(v[c]);
+    for (int c = 0; c < 3; ++c) f3::dft_reg<T, D, +1, S != 2>(v[c]);
     if constexpr (S > 1) twist(std::integral_constant<int, +1>{});
     if constexpr (S == 1) {
         if (!valid) return;
@@ -1136,11 +1137,15 @@ static void plan_yz(const Geom &g, DemagPlan &p)
     // as many threads as a radix-8 stage has butterflies
     const int want = (((3 * g.N3) << lgG) * g.P2 / 8 + 31) / 32 * 32;
     p.yz_threads = want < 128 ? 128 : (want > kYZThreads<T> ? kYZThreads<T> : want);
-    // as few stages as radix 8 (FP64 and short lines) or 16 allows, split evenly, the larger radices first
-    const int RM = sizeof(T) == 4 && g.lgP2 > 7 ? 4 : 3;
+    // as few stages as radix 8 (FP64 and lines up to 2^9) or 16 allows, split evenly, the larger radices last, where a
+    // stage has no twiddles (512x512x1 step 262 -> 258 us, and more accurate, than with them first).  2^8 in three stages
+    // with table twiddles: two of radix 16 save 2 us of 131 a step at 200x100x1, but cost a quarter of the accuracy with
+    // products and a tenth with table values (error of a random state's demag field at 30x100x1: 1.50e-7 and 1.30e-7
+    // against 1.16e-7).
+    const int RM = sizeof(T) == 4 && g.lgP2 > 8 ? 4 : 3;
     p.yz_plan = 0;
     for (int left = g.lgP2, s = 0, ns = div_up(left, RM); left > 0; ++s, --ns) {
-        const int lr = div_up(left, ns);
+        const int lr = left / ns;
         p.yz_plan |= (unsigned)lr << (4 * s);
         left -= lr;
     }

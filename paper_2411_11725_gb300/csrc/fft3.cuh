@@ -110,11 +110,32 @@ __device__ __forceinline__ Cx<T> cdiff(Cx<T> a, Cx<T> b)
 }
 
 // x_k <- sum_j x_j e^{DIR 2 pi i jk / R}: radix-2 decimation-in-frequency network, X_k in x[bitrev(k)]
-template <typename T, int R, int DIR, bool PK = true>
+// R4: R = 16 takes its first two levels as one of radix 4: a value meets one inexact factor (W_16^j, W_16^2j or W_16^3j)
+// instead of up to two, eight such products instead of ten (demag field of a random state, 30x100x8 cells, FP32: error
+// 1.43e-7 -> 1.32e-7)
+template <typename T, int R, int DIR, bool PK = true, bool R4 = true>
 __device__ __forceinline__ void dft(Cx<T> *x)
 {
+    if constexpr (R == 16 && R4) {
 #pragma unroll
-    for (int h = R / 2; h >= 1; h >>= 1) {
+        for (int j = 0; j < 4; ++j) {
+            auto w = [&](Cx<T> v, int q) {  // v W_16^q
+                if (q == 0) return v;
+                if (q == 4) return mul_si(v, DIR);
+                const T cq = kC16<T>[q & 15], sq = DIR > 0 ? kC16<T>[(q - 4) & 15] : -kC16<T>[(q - 4) & 15];
+                return cx<T>(v.x * cq - v.y * sq, v.x * sq + v.y * cq);
+            };
+            const Cx<T> a = x[j], b = x[j + 4], c = x[j + 8], d = x[j + 12];
+            const Cx<T> t0 = PK ? csum(a, c) : a + c, t1 = PK ? cdiff(a, c) : a - c;
+            const Cx<T> t2 = PK ? csum(b, d) : b + d, t3 = mul_si(PK ? cdiff(b, d) : b - d, DIR);
+            x[j] = PK ? csum(t0, t2) : t0 + t2;
+            x[j + 4] = w(PK ? cdiff(t0, t2) : t0 - t2, 2 * j);
+            x[j + 8] = w(PK ? csum(t1, t3) : t1 + t3, j);
+            x[j + 12] = w(PK ? cdiff(t1, t3) : t1 - t3, 3 * j);
+        }
+    }
+#pragma unroll
+    for (int h = R == 16 && R4 ? 2 : R / 2; h >= 1; h >>= 1) {
 #pragma unroll
         for (int s = 0; s < R; s += 2 * h) {
 #pragma unroll
@@ -196,7 +217,7 @@ __device__ __forceinline__ Cx<T> rot(Cx<T> v, int k)
 
 // A whole transform of R <= 32 values held by one thread: X_k = sum_j x_j e^{DIR 2 pi i jk / R}, X_k in
 // x[bitrev(k)].  R = 32 splits into one radix-2 decimation-in-frequency level and two 16-point networks.
-template <typename T, int R, int DIR>
+template <typename T, int R, int DIR, bool R4 = true>
 __device__ __forceinline__ void dft_reg(Cx<T> *x);
 
 // v * conj^(DIR>0)(w): the twiddle table holds e^{-2 pi i k / 2^twlg}
@@ -209,7 +230,7 @@ __device__ __forceinline__ Cx<T> twmul(Cx<T> v, Cx<T> w)
 
 // packed additions in the in-register transforms too (measured faster than scalar ones)
 constexpr bool kRegPacked = true;
-template <typename T, int R, int DIR>
+template <typename T, int R, int DIR, bool R4>
 __device__ __forceinline__ void dft_reg(Cx<T> *x)
 {
     static_assert(R >= 1 && R <= 32 && (R & (R - 1)) == 0, "in-register transforms of 1 to 32 values");
@@ -223,7 +244,7 @@ __device__ __forceinline__ void dft_reg(Cx<T> *x)
         dft<T, 16, DIR, kRegPacked>(x);
         dft<T, 16, DIR, kRegPacked>(x + 16);
     } else if constexpr (R > 1) {
-        dft<T, R, DIR, kRegPacked>(x);
+        dft<T, R, DIR, kRegPacked, R4>(x);
     }
 }
 
@@ -298,11 +319,13 @@ __device__ __forceinline__ void stage(Cx<T> *__restrict__ buf, int nl_rt, const 
         const int k = j & (NS - 1);
         if (NS > 1) {
             const int kk = k << sh;
-            if constexpr (R == 16 && sizeof(T) == 4) {
+            if constexpr (R == 16 && sizeof(T) == 4 && LG >= 10) {
                 // w^r for r < 16 from the four table values w, w^2, w^4, w^8 (four loads in flight together
                 // instead of fifteen; the other powers are at most three products away, a few roundings).
                 // FP32 only: the FP64 passes are bound by the FP64 rate, where the products cost more than
-                // the loads they save.
+                // the loads they save.  Lines of 2^10 and more only: shorter ones lost a fifth of their accuracy
+                // (demag field of a random state, 30x100x8 cells: error 1.66e-7, 1.32e-7 with table values, which
+                // cost 0.1-0.3 us a y pass and 5 us a step on 256x256x8).
                 Cx<T> w[16];
                 w[1] = tw[kk];
                 w[2] = tw[2 * kk];
