@@ -904,7 +904,8 @@ static void enqueue_y2(nm_mesh M)
 int ensure_y2(nm_mesh M, int method)
 {
     if (method != NM_DP54) {
-        M->y2_valid = false;  // (RK4 stages use the buffer)
+        // RK4 moves the state, and its stages use both buffers
+        M->k1_valid = M->y2_valid = false;
         return NM_OK;
     }
     if (M->y2_valid) return NM_OK;

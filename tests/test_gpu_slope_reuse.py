@@ -1,0 +1,51 @@
+"""The slope that a Dormand-Prince run keeps for its next step is formed anew whenever the state or the field behind it
+has changed.  Each sequence against a fresh mesh that starts from the state in between; the same kernels on the same
+values, so the states agree bit for bit.
+"""
+import numpy as np
+import pytest
+
+import nm_inputs as inp
+from helpers import gpu_mesh
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nmgb():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2411_11725_gb300 as nmgb
+    nmgb.load()
+    return nmgb
+
+
+def _problem(heterogeneous):
+    p = inp.random_problem(np.random.default_rng(4), (9, 6, 3), heterogeneous=heterogeneous)
+    p.h_freq = 0.0
+    p.h_cell = None
+    return p
+
+
+def _restart(nmgb, p, precision, me):
+    """a new mesh at the resident state, time and step of me"""
+    other = gpu_mesh(nmgb, p, precision)
+    other.set_state(*me.get_state())
+    return other
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("heterogeneous", [False, True])
+def test_rk4_between_dp5_runs(nmgb, precision, heterogeneous):
+    p = _problem(heterogeneous)
+    me = gpu_mesh(nmgb, p, precision)
+    me.set_state(p.m0, 0.0, 1e-13)
+    me.run_steps(2, nmgb.DP54)
+    me.run_steps(3, nmgb.RK4)
+    ref = _restart(nmgb, p, precision, me)
+    for mesh in (me, ref):
+        mesh.run_steps(2, nmgb.DP54)
+    assert np.array_equal(me.get_state()[0], ref.get_state()[0])
+    me.close()
+    ref.close()
