@@ -509,6 +509,7 @@ extern "C" int nm_set_field(nm_mesh M, int kind, const double *data, const doubl
     if (!M) return fail(NM_ERR_ARG, "mesh is NULL");
     if (!isfinite(freq_hz) || !isfinite(phase)) return fail(NM_ERR_ARG, "freq/phase must be finite");
     free_graphs(M);
+    M->k1_valid = false;  // (the slope of the old field)
     if (kind == NM_FIELD_HEXT_UNIFORM) {
         if (!amp) return fail(NM_ERR_ARG, "amp is NULL");
         for (int k = 0; k < 3; ++k) {

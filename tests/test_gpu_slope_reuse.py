@@ -49,3 +49,27 @@ def test_rk4_between_dp5_runs(nmgb, precision, heterogeneous):
     assert np.array_equal(me.get_state()[0], ref.get_state()[0])
     me.close()
     ref.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("kind", ["uniform", "cell", "cell off"])
+def test_field_changed_between_dp5_runs(nmgb, precision, kind):
+    p = _problem(False)
+    h_cell = np.random.default_rng(5).standard_normal(p.n + (3,)) * 1e5
+    if kind == "cell off":
+        p.h_cell = h_cell
+    me = gpu_mesh(nmgb, p, precision)
+    me.set_state(p.m0, 0.0, 1e-13)
+    me.run_steps(2, nmgb.DP54)
+    if kind == "uniform":
+        p.h_uniform = (2e5, -1e5, 3e5)
+        me.set_uniform_field(p.h_uniform)
+    else:
+        p.h_cell = h_cell if kind == "cell" else None
+        me.set_zeeman(p.h_uniform, 0.0, p.h_phase, p.h_cell, p.cell_freq, p.cell_phase)
+    ref = _restart(nmgb, p, precision, me)
+    for mesh in (me, ref):
+        mesh.run_steps(2, nmgb.DP54)
+    assert np.array_equal(me.get_state()[0], ref.get_state()[0])
+    me.close()
+    ref.close()
