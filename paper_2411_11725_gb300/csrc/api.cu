@@ -938,6 +938,8 @@ extern "C" int nm_llg_step(nm_mesh M, int method, double *t, double *dt, double 
     if (!(*dt > 0) || !isfinite(*dt) || !isfinite(*t)) return fail(NM_ERR_ARG, "dt must be positive and finite");
     if ((rc = pull_ctl(M))) return rc;
     StepCtl *h = M->hctl;
+    // the kept first slope belongs to the resident time
+    if (h->t != *t && (M->hu_freq != 0.0 || (M->has_hcell && M->hc_freq != 0.0))) M->k1_valid = false;
     h->t = *t;
     h->dt = *dt;
     h->rtol = rtol;

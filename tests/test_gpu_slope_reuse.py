@@ -73,3 +73,21 @@ def test_field_changed_between_dp5_runs(nmgb, precision, kind):
     assert np.array_equal(me.get_state()[0], ref.get_state()[0])
     me.close()
     ref.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_step_from_another_time(nmgb, precision):
+    """With a field that oscillates, a step from a time other than the resident one has another first slope."""
+    p = _problem(False)
+    p.h_uniform, p.h_freq = (3e6, 0.0, 0.0), 1e12
+    me = gpu_mesh(nmgb, p, precision)
+    me.set_state(p.m0, 0.0, 1e-14)
+    me.run_steps(1, nmgb.DP54)
+    m, t, _ = me.get_state()
+    ref = gpu_mesh(nmgb, p, precision)
+    ref.set_state(m, t + 3e-13, 1e-14)
+    for mesh in (me, ref):
+        assert mesh.llg_step(nmgb.DP54, t + 3e-13, 1e-14)[0]
+    assert np.array_equal(me.get_state()[0], ref.get_state()[0])
+    me.close()
+    ref.close()
