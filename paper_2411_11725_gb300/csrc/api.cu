@@ -1090,6 +1090,7 @@ extern "C" int nm_profile_step(nm_mesh M, int method, int reps, double rtol, dou
     h->status = NM_OK;
     if ((rc = push_ctl(M))) return rc;
     if ((rc = ensure_k1(M, method))) return rc;
+    if ((rc = ensure_mf(M))) return rc;
     free_graphs(M);  // graphs hold no markers
     std::vector<double> acc;
     int nk = 0;

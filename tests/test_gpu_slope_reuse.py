@@ -91,3 +91,23 @@ def test_step_from_another_time(nmgb, precision):
     assert np.array_equal(me.get_state()[0], ref.get_state()[0])
     me.close()
     ref.close()
+
+
+@pytest.mark.parametrize("method", ["RK4", "DP54"])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_profiled_step_first(nmgb, precision, method):
+    """The first use of a state: the FP32 copy of the one before must not be used."""
+    p = _problem(False)
+    out = []
+    for profiled in (True, False):
+        me = gpu_mesh(nmgb, p, precision)
+        me.set_state(np.roll(p.m0, 1, axis=0), 0.0, 1e-13)
+        me.run_steps(1, getattr(nmgb, method))
+        me.set_state(p.m0, 0.0, 1e-13)
+        if profiled:
+            me.profile_step(getattr(nmgb, method), reps=1)
+        else:
+            me.run_steps(1, getattr(nmgb, method))
+        out.append(me.get_state()[0])
+        me.close()
+    assert np.array_equal(out[0], out[1])
