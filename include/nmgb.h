@@ -245,6 +245,8 @@ int nm_h_eff_vjp(nm_mesh mesh, const void *m, const void *v, unsigned terms, dou
  * with grad_Ms, grad_m0 and grad_h all NULL only the forward run and its loss are computed;
  * grad_h (3 values: dL/dh of the uniform applied field amplitude of nm_set_field, the design variable of
  * the paper's field-angle inverse problem, section "Inverse Problems").
+ * Where the device has the room (3 nodal and, with the demag term, 3 cell values per stage), the reverse
+ * sweep keeps a step's fields for its transpose products; otherwise it forms them twice.
  * The resident state ends at t_end.  Synchronises.  Errors: as nm_run_until, NM_ERR_OOM. */
 int nm_adjoint_run(nm_mesh mesh, int method, double t_end, double rtol, double atol, double dt0,
                    double sample_dt, const double *weight, const double *target, int include_initial,
@@ -264,8 +266,8 @@ int nm_adjoint_run(nm_mesh mesh, int method, double t_end, double rtol, double a
  * NULL = 0).  Outputs (HOST FP64, each may be NULL except loss): loss; grad_m0 = a(t0) (nodal vector
  * field); grad_Ms = u(t0) for the cell Ms map (cell scalar field); grad_h = u(t0) for the uniform
  * applied field amplitude (3 values); m0_rec = the reconstructed m(t0) (nodal vector field).  m is
- * renormalised after each step, forward and backward, as set by nm_set_integrator.  The resident state
- * ends at t_end.  Synchronises.  Errors: NM_ERR_ARG (n_steps < 1, t_end <= t0, NULL weight or loss),
+ * renormalised after each step, forward and backward, as set by nm_set_integrator.  Keeps fields as
+ * nm_adjoint_run does.  The resident state ends at t_end.  Synchronises.  Errors: NM_ERR_ARG (n_steps < 1, t_end <= t0, NULL weight or loss),
  * NM_ERR_STATE (no material or state), NM_ERR_OOM, NM_ERR_CUDA. */
 int nm_adjoint_continuous(nm_mesh mesh, double t_end, long n_steps, const double *weight, const double *target,
                           double *loss, double *grad_m0, double *grad_Ms, double *grad_h, double *m0_rec);

@@ -161,10 +161,37 @@ template <typename T>
 struct AdjBufs {
     T *Y[8];      // stage inputs y_1..y_S
     T *YB[8];     // stage adjoints ybar_1..ybar_S
-    T *F[8], *H[8];  // fields at the stage inputs: nodal, demag cell field
+    T *F[8], *H[8];  // fields at the stage inputs: nodal, demag cell field (keep_fields; NULL: formed again where needed)
     T *mu, *lamT;
     double *lam, *lamt, *partials, *scalar;
 };
+
+// Room for the fields of a step's stages, F and H (H with the demag term alone), for a reverse sweep.  All of it or none:
+// a call that lacks the memory forms each field twice instead (run_stages, and llg_vjp on its own workspaces), as much
+// memory less as the fields take: at 1024x1024x32 in FP32 3.3 GB with RK4, 4.9 GB with Dormand-Prince.
+template <typename T>
+void keep_fields(nm_mesh M, const Tableau &tb, AdjBufs<T> &A, std::vector<void *> &owned)
+{
+    const size_t first = owned.size();
+    auto get = [&](T **p, size_t n) {
+        if (cudaMallocAsync((void **)p, n * sizeof(T), M->st) == cudaSuccess) {
+            owned.push_back(*p);
+            return true;
+        }
+        cudaGetLastError();
+        *p = nullptr;
+        return false;
+    };
+    for (int s = tb.fsal ? 1 : 0; s < tb.S; ++s) {
+        if (get(&A.F[s], 3 * M->g.ns) && (!(M->terms & NM_DEMAG) || get(&A.H[s], 3 * M->g.cs))) continue;
+        while (owned.size() > first) {
+            cudaFreeAsync(owned.back(), M->st);
+            owned.pop_back();
+        }
+        for (int i = 0; i < tb.S; ++i) A.F[i] = A.H[i] = nullptr;
+        return;
+    }
+}
 
 // t and dt of the next step, written on the device: no read-back, so the host enqueues the reverse sweep ahead of the GPU
 // (with a pull and a push of the control block per step, a gradient over 24 RK4 steps on 256x64x1 cells took 15.4 instead
@@ -218,11 +245,12 @@ void run_stages(nm_mesh M, const Tableau &tb, AdjBufs<T> &A)
 }
 
 // The same for the step from t with size dt (also in ctl) that is walked backwards next: its fields stay in
-// A.F and A.H for the transpose products, which would otherwise evaluate each of them again (a gradient over 24
+// A.F and A.H, where there is room for them, for the transpose products, which would otherwise evaluate each of them again (a gradient over 24
 // RK4 steps on 256x64x1 cells 22.4 -> 16.4 ms, with the two fields that heff_vjp_core saves).
 template <typename T>
 void run_stages_kept(nm_mesh M, const Tableau &tb, AdjBufs<T> &A, double t, double dt)
 {
+    if (!A.F[tb.S - 1]) return run_stages<T>(M, tb, A);
     const Geom &g = M->g;
     const double gam = M->gamma / (1.0 + M->alpha * M->alpha);
     KList in{};
@@ -269,11 +297,16 @@ int finish_step(nm_mesh M, const Tableau &tb)
 }
 
 // ybar = J_f(y)^T u at time t (LLG right-hand side), u = sum lu, gMs += its Ms part; F and H: the nodal and
-// demag cell fields at y
+// demag cell fields at y (F NULL: formed here)
 template <typename T>
 void llg_vjp(nm_mesh M, const T *y, double t, const LinComb &lu, const T *F, const T *H, T *ybar)
 {
     const Geom &g = M->g;
+    if (!F) {
+        field_at<T>(M, y, M->terms, t, (T *)M->vj_h, (T *)M->vj_H);
+        F = (const T *)M->vj_h;
+        H = (const T *)M->vj_H;
+    }
     // the uniform applied field adds h s(t) to H at every magnetic node: dL/dh += s(t) sum_n q_n
     double *gh = (M->terms & NM_ZEE) ? M->vj_gh : nullptr;
     launch_llg_vjp_local<T>(g, y, F, lu, (const T *)M->inv_mass, M->gamma / (1.0 + M->alpha * M->alpha), M->alpha,
@@ -406,8 +439,6 @@ int adjoint_run_t(nm_mesh M, int method, double t_end, double rtol, double atol,
     for (int s = 0; s < tb.S; ++s) {
         ADJ_TRY(galloc((void **)&A.Y[s], nb3));
         ADJ_TRY(galloc((void **)&A.YB[s], nb3));
-        ADJ_TRY(galloc((void **)&A.F[s], nb3));
-        ADJ_TRY(galloc((void **)&A.H[s], 3 * g.cs * sizeof(T)));
     }
     ADJ_TRY(galloc((void **)&A.mu, nb3));
     ADJ_TRY(galloc((void **)&A.lamT, nb3));
@@ -543,6 +574,7 @@ int adjoint_run_t(nm_mesh M, int method, double t_end, double rtol, double atol,
         ADJ_TRY(galloc((void **)&seg_m[i], nd3));
         if (tb.fsal) ADJ_TRY(galloc((void **)&seg_k[i], nb3));
     }
+    keep_fields<T>(M, tb, A, owned);  // (last: what is left)
     const long nseg = (n + C - 1) / C;
     for (long seg = nseg - 1; seg >= 0; --seg) {
         const long s0 = seg * C, s1 = (s0 + C < n) ? s0 + C : n;
@@ -576,12 +608,11 @@ int adjoint_run_t(nm_mesh M, int method, double t_end, double rtol, double atol,
         KList none{};
         ADJ_TRY(set_ctl(M, t0, dt));
         launch_stage_input<T>(g, M->m, none, M->ctl, A.Y[0], M->st);
-        field_at<T>(M, A.Y[0], M->terms, t0, A.F[0], A.H[0]);
         LinComb lu{};
         lu.pt[0] = A.mu;
         lu.at[0] = 1.0;
         lu.nt = 1;
-        llg_vjp<T>(M, A.Y[0], t0, lu, A.F[0], A.H[0], A.YB[0]);
+        llg_vjp<T>(M, A.Y[0], t0, lu, nullptr, nullptr, A.YB[0]);
         LinComb lc{};
         lc.pd[0] = A.lam;
         lc.ad[0] = 1.0;
@@ -711,8 +742,6 @@ int continuous_adjoint_t(nm_mesh M, double t_end, long n, const double *weight, 
     for (int s = 0; s < tb.S; ++s) {
         CA_TRY(galloc((void **)&A.Y[s], nb3));
         CA_TRY(galloc((void **)&A.YB[s], nb3));  // ka_s
-        CA_TRY(galloc((void **)&A.F[s], nb3));
-        CA_TRY(galloc((void **)&A.H[s], 3 * g.cs * sizeof(T)));
     }
     T *YB = nullptr;
     double *a = nullptr, *as = nullptr, *W = nullptr, *tgt = nullptr, *tmp = nullptr, *m_end = nullptr;
@@ -741,6 +770,8 @@ int continuous_adjoint_t(nm_mesh M, double t_end, long n, const double *weight, 
         M->vj_gh = gh;
     }
     CUDA_TRY(cudaMemsetAsync(M->vj_gMs, 0, g.cs * sizeof(double), M->st));
+
+    keep_fields<T>(M, tb, A, owned);
 
     // forward: n RK4 steps to t_end
     CA_TRY(pull_ctl(M));
