@@ -268,7 +268,7 @@ int nm_adjoint_run(nm_mesh mesh, int method, double t_end, double rtol, double a
  * applied field amplitude (3 values); m0_rec = the reconstructed m(t0) (nodal vector field).  m is
  * renormalised after each step, forward and backward, as set by nm_set_integrator.  Keeps fields as
  * nm_adjoint_run does.  The resident state ends at t_end.  Synchronises.  Errors: NM_ERR_ARG (n_steps < 1, t_end <= t0, NULL weight or loss),
- * NM_ERR_STATE (no material or state), NM_ERR_OOM, NM_ERR_CUDA. */
+ * NM_ERR_STATE (no material or state), NM_ERR_OOM, NM_ERR_TIMEOUT (as nm_llg_step), NM_ERR_CUDA. */
 int nm_adjoint_continuous(nm_mesh mesh, double t_end, long n_steps, const double *weight, const double *target,
                           double *loss, double *grad_m0, double *grad_Ms, double *grad_h, double *m0_rec);
 

@@ -193,6 +193,14 @@ void keep_fields(nm_mesh M, const Tableau &tb, AdjBufs<T> &A, std::vector<void *
     }
 }
 
+// Status of the device work enqueued so far (synchronises): a demag pass whose bounded wait ran out
+int check_status(nm_mesh M, const char *what)
+{
+    int rc = pull_ctl(M);
+    if (rc) return rc;
+    return M->hctl->status == NM_OK ? NM_OK : fail(M->hctl->status, "%s failed (status %d)", what, M->hctl->status);
+}
+
 // t and dt of the next step, written on the device: no read-back, so the host enqueues the reverse sweep ahead of the GPU
 // (with a pull and a push of the control block per step, a gradient over 24 RK4 steps on 256x64x1 cells took 15.4 instead
 // of 14.3 ms)
@@ -478,8 +486,11 @@ int adjoint_run_t(nm_mesh M, int method, double t_end, double rtol, double atol,
         release_all();
         return fail(NM_ERR_ARG, "need t_end > t and a positive step");
     }
+    h->status = NM_OK;
+    ADJ_TRY(push_ctl(M));
     M->k1_valid = false;
     ADJ_TRY(ensure_k1(M, method));  // k1_0 = f(m_0)
+    ADJ_TRY(check_status(M, "first slope"));
     std::vector<double> ts, dts;
     std::vector<char> sample_end;
     std::vector<double *> ck_m;
@@ -645,7 +656,7 @@ int adjoint_run_t(nm_mesh M, int method, double t_end, double rtol, double atol,
     ADJ_TRY(set_ctl(M, t_final, dt_final));
     M->k1_valid = false;
     CHECK_LAUNCH();
-    CUDA_TRY(cudaStreamSynchronize(M->st));
+    ADJ_TRY(check_status(M, "reverse sweep"));
     release_all();
     CUDA_TRY(cudaStreamSynchronize(M->st));
     *loss_out = loss;
@@ -771,6 +782,8 @@ int continuous_adjoint_t(nm_mesh M, double t_end, long n, const double *weight, 
     }
     CUDA_TRY(cudaMemsetAsync(M->vj_gMs, 0, g.cs * sizeof(double), M->st));
 
+    M->hctl->status = NM_OK;
+    CA_TRY(push_ctl(M));
     keep_fields<T>(M, tb, A, owned);
 
     // forward: n RK4 steps to t_end
@@ -857,7 +870,7 @@ int continuous_adjoint_t(nm_mesh M, double t_end, long n, const double *weight, 
     CA_TRY(set_ctl(M, t_end, dt));
     M->k1_valid = false;
     CHECK_LAUNCH();
-    CUDA_TRY(cudaStreamSynchronize(M->st));
+    CA_TRY(check_status(M, "adjoint integration"));
     release_all();
     CUDA_TRY(cudaStreamSynchronize(M->st));
     return NM_OK;

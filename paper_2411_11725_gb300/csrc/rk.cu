@@ -466,7 +466,6 @@ __global__ void k_set_ctl(StepCtl *ctl, double t, double dt)
     ctl->dt = dt;
     ctl->t_end = 0.0;
     ctl->done = 0;
-    ctl->status = NM_OK;
 }
 
 // Volume-weighted mean of m: per-block partial sums of (w m_x, w m_y, w m_z, w).

@@ -41,7 +41,7 @@ void launch_dp5_update(const Geom &g, double *m, const KList &kb, const T *k7, T
 template <typename T>
 void launch_rk4_update(const Geom &g, double *m, const KList &kb, StepCtl *ctl, int renorm, cudaStream_t st,
                        float *mf = nullptr);
-// t and dt of the step control, with no end time, not done and no error
+// t and dt of the step control, with no end time and not done (the status word stays: a wait that ran out before)
 void launch_set_ctl(StepCtl *ctl, double t, double dt, cudaStream_t st);
 template <typename T>
 void launch_mean(const Geom &g, const double *m, const T *vol, double *partials, double *out, cudaStream_t st);
