@@ -45,13 +45,13 @@ constexpr int pow2_floor_c(int v)
     return p;
 }
 // Compile-time tile of the z convolution for lines of 2^LG: G kx columns x KY octant rows (each with its
-// mirror) x 3 components, 16 values per thread for short FP32 lines (128-byte rows), 8 otherwise.
+// mirror) x 3 components, 8 values per thread, 64-byte rows where they fit (lines beyond the register tiles: ZRTile).
 template <typename T, int LG>
 struct ZTile {
     static constexpr int P3 = 1 << LG;
-    static constexpr int EPT = (sizeof(T) == 4 && LG <= 5) ? 16 : 8;
+    static constexpr int EPT = 8;
     static constexpr int BUDGET = EPT * kMaxThreads<T>;
-    static constexpr int G0 = EPT == 16 ? 16 : (int)(64 / sizeof(Cx<T>));
+    static constexpr int G0 = (int)(64 / sizeof(Cx<T>));
     static constexpr int fit_g(int g) { return (g > 1 && 6 * g * P3 > BUDGET) ? fit_g(g / 2) : g; }
     static constexpr int G = fit_g(G0);
     static constexpr int KY = pow2_floor_c(BUDGET / (6 * G * P3)) > 0 ? pow2_floor_c(BUDGET / (6 * G * P3)) : 1;
@@ -522,7 +522,7 @@ __device__ __forceinline__ int z_row_ky(const Geom &g, int a20, int r)
 // Stage a z tile in shared memory with cp.async: the N3 spectrum rows of its 3 x 2KY lines of G kx
 // columns (element z of line l = (c * 2KY + r) * G + g at buf[z * nl + l]), then the tensor slice
 // [component][a3][row][kx] behind the NL * P3 spectrum values; ends with a barrier.
-template <typename T, int G, int KY, int P3, bool TENSOR = true>
+template <typename T, int G, int KY, int P3>
 __device__ __forceinline__ void z_tile_load(const Geom &g, const DemagBufs<T> &b, Cx<T> *buf, int kx0, int a20)
 {
     constexpr int R2 = 2 * KY, nl = 3 * R2 * G, H3 = P3 / 2 + 1;
@@ -541,7 +541,7 @@ __device__ __forceinline__ void z_tile_load(const Geom &g, const DemagBufs<T> &b
     T *ten = reinterpret_cast<T *>(buf + nl * P3);
     constexpr int trowb = G * (int)sizeof(T);
     constexpr int tcb = trowb >= 16 ? 16 : trowb, tch = trowb / tcb;
-    for (int t = threadIdx.x; TENSOR && t < 6 * H3 * KY * tch; t += blockDim.x) {
+    for (int t = threadIdx.x; t < 6 * H3 * KY * tch; t += blockDim.x) {
         const int row = t / tch, ch = t - row * tch;
         const int rr = row % KY, kq = row / KY, a3 = kq % H3, comp = kq / H3;
         const int a2 = a20 + rr;
@@ -1151,7 +1151,7 @@ static void plan_yz(const Geom &g, DemagPlan &p)
     }
 }
 
-// Launch shapes: every block transforms at most 8 complex values per thread; the y and z passes take
+// Launch shapes: every block transforms at most 8 (16) complex values per thread; the y and z passes take
 // up to kMaxThreads<T> threads so that their rows span at least 64 bytes where the size allows.
 template <typename T>
 DemagPlan demag_plan(const Geom &g)
@@ -1159,7 +1159,6 @@ DemagPlan demag_plan(const Geom &g)
     DemagPlan p{};
     p.ok = true;
     const size_t cs = sizeof(Cx<T>);
-    const long budget = 8L * kMaxThreads<T>;
     if (g.P1 > 1) {
         const int xept = x_ept<T>(g);
         p.x_ept = xept;
