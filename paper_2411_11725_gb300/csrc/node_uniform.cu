@@ -27,7 +27,8 @@ namespace nm {
 // Tile of 32 x 4 nodes walked along z by 128 threads, eight FP32 blocks per SM at 64 registers.  Measured per
 // stage at 1024x1024x32 (FP32) / 512x512x16, with sums of the values: 0.59 ms / 87 us, against 1.04 ms / 154 us for the
 // assembled 27-point form and 0.64 ms / 99 us with two rows per thread (96 registers, five blocks per SM).  The
-// differences cost 2 / 5 %: mean stage of a Dormand-Prince step, with its error terms, 0.644 -> 0.658 ms / 95 -> 100 us.
+// differences cost 2 / 5 %: mean stage of a Dormand-Prince step, with its error terms, 0.644 -> 0.658 ms / 95 -> 100 us;
+// stages 2 and 3 of an RK4 step now 0.51 ms / 84 us.
 constexpr int kUSlots = 3;
 
 template <typename T>
@@ -41,8 +42,8 @@ struct NodeUSmem {
 // the node that stands for index i of an axis of n nodes: its mirror image beside an end, an end beyond that
 __device__ __forceinline__ int mirror(int i, int n) { return i < 0 ? 1 : (i < n ? i : (i == n ? n - 2 : n - 1)); }
 
-// (The instances of the last two Dormand-Prince stages take 72 registers, seven blocks: at 64 kLast spills and takes
-// 219 us at 512x512x16 where stage 5 takes 101; with 72 it takes 119 and kErr 94, against 63 without the error.)
+// (The instances of the last two Dormand-Prince stages take 72 registers, seven blocks: at 64 kLast spilled and took
+// 219 us at 512x512x16 where stage 5 took 101; with 72 it takes 119 where stage 5 takes 106, and kErr 102.)
 template <typename T, int NK, bool M64>
 __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK == kErr || NK == kRk4 ? 7 : 8) : 4) k_node_u(const __grid_constant__ NodeUArgs<T> p)
 {
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
             const int n = z * np + n2 * p.nn1 + n1;
             T hx, hy, hz, cx, cy, cz, mx, my, mz;
             vget(vadd(acc, sizeof(T) == 4 ? vadd(dz, fin) : fin), hx, hy, hz);
-            const T pe = p.can * (accR + finR);
+            const T ps = accR + finR, pe = sizeof(T) == 4 ? fma(p.can, ps, p.canl * ps) : p.can * ps;
             hx += p.e0 * pe;
             hy += p.e1 * pe;
             hz += p.e2 * pe;
@@ -214,17 +215,20 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
                 cy += p.hdmi[p.ns + n];
                 cz += p.hdmi[2 * p.ns + n];
             }
+            // f (1 + wl) h + c, where f (1 + wl) is no FP32 number
+            auto corrected = [&](T &x, T &y, T &z, T f, T ax, T ay, T az) {
+                const T l = f * p.wl;
+                x = fma(f, x, sizeof(T) == 4 ? fma(l, x, ax) : ax);
+                y = fma(f, y, sizeof(T) == 4 ? fma(l, y, ay) : ay);
+                z = fma(f, z, sizeof(T) == 4 ? fma(l, z, az) : az);
+            };
             // (powers of two: the share of the node's cells in those of a node inside, and its inverse)
             if (p.raw) {
                 const T f = (bx ? T(1) : T(0.5)) * (by ? T(1) : T(0.5));
-                hx = f * hx + cx;
-                hy = f * hy + cy;
-                hz = f * hz + cz;
+                corrected(hx, hy, hz, f, cx, cy, cz);
             } else {
                 const T fz = z >= 1 && z < p.N3 ? T(1) : T(2), im = p.im1 * fz * (bx ? T(1) : T(2)) * (by ? T(1) : T(2));
-                hx = fz * hx + im * cx;
-                hy = fz * hy + im * cy;
-                hz = fz * hz + im * cz;
+                corrected(hx, hy, hz, fz, im * cx, im * cy, im * cz);
                 if (p.zee) {
                     hx += sm.hf[0];
                     hy += sm.hf[1];
@@ -385,9 +389,31 @@ static void launch_node_uniform(const LocalParams<T> &p, const T *y, T *out, T *
         a.v1 = (T)(4.0 * cx - 2.0 * cy + 4.0 * cz);
         a.v2 = (T)(4.0 * cy - 2.0 * cx + 4.0 * cz);
         a.vs = (T)(cx + cy + cz);
-        a.vz = (T)(36.0 * cz);
-        a.vzl = (T)(36.0 * cz - (double)a.vz);
-        a.can = (T)(f * p.uan);
+        // 1 + wl: the factor that brings the rounded weights closest to the true ones, neighbour by neighbour and at the node
+        // itself (with cubic cells they are multiples of one number and share its rounding, up to 6e-8: an error of every
+        // exchange field that does not average out)
+        const double w[6] = {8.0 * cx - 4.0 * cy - 4.0 * cz, 8.0 * cy - 4.0 * cx - 4.0 * cz, 2.0 * cx + 2.0 * cy - cz,
+                             4.0 * cx - 2.0 * cy + 4.0 * cz, 4.0 * cy - 2.0 * cx + 4.0 * cz, cx + cy + cz};
+        const double r[6] = {(double)a.w1[0], (double)a.w2[0], (double)a.ws, (double)a.v1, (double)a.v2, (double)a.vs};
+        auto sums = [](const double *v, double *out) {
+            for (int i = 0; i < 6; ++i) out[i] = (i < 3 ? 2.0 : 1.0) * v[i];
+            out[6] = 2.0 * v[3] + 2.0 * v[4] + 4.0 * v[5];        // (from the node straight above or below)
+            out[7] = 4.0 * v[0] + 4.0 * v[1] + 8.0 * v[2];        // (from the node itself)
+        };
+        const double many[8] = {2, 2, 4, 4, 4, 8, 2, 1};
+        double sw[8], sr[8], rw = 0.0, rr = 0.0;
+        sums(w, sw);
+        sums(r, sr);
+        for (int i = 0; i < 8; ++i) {
+            rw += many[i] * sr[i] * sw[i];
+            rr += many[i] * sr[i] * sr[i];
+        }
+        const double one = sizeof(T) == 4 && rr > 0.0 ? rw / rr : 1.0;
+        a.wl = (T)(one - 1.0);
+        a.vz = (T)(36.0 * cz / one);
+        a.vzl = (T)(36.0 * cz / one - (double)a.vz);
+        a.can = (T)(f * p.uan / one);
+        a.canl = (T)(f * p.uan / one - (double)a.can);
         a.im1 = (T)f;
     } else {
         const double f = p.raw ? 1.0 : p.uim, cx = f * p.ucx, cy = f * p.ucy;

@@ -130,6 +130,7 @@ struct NodeUArgs {
     T w1[2], w2[2], ws;
     T can;                      // 2 Ku V / 216 (2D basis: / 36 per layer)
     T v1, v2, vs, vz, vzl, cx, cy, cz;
+    T canl, wl;                 // 3D basis, FP32: what the rounding of can left, and of w and v together (relative)
     T e0, e1, e2;
     T im1, mu0V8;               // 1 / (mu0 V/8 Ms) or 1 when raw, mu0 V/8 (2D basis: 1 / (mu0 V/4 Ms N3), mu0 V/4)
     T gam, alpha;
