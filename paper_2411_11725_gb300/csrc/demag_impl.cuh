@@ -81,8 +81,9 @@ struct YTile {
 };
 
 // x passes, values per thread: radix-16 stages (16) for FP32 lines of 2^10 complex values, and for those of 2^7 and 2^8,
-// where they save a stage, once the lines fill the GPU with half the threads (kXWide threads or more).  Steps: 256x256x8
-// (98k threads) 515 -> 491 us, but 256x256x4 (49k) 285 -> 300, 128x128x16 (49k) 292 -> 303, 200x50x1 (2k) 125 -> 152.
+// where they save a stage, once the lines fill the GPU with half the threads (kXWide threads or more).  Steps with 8 and 16
+// values: 256x256x8 (98k threads) 489 / 472 us, 128x200x17 (82k) 594 / 590, but 128x128x16 (49k) 306 / 316, 256x256x4 (49k)
+// 278 / 294, 200x50x1 (2k) 121 / 150.
 constexpr long kXWide = 152 * 512;
 template <typename T>
 constexpr bool x_ept_choice(int LG)
@@ -1118,10 +1119,10 @@ static void init_attributes_t()
 
 // Tile of the fused y-z convolution.  Single-layer meshes always take it.  Meshes of several layers take it where
 // a column's tile is so small that the three launches it replaces cost more than its serial phases (FP32 steps,
-// fused against separate: 16x16x4 131 against 142 us, 64x32x4 143 / 150, 64x64x2 148 / 154, but 128x64x4 168 / 168
-// and 128x128x8 254 / 231; FP64: 64x64x4 611 / 657, 128x128x4 1253 / 1332).  G is the widest tile that leaves at
-// least 128 blocks: wider rows move whole sectors, narrower ones fill the GPU (FP32 steps with G = 1, 2, 4: 64x64x1
-// 142, 142, 146 us; 200x50x1 164, 144, 146; 512x512x1 536, 427, 357; 1024x1024x1 1491, 1289, 1122).
+// fused against separate: 16x16x4 107 against 117 us, 64x32x4 117 / 129, 64x64x2 125 / 132, but 128x64x4 150 / 152, 131x67x5
+// 214 / 187 and 128x128x8 252 / 213; FP64: 64x64x4 602 / 664, 128x128x4 1103 / 1208, 256x256x4 3593 / 3638).  G is the widest
+// tile that leaves at least 128 blocks: wider rows move whole sectors, narrower ones fill the GPU (FP32 steps with G = 1, 2,
+// 4: 64x64x1 111, 115, 117 us; 200x50x1 120, 121, 123; 512x512x1 511, 392, 330; 1024x1024x1 1547, 1252, 1087).
 template <typename T>
 static void plan_yz(const Geom &g, DemagPlan &p)
 {
