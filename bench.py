@@ -455,7 +455,7 @@ def run_ours(args, rank, world, dist):
                    "GBps": (v[2] / v[1]) / (v[0] / v[1] * 1e-3) / 1e9,
                    "frac_of_peak": (v[2] / v[1]) / (v[0] / v[1] * 1e-3) / 1e9 / peak}
                for k, v in groups.items()}
-    launches_per_step = len(prof) + 1  # dp5_error_control is two kernels
+    launches_per_step = len(prof)  # one mark per launch
     serving = None
     if args.serve_requests > 0:
         serving = run_serving(args.serve_requests, int(args.serve_budget_gb * (1 << 30)), args.serve_max_active)
