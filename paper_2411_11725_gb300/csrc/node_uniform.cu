@@ -27,8 +27,8 @@ namespace nm {
 // Tile of 32 x 4 nodes walked along z by 128 threads, eight FP32 blocks per SM at 64 registers.  Measured per
 // stage at 1024x1024x32 (FP32) / 512x512x16, with sums of the values: 0.59 ms / 87 us, against 1.04 ms / 154 us for the
 // assembled 27-point form and 0.64 ms / 99 us with two rows per thread (96 registers, five blocks per SM).  The
-// differences cost 2 / 5 %: mean stage of a Dormand-Prince step, with its error terms, 0.644 -> 0.658 ms / 95 -> 100 us;
-// stages 2 and 3 of an RK4 step now 0.51 ms / 84 us.
+// differences cost 1.5 / 2.5 %: mean stage of a Dormand-Prince step, with its error terms, 0.648 -> 0.657 ms / 96 -> 98 us
+// (100 us with reads for the elements past the mirror nodes too, and 13.4 instead of 11.5 us at 15x200x13).
 constexpr int kUSlots = 3;
 
 template <typename T>
@@ -39,8 +39,8 @@ struct NodeUSmem {
     T hf[4];               // uniform applied field, time factor of the cell field
 };
 
-// the node that stands for index i of an axis of n nodes: its mirror image beside an end, an end beyond that
-__device__ __forceinline__ int mirror(int i, int n) { return i < 0 ? 1 : (i < n ? i : (i == n ? n - 2 : n - 1)); }
+// the node that stands for index i >= -1 of an axis of n nodes: its mirror image beside an end, none (-1) beyond that
+__device__ __forceinline__ int mirror(int i, int n) { return i < 0 ? 1 : (i < n ? i : (i == n ? n - 2 : -1)); }
 
 // (The instances of the last two Dormand-Prince stages take 72 registers, seven blocks: at 64 kLast spilled and took
 // 219 us at 512x512x16 where stage 5 took 101; with 72 it takes 119 where stage 5 takes 106, and kErr 102.)
@@ -69,14 +69,15 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
         sm.hf[2] = (T)(p.hu2 * su);
         sm.hf[3] = (T)u_time_factor<T>(p.hc_freq, p.hc_phase, t);
     }
-    // the elements of every node and cell plane that this thread copies: offset within the plane (outside the mesh: of the
-    // mirror node beside an end, of an end beyond that), or -1 outside the cells (zero fill)
+    // the elements of every node and cell plane that this thread copies: offset within the plane (of the mirror node
+    // beside an end of the mesh), or -1 where there is none (zero fill)
     constexpr int EN = (S::SX * S::SY + kUThreads - 1) / kUThreads, EC = (S::CX * S::CY + kUThreads - 1) / kUThreads;
     int no[EN], co[EC];
 #pragma unroll
     for (int k = 0; k < EN; ++k) {
         const int t = threadIdx.x + k * kUThreads, r = t / S::SX, c = t - r * S::SX;
-        no[k] = mirror(y0 - 1 + r, p.nn2) * p.nn1 + mirror(x0 - 1 + c, p.nn1);
+        const int i = mirror(x0 - 1 + c, p.nn1), j = mirror(y0 - 1 + r, p.nn2);
+        no[k] = i >= 0 && j >= 0 ? j * p.nn1 + i : -1;
     }
 #pragma unroll
     for (int k = 0; k < EC; ++k) {
@@ -93,9 +94,10 @@ __global__ void __launch_bounds__(kUThreads, sizeof(T) == 4 ? (NK == kLast || NK
             for (int k = 0; k < EN; ++k) {
                 const int t = threadIdx.x + k * kUThreads;
                 if (t < S::SX * S::SY) {
-                    const T *src = p.y + (q * np + no[k]);
+                    const bool in = no[k] >= 0;
+                    const T *src = p.y + (in ? q * np + no[k] : 0);
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) cp_elem(sm.y.p(s, t, c), src + c * p.ns, true);
+                    for (int c = 0; c < 3; ++c) cp_elem(sm.y.p(s, t, c), src + c * p.ns, in);
                 }
             }
         }
