@@ -1138,14 +1138,14 @@ static void plan_yz(const Geom &g, DemagPlan &p)
     // as many threads as a radix-8 stage has butterflies
     const int want = (((3 * g.N3) << lgG) * g.P2 / 8 + 31) / 32 * 32;
     p.yz_threads = want < 128 ? 128 : (want > kYZThreads<T> ? kYZThreads<T> : want);
-    // as few stages as radix 8 (FP64 and lines up to 2^9) or 16 allows, split evenly, the larger radices last, where a
-    // stage has no twiddles (512x512x1 step 262 -> 258 us, and more accurate, than with them first; FP32 lines of 2^11, which
-    // have a second stage of radix 16 either way, take them first: 203 against 214 us at 111x528x1).  2^8 in three stages
-    // with table twiddles: two of radix 16 save 2 us of 131 a step at 200x100x1, but cost a quarter of the accuracy with
-    // products and a tenth with table values (error of a random state's demag field at 30x100x1: 1.50e-7 and 1.30e-7
-    // against 1.16e-7).
+    // As few stages as radix 8 (FP64 and lines up to 2^9) or 16 allows, split evenly.  2^8 in three stages with table
+    // twiddles: two of radix 16 save 2 us of 131 a step at 200x100x1, but cost a quarter of the accuracy with products and a
+    // tenth with table values (error of a random state's demag field at 30x100x1: 1.50e-7 and 1.30e-7 against 1.18e-7).
+    // FP32: the larger radices first, more reads in flight (200x50x1 step 115 against 117 us, 200x100x1 130 / 132, 111x528x1
+    // 203 / 214), but for 2^10, whose one radix-16 stage comes last, where it has no twiddles (512x512x1 255 against 260 us,
+    // and more accurate: 30x400x1 1.25e-7 against 1.42e-7).  FP64: last (64x64x1 359 / 368 us, 128x128x4 1099 / 1133).
     const int RM = sizeof(T) == 4 && g.lgP2 > 8 ? 4 : 3;
-    const bool larger_first = sizeof(T) == 4 && g.lgP2 == 11;
+    const bool larger_first = sizeof(T) == 4 && g.lgP2 != 10;
     p.yz_plan = 0;
     for (int left = g.lgP2, s = 0, ns = div_up(left, RM); left > 0; ++s, --ns) {
         const int lr = larger_first ? div_up(left, ns) : left / ns;
