@@ -132,7 +132,7 @@ struct NodeUArgs {
     T v1, v2, vs, vz, vzl, cx, cy, cz;
     T canl, wl;                 // 3D basis, FP32: what the rounding of can left, and of w and v together (relative)
     T e0, e1, e2;
-    T im1, mu0V8;               // 1 / (mu0 V/8 Ms) or 1 when raw, mu0 V/8 (2D basis: 1 / (mu0 V/4 Ms N3), mu0 V/4)
+    T im1, mu0V8;               // 1 / mass of such a node (1 when raw); mu0 V/8 (2D basis: mu0 V/4)
     T gam, alpha;
     const T *y, *MsH, *Msh, *hdmi;
     T *out, *y_next;
